@@ -143,7 +143,9 @@ spmv_status spmv_row_histogram(spmv_handle h, int32_t nbins, int64_t *counts);
  * family 5: sorted row-slice kernel (SELL-C-sigma with C = 64: in each window
  *           of param rows, a power of two from 32 to 2^20, default 4096, the
  *           rows ordered by length and stored 64 rows at a time, two rows per
- *           lane; rows of more than 128 entries summed by a whole warp); FP64,
+ *           lane; rows of more than 128 entries summed by a whole warp; slices
+ *           whose slot rows each lie on one diagonal, as on a grid stencil, run
+ *           without column indices); FP64,
  *           and FP32 storage with the default accumulator (FP32 runs: a whole
  *           row when no row exceeds 9 entries, else blocks of 4 entries folded
  *           into float-float), other combinations run the slot-major kernel;

@@ -105,6 +105,7 @@ struct SlotTable {
 
 // Sorted row-slice copy of a matrix for plan family 5 (per window sigma).
 struct SellTable {
+    void *meta = nullptr;       // one allocation: the tables d .. diag below
     int2 *d = nullptr;          // per slice: first slot row and width (width < 0: long row)
     int32_t *srows = nullptr;   // kSellC rows per slice (-1: none)
     int32_t *cstart = nullptr;  // n_ctas + 1: first slice of each CTA of a launch
@@ -115,6 +116,11 @@ struct SellTable {
     int32_t n_long = 0;
     int64_t slot_rows = 0;
     bool vals_valid = false;
+    // diagonal slices: descriptors with each slice's place in diag (in slice order
+    // and in launch order), and the diagonals of the slot rows, padded to 4 per slice
+    int4 *dtmp = nullptr, *dorder = nullptr;
+    int4 *diag = nullptr;
+    bool diagonal = false;      // enough slices are diagonal for k_sell_diag
 };
 
 struct ChunkTable {
@@ -244,6 +250,11 @@ void make_slot_chunks(const int32_t *rp, int32_t n_rows, int E, std::vector<Chun
 // Rows longer than this are summed by a whole warp from the CRS arrays instead
 // of by one lane of a slice.
 constexpr int32_t kSellLongRow = 128;
+// Share of the slots that diagonal slices must cover for k_sell_diag to run (the
+// others read column indices there too, without k_sell's loads a block ahead).
+// The 27-point pattern on 24^3 (0.73) runs in 4.7 us (FP64; 3.5 FP32) against
+// 9.4 (7.0) on k_sell.
+constexpr double kDiagMinShare = 0.5;
 
 // Slices of the sorted row-slice layout: in each window of sigma rows, the rows
 // of at most kSellLongRow entries ordered by length (longest first, ties in row
@@ -254,7 +265,7 @@ constexpr int32_t kSellLongRow = 128;
 bool make_sell_slices(const int32_t *rp, int32_t n_rows, int32_t sigma, std::vector<int2> &out,
                       std::vector<int32_t> &srows, int32_t *n_long, int64_t *slot_rows) {
     int64_t off = kSellU;
-    std::vector<int32_t> idx;
+    std::vector<int32_t> idx, sorted;
     for (int64_t w0 = 0; w0 < n_rows; w0 += sigma) {
         const int32_t w1 = static_cast<int32_t>(std::min<int64_t>(n_rows, w0 + sigma));
         idx.clear();
@@ -267,13 +278,20 @@ bool make_sell_slices(const int32_t *rp, int32_t n_rows, int32_t sigma, std::vec
                 idx.push_back(r);
             }
         }
-        std::stable_sort(idx.begin(), idx.end(),
-                         [rp](int32_t a, int32_t b) { return rp[a + 1] - rp[a] > rp[b + 1] - rp[b]; });
+        // longest first, ties in row order: a counting sort
+        int32_t at[kSellLongRow + 2] = {0};  // place of the next row of length kSellLongRow - q
+        for (int32_t r : idx) ++at[kSellLongRow - (rp[r + 1] - rp[r]) + 1];
+        for (int q = 1; q <= kSellLongRow + 1; ++q) at[q] += at[q - 1];
+        sorted.resize(idx.size());
+        for (int32_t r : idx) sorted[static_cast<size_t>(at[kSellLongRow - (rp[r + 1] - rp[r])]++)] = r;
+        idx.swap(sorted);
         for (size_t i = 0; i < idx.size(); i += kSellC) {
             const int32_t w = rp[idx[i] + 1] - rp[idx[i]];
             if (off > INT32_MAX) return false;
             out.push_back(make_int2(static_cast<int32_t>(off), w));
-            for (size_t l = 0; l < kSellC; ++l) srows.push_back(i + l < idx.size() ? idx[i + l] : -1);
+            const size_t real = std::min<size_t>(kSellC, idx.size() - i);
+            srows.insert(srows.end(), idx.begin() + i, idx.begin() + i + real);
+            srows.insert(srows.end(), kSellC - real, -1);
             off += w;
         }
     }
@@ -330,9 +348,7 @@ void sell_ranges(const std::vector<int2> &d, const int32_t *rp, int G, std::vect
 }
 
 void free_sell(SellTable &t) {
-    cudaFree(t.d);
-    cudaFree(t.srows);
-    cudaFree(t.cstart);
+    cudaFree(t.meta);
     cudaFree(t.vals);
     cudaFree(t.cols);
     t = SellTable();
@@ -395,6 +411,7 @@ struct spmv_matrix {
     std::vector<int32_t> h_rp;
     // plan
     double col_random = 0.0;  // column_randomness() of the pattern
+    double col_diag = 0.0;    // diagonal_rows() of the pattern
     int32_t max_row = 0x7fffffff;  // longest row (set by the tuner)
     int family = 0;  // 0 warp chunks, 1 row-vector, 2 staged tiles, 3 three-stage chunks
     int E = 16;      // entries per lane (family 0) or per thread segment (family 2)
@@ -409,6 +426,7 @@ struct spmv_matrix {
     std::map<int, SellTable> sellsT;                    // sigma -> sorted row-slice copy of A^T (reverse pass)
     double sell_padT = -1.0;                            // padding of A^T's slices (computed on first use)
     int32_t sigma = 4096;                               // family 5: rows per sorting window
+    bool sell_if_diag = false;                          // family 5 by the tuner for its diagonal slices only
     double sell_pad = 1.0;                              // padding of sorted slices of 4096-row windows
     int32_t *d_rmap = nullptr;                          // output row of each stored row
     // transposed structure (built on first use)
@@ -526,11 +544,9 @@ int pick_E(int vk, int xk, int yk, int acc, int want) {
 //   12 entries per row: the sorted row-slice kernel (family 5, windows of 4096
 //   rows), when its padding is at most 10 % (27-point 128^3: 113.0 against
 //   139.1 us in FP64, 89.6 against 102.9 us with FP32 storage, against the best
-//   chunk kernels).  With short rows it gains little alone and loses next to
-//   other kernels: on the 7-point 160^3 matrix 69.3 against 71.5 us in a loop
-//   of products, but 74-80 against 70-74 us right after a kernel that wrote
-//   33 MB (the write-back of that kernel's dirty lines lands on a product
-//   already at 90 % of the copy bandwidth), and FP64 CG 109 against 105 ms.
+//   chunk kernels).  With short rows it takes stencils on a grid, whose slices
+//   need no column indices (k_sell_diag, kDiagMinRows); the others keep the
+//   chunk kernels, which read as many bytes.
 //   Scattered columns: one row per lane gathers x from as many places as the
 //   slice has rows, so the slot-major chunk kernel (family 4) stays ahead
 //   (Hamiltonian-like 150.4 against 167.3 us): FP64 with E = 7 entries per lane
@@ -547,6 +563,13 @@ int pick_E(int vk, int xk, int yk, int acc, int want) {
 constexpr int32_t kSellSigma = 4096;
 constexpr double kSellMaxPadding = 0.10;
 constexpr double kSellMinRowLength = 12.0;
+// FP64 matrices with shorter rows take the row slices when at least this share
+// of the rows lies on the previous row's diagonals, so that nearly all slices
+// are diagonal (k_sell_diag), and they are large enough to fill the GPU's warps:
+// 5-point 128^2 2.4 against 2.5 us on the slot-major kernel, 256^2 3.1 against
+// 3.4, 2000^2 42 against 50; 7-point 64^3 6.2 against 6.8, 160^3 55 against 68.
+constexpr double kDiagMinRows = 0.9;
+constexpr int32_t kDiagMinSize = 16384;
 // Batched slot-major launch: each member's entries per lane from its own mean
 // row length, E = 7 below this many entries per row, else 9.  The threshold is
 // lower than a single matrix's (8): on the 256-matrix batch of 5-point
@@ -573,8 +596,12 @@ void autotune(spmv_matrix *h) {
         h->family = 4;
         h->E = (mean < 8.0) ? 7 : 9;
     }
-    if (!scattered && h->sell_pad <= kSellMaxPadding && (h->vk == kF32 || mean >= kSellMinRowLength))
+    const bool diagonal = h->col_diag >= kDiagMinRows && h->n_rows >= kDiagMinSize;
+    const bool sells = h->vk == kF32 || mean >= kSellMinRowLength;
+    if (!scattered && h->sell_pad <= kSellMaxPadding && (sells || diagonal)) {
         h->family = 5;
+        h->sell_if_diag = !sells;
+    }
 }
 
 // Share of entries (sampled rows) whose column is more than 8 away from every
@@ -599,6 +626,24 @@ double column_randomness(const int32_t *rp, const int32_t *col, int32_t n_rows) 
         }
     }
     return total ? static_cast<double>(far) / total : 0.0;
+}
+
+// Share of (sampled) rows whose entries lie on the same diagonals, in the same
+// order, as the previous row's: near 1 for stencils on a grid, where a slice of
+// 64 rows of one length then needs one diagonal per slot row instead of column
+// indices.
+double diagonal_rows(const int32_t *rp, const int32_t *col, int32_t n_rows) {
+    if (!col || n_rows < 2) return 0.0;
+    const int32_t step = std::max<int32_t>(1, n_rows / 32768) | 1;  // odd: no grid line is sampled alone
+    int64_t same = 0, total = 0;
+    for (int32_t i = 1; i < n_rows; i += step) {
+        const int32_t len = rp[i + 1] - rp[i];
+        bool eq = len > 0 && len == rp[i] - rp[i - 1];
+        for (int32_t k = 0; eq && k < len; ++k) eq = col[rp[i] + k] - col[rp[i - 1] + k] == 1;
+        same += eq ? 1 : 0;
+        ++total;
+    }
+    return total ? static_cast<double>(same) / total : 0.0;
 }
 
 ChunkTable *get_chunks(spmv_matrix *h, int E, bool transposed) {
@@ -662,6 +707,57 @@ SlotTable *get_slots(spmv_matrix *h, int E, cudaStream_t s, bool transposed = fa
     return &t;
 }
 
+// The tables of a row-slice copy (descriptors, rows, CTA ranges, places of the
+// diagonals) in one allocation and one copy on s.
+bool upload_sell(SellTable &t, const std::vector<int2> &d, const std::vector<int32_t> &sr,
+                 const std::vector<int32_t> &ws, cudaStream_t s) {
+    std::vector<int4> order(d.size());
+    size_t packed = 2;  // a block of 8 slot rows reads two elements
+    for (size_t i = 0; i < d.size(); ++i) {
+        order[i] = make_int4(d[i].x, d[i].y, static_cast<int>(i), static_cast<int>(packed - 2));
+        packed += d[i].y > 0 ? static_cast<size_t>(d[i].y + 3) / 4 : 0;
+    }
+    const size_t o_order = 0, o_d = o_order + sizeof(int4) * order.size(), o_sr = o_d + sizeof(int2) * d.size(),
+                 o_ws = o_sr + 4 * sr.size(), host_end = o_ws + 4 * ws.size() + 8, o_out = (host_end + 15) / 16 * 16,
+                 o_diag = o_out + sizeof(int4) * order.size();
+    std::vector<char> host(host_end, 0);  // the last two words: the marking's counts
+    if (!d.empty()) {
+        std::memcpy(host.data() + o_order, order.data(), sizeof(int4) * order.size());
+        std::memcpy(host.data() + o_d, d.data(), sizeof(int2) * d.size());
+        std::memcpy(host.data() + o_sr, sr.data(), 4 * sr.size());
+    }
+    std::memcpy(host.data() + o_ws, ws.data(), 4 * ws.size());
+    if (cudaMalloc(&t.meta, o_diag + sizeof(int4) * packed) != cudaSuccess) {
+        t.meta = nullptr;
+        return false;
+    }
+    char *m = static_cast<char *>(t.meta);
+    t.dtmp = reinterpret_cast<int4 *>(m + o_order);
+    t.dorder = reinterpret_cast<int4 *>(m + o_out);
+    t.d = reinterpret_cast<int2 *>(m + o_d);
+    t.srows = reinterpret_cast<int32_t *>(m + o_sr);
+    t.cstart = reinterpret_cast<int32_t *>(m + o_ws);
+    t.diag = reinterpret_cast<int4 *>(m + o_diag);
+    return cudaMemcpyAsync(m, host.data(), host.size(), cudaMemcpyHostToDevice, s) == cudaSuccess &&
+           cudaMemsetAsync(t.diag, 0, sizeof(int4) * packed, s) == cudaSuccess;
+}
+
+// Marks the diagonal slices of a row-slice copy whose columns are laid out on s:
+// the diagonals into diag, the descriptors in launch order into dorder.  Waits
+// for s; false on an error.
+bool mark_diagonals(SellTable &t, cudaStream_t s) {
+    if (t.n == 0) return true;
+    uint32_t *count = reinterpret_cast<uint32_t *>(t.cstart + t.n_ctas + 1);  // [0]: slot rows of diagonal slices
+    uint32_t in = 0;
+    if (launch_sell_mark_diag(t.dtmp, t.n, t.srows, t.cols, t.diag, count, t.dorder, s) != cudaSuccess ||
+        cudaMemcpyAsync(&in, count, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return false;
+    const double all = static_cast<double>(t.slot_rows - kSellU) + static_cast<double>(t.n_long) * kSellLongRow;
+    t.diagonal = in > 0 && static_cast<double>(in) >= kDiagMinShare * all;
+    return true;
+}
+
 // The sorted row-slice copy for window sigma (built on first use; its values are
 // laid out again on the stream after spmv_set_values).  transposed: the copy of
 // A^T, from the transposed structure and the values laid out in A^T order.
@@ -687,17 +783,13 @@ SellTable *get_sell(spmv_matrix *h, int32_t sigma, cudaStream_t s, bool transpos
         sell_ranges(d, h_rp, t.n_ctas, ws);
         const size_t nslots = static_cast<size_t>(t.slot_rows) * kSellC;
         const size_t vb = (h->vk == kF64) ? 8 : 4;
-        bool ok = dmalloc(&t.d, d.size()) == cudaSuccess && dmalloc(&t.srows, sr.size()) == cudaSuccess &&
-                  dmalloc(&t.cstart, ws.size()) == cudaSuccess &&
-                  cudaMalloc(&t.vals, nslots * vb + 16) == cudaSuccess && dmalloc(&t.cols, nslots + 4) == cudaSuccess;
-        ok = ok && cudaMemcpy(t.cstart, ws.data(), 4 * ws.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+        bool ok = upload_sell(t, d, sr, ws, s) && cudaMalloc(&t.vals, nslots * vb + 16) == cudaSuccess &&
+                  dmalloc(&t.cols, nslots + 4) == cudaSuccess;
         // the leading padding rows: value 0, column -1
         ok = ok && cudaMemsetAsync(t.vals, 0, static_cast<size_t>(kSellU) * kSellC * vb, s) == cudaSuccess &&
              cudaMemsetAsync(t.cols, 0xff, static_cast<size_t>(kSellU) * kSellC * 4, s) == cudaSuccess;
-        ok = ok && (d.empty() || cudaMemcpy(t.d, d.data(), sizeof(int2) * d.size(), cudaMemcpyHostToDevice) ==
-                                     cudaSuccess);
-        ok = ok && (sr.empty() || cudaMemcpy(t.srows, sr.data(), 4 * sr.size(), cudaMemcpyHostToDevice) == cudaSuccess);
         ok = ok && launch_sell_relayout(t.d, t.srows, t.n, d_rp, h->vk, d_val, d_col, t.vals, t.cols, s) == cudaSuccess;
+        ok = ok && mark_diagonals(t, s);
         if (!ok) {
             free_sell(t);
             (void)cudaGetLastError();  // a failed allocation must not surface at a later launch check
@@ -808,6 +900,7 @@ spmv_status create_from_host(spmv_handle *out, int32_t n_rows, int32_t n_cols, i
     h->vk = store_t;
     h->h_rp = std::move(h_rp);
     h->col_random = column_randomness(h->h_rp.data(), host_col, n_rows);
+    h->col_diag = diagonal_rows(h->h_rp.data(), host_col, n_rows);
     spmv_status st = upload_matrix(h, nullptr, col_idx, val, val_t, dev_ptrs, s);
     if (st != SPMV_OK) {
         destroy_matrix(h);
@@ -857,6 +950,7 @@ bool sell_launch_of(spmv_matrix *h, double alpha, const void *x, int xk, double 
     const int acc = (h->vk == kF32) ? h->acc32 : kAccF64;
     SellTable *lt = nullptr;
     if (!sell_ops(h->vk, xk, yk, acc, ops, h->max_row) || (lt = get_sell(h, h->sigma, s)) == nullptr) return false;
+    if (h->sell_if_diag && !lt->diagonal) return false;  // few diagonal slices after all: the slot-major kernel
     *lp = SellParams{};
     lp->slices = lt->d;
     lp->srows = lt->srows;
@@ -868,6 +962,9 @@ bool sell_launch_of(spmv_matrix *h, double alpha, const void *x, int xk, double 
     lp->n_slices = lt->n;
     lp->alpha = alpha;
     lp->beta = beta;
+    lp->dorder = lt->diagonal ? lt->dorder : nullptr;
+    lp->diag = lt->diag;
+    lp->dshort = lt->slot_rows <= 8LL * lt->n;
     return true;
 }
 
@@ -1028,6 +1125,7 @@ spmv_status ensure_mirror32(spmv_matrix *h, cudaStream_t s) {
     m->d_col = h->d_col;
     m->h_rp = h->h_rp;
     m->col_random = h->col_random;
+    m->col_diag = h->col_diag;
     const size_t nent = static_cast<size_t>(h->nnz) + kEntryPad;
     if (cudaMalloc(&m->d_val, nent * 4) != cudaSuccess || dmalloc(&m->d_err, 1) != cudaSuccess) {
         destroy_matrix(m);
@@ -1053,8 +1151,8 @@ spmv_status ensure_mirror32(spmv_matrix *h, cudaStream_t s) {
 static spmv_status ready_for_capture(spmv_matrix *h, int xk, int yk) {
     const int acc = (h->vk == kF32) ? h->acc32 : kAccF64;
     SellOps lops;
-    if (h->family == 5 && !h->d_rmap && sell_ops(h->vk, xk, yk, acc, &lops, h->max_row) &&
-        get_sell(h, h->sigma, nullptr))
+    SellParams lp;
+    if (sell_launch_of(h, 1.0, nullptr, xk, 0.0, nullptr, yk, nullptr, &lops, &lp))
         return cudaDeviceSynchronize() == cudaSuccess ? SPMV_OK : SPMV_ERR_CUDA;
     SlotOps sops;
     if ((h->family == 4 || h->family == 5 || h->family == 6) &&
@@ -1301,6 +1399,7 @@ spmv_status spmv_row_histogram(spmv_handle h, int32_t nbins, int64_t *counts) {
 
 spmv_status spmv_set_plan(spmv_handle h, int32_t family, int32_t param) {
     if (!h || family < 0 || family > 6) return SPMV_ERR_INVALID_ARG;
+    h->sell_if_diag = false;
     if (family == 6) {
         const bool f64 = h->vk == kF64;
         if (param != 0 && !(f64 ? (param == 7 || param == 9) : (param == 9 || param == 15)))
@@ -1767,6 +1866,9 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
                 lp.n_ctas = t->n_ctas;
                 lp.alpha = alpha;
                 lp.beta = 0.0;
+                lp.dorder = t->diagonal ? t->dorder : nullptr;
+                lp.diag = t->diag;
+                lp.dshort = t->slot_rows <= 8LL * t->n;
                 if (lops.launch(lp, s) != cudaSuccess) return SPMV_ERR_CUDA;
                 done = true;
             }

@@ -84,6 +84,14 @@ cudaError_t launch_sell_relayout(const void *slices, const int32_t *srows, int32
                                  int vk, const void *val, const int32_t *col, void *vals_out, int32_t *cols_out,
                                  cudaStream_t s);
 
+// Finds the diagonal slices (in every slot row all 64 rows are stored and column -
+// row is one number): their diagonals into diag (int4 elements, from each slice's
+// place dtmp[s].w on), place -1 for the others, and all descriptors into dorder,
+// the others first.  The slot rows and the number of the diagonal slices are
+// added to count[0] and [1].
+cudaError_t launch_sell_mark_diag(void *dtmp, int32_t n_slices, const int32_t *srows, const int32_t *cols,
+                                  void *diag, uint32_t *count, void *dorder, cudaStream_t s);
+
 cudaError_t launch_rowvec(const KParams &p, const int32_t n_rows, int vk, int xk, int yk, int acc,
                           int T, cudaStream_t s);
 

@@ -47,6 +47,10 @@ struct SellParams {
     int32_t n_slices;
     int32_t n_ctas;        // CTAs of the launch
     double alpha, beta;
+    // diagonal slices (k_sell_diag below); dorder is null when k_sell runs
+    const int4 *dorder;    // n_slices: x, y = the descriptor, z = the slice, w = its place in diag (-1: not diagonal)
+    const int4 *diag;      // column minus row of each slot row of the diagonal slices, 4 to an element
+    bool dshort;           // at most 8 slot rows per slice on average
 };
 
 // For i = 0 .. cnt-1 and both rows h of the lane, in that order:
@@ -76,6 +80,18 @@ __device__ __forceinline__ void sell_fma_tail(ACC (&acc)[kSellK], const VT (&v)[
         default:
             break;
     }
+}
+
+// As ld_stream, but free for the compiler to schedule among other loads.
+__device__ __forceinline__ double ld_stream_p(const double *p, uint64_t pol) {
+    double v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ float ld_stream_p(const float *p, uint64_t pol) {
+    float v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+    return v;
 }
 
 // Final store of stored row `row` of m; `old` is y[row] widened, loaded ahead
@@ -285,6 +301,163 @@ template <typename VT, typename XT, typename YT, typename ACC, bool DOT = false>
 __global__ void __launch_bounds__(256) k_sell(const SellParams p, const RedOut o) {
     double dsum = 0.0;
     sell_walk<VT, XT, YT, ACC, DOT>(p, dsum);
+    if constexpr (DOT) {
+        __shared__ double s_red[32];
+        finish(block_sum(dsum, s_red), o, s_red);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Diagonal slices.  In a stencil-like matrix nearly every slice has full rows
+// whose entries at slot row j all lie on one diagonal: column - row is the same
+// number in its 64 rows (k_sell_mark_diag finds these slices once, when the copy
+// is built).  Such a slice needs no column indices: 4 bytes per slot row instead
+// of 256, a third of the matrix bytes in FP64 and half in FP32, and the address
+// of a gather is row + diagonal, known without waiting for a column load.  So
+// nothing is staged ahead in registers: a warp takes half a slice (one row per
+// lane), issues up to 8 slot rows of values and gathers, then their FMAs, and the
+// resident warps hide each other's latency.  The sums run in the same order as
+// in k_sell (and the FP32 runs fold at the same places).  Slices that are not
+// diagonal (the grid's boundary rows: a few per cent) take the same path with
+// their column indices.
+// ---------------------------------------------------------------------------
+
+// CNT slot rows of a half slice: values at vb (kSellC apart), and their columns
+// row + diagonal (DIAG; 8 diagonals at dp) or as stored (cb).
+template <int CNT, bool DIAG, typename ACC, typename VT, typename XT>
+__device__ __forceinline__ void sell_diag_block(ACC &acc, const VT *__restrict__ vb, const int32_t *__restrict__ cb,
+                                                const int4 *__restrict__ dp, int row, const XT *__restrict__ x,
+                                                uint64_t pol) {
+    int32_t c[CNT];
+    if constexpr (DIAG) {
+        const int4 a = __ldg(dp);
+        int4 b = make_int4(0, 0, 0, 0);
+        if constexpr (CNT > 4) b = __ldg(dp + 1);
+        const int32_t g[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int u = 0; u < CNT; ++u) c[u] = row + g[u];
+    } else {
+#pragma unroll
+        for (int u = 0; u < CNT; ++u) c[u] = __ldg(cb + u * kSellC);
+    }
+    VT v[CNT];
+    XT xv[CNT];
+#pragma unroll
+    for (int u = 0; u < CNT; ++u) v[u] = ld_stream_p(vb + u * kSellC, pol);
+#pragma unroll
+    for (int u = 0; u < CNT; ++u) xv[u] = (DIAG || c[u] >= 0) ? __ldg(x + c[u]) : XT(0);
+#pragma unroll
+    for (int u = 0; u < CNT; ++u) {
+        acc.fma(v[u], xv[u]);
+        if (u % kSellU == kSellU - 1 || u == CNT - 1) end_run(acc);
+    }
+}
+
+// All w slot rows of a half slice.
+template <bool DIAG, typename ACC, typename VT, typename XT>
+__device__ __forceinline__ void sell_diag_row(ACC &acc, int w, const VT *__restrict__ vb,
+                                              const int32_t *__restrict__ cb, const int4 *__restrict__ dp, int row,
+                                              const XT *__restrict__ x, uint64_t pol) {
+    for (; w >= 8; w -= 8) {
+        sell_diag_block<8, DIAG>(acc, vb, cb, dp, row, x, pol);
+        vb += 8 * kSellC;
+        if constexpr (DIAG) dp += 2;
+        else cb += 8 * kSellC;
+    }
+    switch (w) {
+        case 7: sell_diag_block<7, DIAG>(acc, vb, cb, dp, row, x, pol); break;
+        case 6: sell_diag_block<6, DIAG>(acc, vb, cb, dp, row, x, pol); break;
+        case 5: sell_diag_block<5, DIAG>(acc, vb, cb, dp, row, x, pol); break;
+        case 4: sell_diag_block<4, DIAG>(acc, vb, cb, dp, row, x, pol); break;
+        case 3: sell_diag_block<3, DIAG>(acc, vb, cb, dp, row, x, pol); break;
+        case 2: sell_diag_block<2, DIAG>(acc, vb, cb, dp, row, x, pol); break;
+        case 1: sell_diag_block<1, DIAG>(acc, vb, cb, dp, row, x, pol); break;
+        default: break;
+    }
+}
+
+// Store of one FP64 row sum.  The form of the update is an integer fixed per
+// launch, so a row costs the FP64 pipe nothing (y = v) or one or two operations;
+// tests on alpha and beta at the store cost it about four per row (with 5 and 7
+// entries per row, 62 and 79 us instead of 47 and 60 us on the 2000^2 and 160^3
+// Laplacians).
+__device__ __forceinline__ double sell_diag_store(double *__restrict__ y, int row, double v, double alpha, double beta,
+                                                  int emode) {
+    if (emode == kEpiScale) v = alpha * v;
+    else if (emode == kEpiAdd) v = v + y[row];
+    else if (emode == kEpiGeneral) v = fma(alpha, v, beta * y[row]);
+    y[row] = v;
+    return v;
+}
+
+template <typename VT, typename XT, typename YT, typename ACC, bool DOT>
+__device__ __forceinline__ void sell_diag_walk(const SellParams &p, double &dsum) {
+    constexpr int C = kSellC;
+    const int lane = threadIdx.x & 31;
+    const int n = 2 * p.n_slices;  // half slices
+    const int nw = gridDim.x * 8;
+    const uint64_t pol = l2_evict_first_policy();
+    const XT *__restrict__ x = static_cast<const XT *>(p.m.x);
+    YT *__restrict__ y = static_cast<YT *>(p.m.y);
+    const VT *__restrict__ vals = static_cast<const VT *>(p.vals);
+    const double alpha = p.alpha, beta = p.beta;
+    const int emode = epi_mode(alpha, beta);
+    int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= n) return;
+    auto desc_of = [&](int k) { return __ldg(p.dorder + (k < n ? k >> 1 : p.n_slices - 1)); };
+    auto row_of = [&](const int4 &d, int k) {
+        return __ldg(p.srows + static_cast<int64_t>(d.z) * C + (k & 1) * 32 + lane);
+    };
+    int4 d = desc_of(i), dn = desc_of(i + nw);
+    int r = row_of(d, i);
+    for (; i < n; i += nw) {
+        const int4 d2 = desc_of(i + 2 * nw);
+        const int rn = row_of(dn, i + nw);
+        if (d.y < 0) {
+            if ((i & 1) == 0) {
+                const int row = d.x;
+                const ChunkDesc cd{__ldg(p.m.rp + row), __ldg(p.m.rp + row + 1), row, (row + 1) | kChunkLong};
+                long_row<VT, XT, YT, ACC, false>(p.m, cd, x, y, alpha, beta, emode == kEpiPlain, lane);
+                if constexpr (DOT) {
+                    if (lane == 0) dsum = fma(widen(x[row]), widen(y[row]), dsum);  // lane 0 stored it
+                }
+            }
+        } else {
+            const int64_t base = static_cast<int64_t>(d.x) * C + (i & 1) * 32 + lane;
+            ACC acc;
+            acc.zero();
+            if (d.w >= 0)
+                sell_diag_row<true>(acc, d.y, vals + base, static_cast<const int32_t *>(nullptr), p.diag + d.w, r, x, pol);
+            else
+                sell_diag_row<false>(acc, d.y, vals + base, p.cols + base, static_cast<const int4 *>(nullptr), r, x, pol);
+            if (r >= 0) {
+                YT q;
+                if constexpr (std::is_same<ACC, AccF64>::value) {
+                    q = sell_diag_store(y, r, acc.get(), alpha, beta, emode);
+                } else {
+                    const double old = emode >= kEpiAdd ? widen(y[r]) : 0.0;
+                    q = sell_store<VT>(p.m, x, y, r, acc, alpha, beta, emode == kEpiPlain, old);
+                }
+                if constexpr (DOT) dsum = fma(widen(__ldg(x + r)), widen(q), dsum);
+            }
+        }
+        d = dn;
+        dn = d2;
+        r = rn;
+    }
+}
+
+// CTAs per SM the registers must allow.  Rows of up to 8 entries (SHORT: one
+// block per half slice, so the warps are latency-bound) take one more: 160^3
+// Laplacian FP64 55.3 against 60.3 us, FP32 28.9 against 30.2; longer rows lose
+// by it (27-point 128^3: FP64 106.6 against 98.6, FP32 46.6 against 44.9 us).
+template <typename VT, bool SHORT>
+constexpr int kSellDiagCtas = (sizeof(VT) == 8 ? 4 : 5) + (SHORT ? 1 : 0);
+
+template <typename VT, typename XT, typename YT, typename ACC, bool SHORT, bool DOT>
+__global__ void __launch_bounds__(256, (kSellDiagCtas<VT, SHORT>)) k_sell_diag(const SellParams p, const RedOut o) {
+    double dsum = 0.0;
+    sell_diag_walk<VT, XT, YT, ACC, DOT>(p, dsum);
     if constexpr (DOT) {
         __shared__ double s_red[32];
         finish(block_sum(dsum, s_red), o, s_red);
@@ -553,8 +726,33 @@ struct SellKernel {
         const int64_t want = (static_cast<int64_t>(n_slices) + 7) / 8;
         return static_cast<int>(want < lim ? want : lim);
     }
+    // k_sell_diag on up to its resident CTAs, 8 half slices per CTA and turn
+    template <bool SHORT, bool DOT>
+    static cudaError_t launch_diag(const SellParams &p, const RedOut &o, cudaStream_t s) {
+        static int cached = -1;
+        static int cached_dev = -1;
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (cached < 0 || cached_dev != dev) {
+            int per_sm = 0, sms = 0;
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sell_diag<VT, XT, YT, ACC, SHORT, DOT>, 256,
+                                                              0) != cudaSuccess ||
+                per_sm <= 0)
+                return cudaErrorInvalidConfiguration;
+            cached = per_sm * sms;
+            cached_dev = dev;
+        }
+        const int64_t want = (2 * static_cast<int64_t>(p.n_slices) + 7) / 8;
+        const int grid = static_cast<int>(want < cached ? want : cached);
+        if (DOT && grid > cg_partials_cap()) return cudaErrorInvalidConfiguration;
+        k_sell_diag<VT, XT, YT, ACC, SHORT, DOT><<<grid, 256, 0, s>>>(p, o);
+        return cudaGetLastError();
+    }
     static cudaError_t launch(const SellParams &p, cudaStream_t s) {
         if (p.n_slices <= 0 || p.n_ctas <= 0) return cudaSuccess;
+        if (p.dorder)
+            return p.dshort ? launch_diag<true, false>(p, RedOut{}, s) : launch_diag<false, false>(p, RedOut{}, s);
         k_sell<VT, XT, YT, ACC, false><<<p.n_ctas, 256, 0, s>>>(p, RedOut{});
         return cudaGetLastError();
     }
@@ -562,6 +760,7 @@ struct SellKernel {
     // one slice and at most cg_partials_cap() CTAs
     static cudaError_t launch_dot(const SellParams &p, const RedOut &o, cudaStream_t s) {
         if (p.n_slices <= 0 || p.n_ctas <= 0 || p.n_ctas > cg_partials_cap()) return cudaErrorInvalidValue;
+        if (p.dorder) return p.dshort ? launch_diag<true, true>(p, o, s) : launch_diag<false, true>(p, o, s);
         k_sell<VT, XT, YT, ACC, true><<<p.n_ctas, 256, 0, s>>>(p, o);
         return cudaGetLastError();
     }
