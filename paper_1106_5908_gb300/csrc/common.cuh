@@ -277,6 +277,26 @@ __device__ __forceinline__ double acc_value(const ACC &a, const MatRef &m, int64
     return a.get();
 }
 
+// Form of the update y = alpha*v + beta*y, decided once per launch so that no
+// FP64 comparison or multiply by 1 runs per row (the FP64 pipe is busy with one
+// FMA per entry; Hamiltonian-like product with alpha = 0.5, beta = 0.25 on the
+// slot-major kernel 197.5 -> 187 us): kEpiPlain y = v; kEpiScale
+// y = alpha*v; kEpiAdd y = v + y (alpha = beta = 1, as in the nonlocal part of
+// the split product); kEpiGeneral y = fma(alpha, v, beta*y).
+constexpr int kEpiPlain = 0, kEpiScale = 1, kEpiAdd = 2, kEpiGeneral = 3;
+__host__ __device__ __forceinline__ int epi_mode(double alpha, double beta) {
+    if (beta == 0.0) return alpha == 1.0 ? kEpiPlain : kEpiScale;
+    return (alpha == 1.0 && beta == 1.0) ? kEpiAdd : kEpiGeneral;
+}
+
+template <typename YT>
+__device__ __forceinline__ double epi_apply(double v, const YT *__restrict__ y, double alpha, double beta, int emode) {
+    if (emode == kEpiScale) return alpha * v;
+    if (emode == kEpiAdd) return v + widen(*y);
+    if (emode == kEpiGeneral) return fma(alpha, v, beta * widen(*y));
+    return v;
+}
+
 template <typename V, typename X> __device__ __forceinline__ X ldg_x(const X *p) { return __ldg(p); }
 
 }  // namespace spmv

@@ -376,20 +376,6 @@ __device__ __forceinline__ void sell_diag_row(ACC &acc, int w, const VT *__restr
     }
 }
 
-// Store of one FP64 row sum.  The form of the update is an integer fixed per
-// launch, so a row costs the FP64 pipe nothing (y = v) or one or two operations;
-// tests on alpha and beta at the store cost it about four per row (with 5 and 7
-// entries per row, 62 and 79 us instead of 47 and 60 us on the 2000^2 and 160^3
-// Laplacians).
-__device__ __forceinline__ double sell_diag_store(double *__restrict__ y, int row, double v, double alpha, double beta,
-                                                  int emode) {
-    if (emode == kEpiScale) v = alpha * v;
-    else if (emode == kEpiAdd) v = v + y[row];
-    else if (emode == kEpiGeneral) v = fma(alpha, v, beta * y[row]);
-    y[row] = v;
-    return v;
-}
-
 template <typename VT, typename XT, typename YT, typename ACC, bool DOT>
 __device__ __forceinline__ void sell_diag_walk(const SellParams &p, double &dsum) {
     constexpr int C = kSellC;
@@ -433,7 +419,10 @@ __device__ __forceinline__ void sell_diag_walk(const SellParams &p, double &dsum
             if (r >= 0) {
                 YT q;
                 if constexpr (std::is_same<ACC, AccF64>::value) {
-                    q = sell_diag_store(y, r, acc.get(), alpha, beta, emode);
+                    // no tests on alpha and beta per row: with 5 and 7 entries per row
+                    // they cost 62 and 79 instead of 47 and 60 us (2000^2 and 160^3)
+                    q = epi_apply(acc.get(), y + r, alpha, beta, emode);
+                    y[r] = q;
                 } else {
                     const double old = emode >= kEpiAdd ? widen(y[r]) : 0.0;
                     q = sell_store<VT>(p.m, x, y, r, acc, alpha, beta, emode == kEpiPlain, old);

@@ -106,16 +106,6 @@ __device__ __forceinline__ void store_acc(const MatRef &m, const XT *__restrict_
     store_row(y, row, a.get(), alpha, beta, plain, m.rmap);
 }
 
-// Form of the update y = alpha*v + beta*y, decided once per launch so that no
-// FP64 comparison or multiply by 1 runs per row: kEpiPlain y = v; kEpiScale
-// y = alpha*v; kEpiAdd y = v + y (alpha = beta = 1, as in the nonlocal part of
-// the split product); kEpiGeneral y = fma(alpha, v, beta*y).
-constexpr int kEpiPlain = 0, kEpiScale = 1, kEpiAdd = 2, kEpiGeneral = 3;
-__host__ __device__ __forceinline__ int epi_mode(double alpha, double beta) {
-    if (beta == 0.0) return alpha == 1.0 ? kEpiPlain : kEpiScale;
-    return (alpha == 1.0 && beta == 1.0) ? kEpiAdd : kEpiGeneral;
-}
-
 // Row epilogue of a regular chunk (at most kWarpRowCap rows, lane l owns rows
 // l, l+32, l+64): the output index of each row (through rmap) and, when beta is
 // nonzero, its old y value are loaded before the FMA chains run, so that their
