@@ -109,7 +109,9 @@ spmv_status spmv_create_symmetric(spmv_handle *out, int32_t n, int64_t nnz, cons
 
 /* Replace the stored values (same sparsity pattern) from a device pointer of
  * type t; t may differ from the handle's storage type only as FP64 -> FP32
- * storage or FP32 -> FP64 storage (converted on the device).  Asynchronous. */
+ * storage or FP32 -> FP64 storage (converted on the device).  Asynchronous.  A
+ * row-slice copy on diagonals that served the last values gets the new ones in
+ * the same pass; other derived copies are laid out again when they are used. */
 spmv_status spmv_set_values(spmv_handle h, const void *val, spmv_dtype t, void *stream);
 
 /* Shape and plan of a handle.  plan[0..7] receives: kernel family (as for
@@ -269,10 +271,11 @@ spmv_status spmm_apply(spmv_handle h, int32_t nrhs, double alpha, const void *X,
  *   grad_val[k] = alpha * g[row(k)] * x[col_idx[k]]   (nnz entries, CRS order).
  * Both outputs are overwritten; either may be NULL.  FP64 handles take FP64 g,
  * x and outputs; FP32-storage handles take FP32 g, x and write FP32 outputs.
- * The first call after new values reads A^T's values through the permutation;
- * the second lays them out in A^T order once (kept until spmv_set_values) and
- * from then on grad_x runs on a copy of A^T (row slices for stencil-like
- * matrices with at least 12 entries per row, slot-major otherwise).  Results are
+ * The first call after new values reads A^T's values through the permutation
+ * (on diagonal slices: where A's slices hold them); the second lays them out in
+ * A^T order once (kept until spmv_set_values) and from then on grad_x runs on a
+ * copy of A^T (row slices for stencil-like matrices with at least 12 entries per
+ * row, slot-major otherwise).  Results are
  * unchanged up to summation order. */
 spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void *x,
                           void *grad_x, void *grad_val, void *stream);

@@ -121,6 +121,8 @@ struct SellTable {
     int4 *dtmp = nullptr, *dorder = nullptr;
     int4 *diag = nullptr;
     bool diagonal = false;      // enough slices are diagonal for k_sell_diag
+    int32_t *vpos = nullptr;    // A^T: position of each slot's value in A's copy for window
+    int32_t vpos_sigma = 0;     //      vpos_sigma (built on first use)
 };
 
 struct ChunkTable {
@@ -349,6 +351,7 @@ void sell_ranges(const std::vector<int2> &d, const int32_t *rp, int G, std::vect
 
 void free_sell(SellTable &t) {
     cudaFree(t.meta);
+    cudaFree(t.vpos);
     cudaFree(t.vals);
     cudaFree(t.cols);
     t = SellTable();
@@ -761,13 +764,23 @@ bool mark_diagonals(SellTable &t, cudaStream_t s) {
 // The sorted row-slice copy for window sigma (built on first use; its values are
 // laid out again on the stream after spmv_set_values).  transposed: the copy of
 // A^T, from the transposed structure and the values laid out in A^T order.
-SellTable *get_sell(spmv_matrix *h, int32_t sigma, cudaStream_t s, bool transposed = false) {
+// need_vals: false for a copy whose own values are not used (yet).
+SellTable *get_sell(spmv_matrix *h, int32_t sigma, cudaStream_t s, bool transposed = false, bool need_vals = true) {
     auto &tabs = transposed ? h->sellsT : h->sells;
     const int32_t *h_rp = transposed ? h->h_rowT.data() : h->h_rp.data();
     const int32_t nr = transposed ? h->n_cols : h->n_rows;
     const int32_t *d_rp = transposed ? h->d_rowT : h->d_rp;
     const int32_t *d_col = transposed ? h->d_colT : h->d_col;
     const void *d_val = transposed ? h->d_valT : h->d_val;
+    const size_t vb = (h->vk == kF64) ? 8 : 4;
+    auto alloc_vals = [&](SellTable &t) {
+        const size_t nslots = static_cast<size_t>(t.slot_rows) * kSellC;
+        if (cudaMalloc(&t.vals, nslots * vb + 16) != cudaSuccess) {
+            t.vals = nullptr;
+            return false;
+        }
+        return cudaMemsetAsync(t.vals, 0, static_cast<size_t>(kSellU) * kSellC * vb, s) == cudaSuccess;
+    };
     auto it = tabs.find(sigma);
     if (it == tabs.end()) {
         std::vector<int2> d;
@@ -782,12 +795,10 @@ SellTable *get_sell(spmv_matrix *h, int32_t sigma, cudaStream_t s, bool transpos
         std::vector<int32_t> ws;
         sell_ranges(d, h_rp, t.n_ctas, ws);
         const size_t nslots = static_cast<size_t>(t.slot_rows) * kSellC;
-        const size_t vb = (h->vk == kF64) ? 8 : 4;
-        bool ok = upload_sell(t, d, sr, ws, s) && cudaMalloc(&t.vals, nslots * vb + 16) == cudaSuccess &&
-                  dmalloc(&t.cols, nslots + 4) == cudaSuccess;
-        // the leading padding rows: value 0, column -1
-        ok = ok && cudaMemsetAsync(t.vals, 0, static_cast<size_t>(kSellU) * kSellC * vb, s) == cudaSuccess &&
-             cudaMemsetAsync(t.cols, 0xff, static_cast<size_t>(kSellU) * kSellC * 4, s) == cudaSuccess;
+        bool ok = upload_sell(t, d, sr, ws, s) && dmalloc(&t.cols, nslots + 4) == cudaSuccess;
+        ok = ok && (!need_vals || alloc_vals(t));
+        // the leading padding rows: column -1 (and value 0)
+        ok = ok && cudaMemsetAsync(t.cols, 0xff, static_cast<size_t>(kSellU) * kSellC * 4, s) == cudaSuccess;
         ok = ok && launch_sell_relayout(t.d, t.srows, t.n, d_rp, h->vk, d_val, d_col, t.vals, t.cols, s) == cudaSuccess;
         ok = ok && mark_diagonals(t, s);
         if (!ok) {
@@ -795,16 +806,77 @@ SellTable *get_sell(spmv_matrix *h, int32_t sigma, cudaStream_t s, bool transpos
             (void)cudaGetLastError();  // a failed allocation must not surface at a later launch check
             return nullptr;
         }
-        t.vals_valid = true;
+        t.vals_valid = need_vals;
         it = tabs.emplace(sigma, t).first;
     }
     SellTable &t = it->second;
-    if (!t.vals_valid) {
+    if (need_vals && !t.vals_valid) {
+        if (!t.vals && !alloc_vals(t)) {
+            (void)cudaGetLastError();
+            return nullptr;
+        }
         if (launch_sell_relayout(t.d, t.srows, t.n, d_rp, h->vk, d_val, nullptr, t.vals, nullptr, s) != cudaSuccess)
             return nullptr;
         t.vals_valid = true;
     }
     return &t;
+}
+
+// The slices of A^T with the positions of their values in A's row-slice copy (null
+// when A does not run on diagonal slices, its copy is not there, or A has rows
+// outside the slices): what a reverse pass on new values reads.
+SellTable *get_sell_positions(spmv_matrix *h, cudaStream_t s) {
+    auto f = h->sells.find(h->sigma);
+    if (h->family != 5 || f == h->sells.end()) return nullptr;
+    const SellTable &a = f->second;
+    if (!a.diagonal || a.n_long > 0 || a.slot_rows * kSellC > INT32_MAX) return nullptr;
+    SellTable *t = get_sell(h, kSellSigma, s, true, false);
+    if (!t || !t->diagonal) return nullptr;
+    if (t->vpos && t->vpos_sigma != h->sigma) {  // another plan since: other positions
+        cudaFree(t->vpos);
+        t->vpos = nullptr;
+    }
+    if (!t->vpos) {
+        const size_t nslots = static_cast<size_t>(t->slot_rows) * kSellC;
+        int32_t *rowpos = nullptr;
+        bool ok = dmalloc(&t->vpos, nslots + 4) == cudaSuccess &&
+                  dmalloc(&rowpos, static_cast<size_t>(h->n_rows)) == cudaSuccess &&
+                  cudaMemsetAsync(t->vpos, 0xff, static_cast<size_t>(kSellU) * kSellC * 4, s) == cudaSuccess &&
+                  launch_sell_vpos(a.d, a.srows, a.n, t->d, t->srows, t->n, h->d_rp, h->d_rowT, h->d_colT, h->d_perm,
+                                   rowpos, t->vpos, s) == cudaSuccess &&
+                  cudaStreamSynchronize(s) == cudaSuccess;
+        cudaFree(rowpos);
+        if (!ok) {
+            cudaFree(t->vpos);
+            t->vpos = nullptr;
+            (void)cudaGetLastError();
+            return nullptr;
+        }
+        t->vpos_sigma = h->sigma;
+    }
+    return t;
+}
+
+// Whether every row fits the tile kernels (k_sell_set_values, k_sell_grad_val).
+bool sell_tile_fits(const spmv_matrix *h) { return h->max_row <= sell_tile_max_row() && h->nnz < INT32_MAX - 64; }
+
+// The launch parameters of a row-slice copy of the matrix m.
+SellParams sell_params(const SellTable &t, const MatRef &m, double alpha, double beta) {
+    SellParams p{};
+    p.slices = t.d;
+    p.srows = t.srows;
+    p.cstart = t.cstart;
+    p.n_ctas = t.n_ctas;
+    p.vals = t.vals;
+    p.cols = t.cols;
+    p.m = m;
+    p.n_slices = t.n;
+    p.alpha = alpha;
+    p.beta = beta;
+    p.dorder = t.diagonal ? t.dorder : nullptr;
+    p.diag = t.diag;
+    p.dshort = t.slot_rows <= 8LL * t.n;
+    return p;
 }
 
 void free_chunk_map(std::map<int, ChunkTable> &tabs) {
@@ -951,20 +1023,7 @@ bool sell_launch_of(spmv_matrix *h, double alpha, const void *x, int xk, double 
     SellTable *lt = nullptr;
     if (!sell_ops(h->vk, xk, yk, acc, ops, h->max_row) || (lt = get_sell(h, h->sigma, s)) == nullptr) return false;
     if (h->sell_if_diag && !lt->diagonal) return false;  // few diagonal slices after all: the slot-major kernel
-    *lp = SellParams{};
-    lp->slices = lt->d;
-    lp->srows = lt->srows;
-    lp->cstart = lt->cstart;
-    lp->n_ctas = lt->n_ctas;
-    lp->vals = lt->vals;
-    lp->cols = lt->cols;
-    lp->m = MatRef{h->d_rp, h->d_col, h->d_val, nullptr, x, y, nullptr};
-    lp->n_slices = lt->n;
-    lp->alpha = alpha;
-    lp->beta = beta;
-    lp->dorder = lt->diagonal ? lt->dorder : nullptr;
-    lp->diag = lt->diag;
-    lp->dshort = lt->slot_rows <= 8LL * lt->n;
+    *lp = sell_params(*lt, MatRef{h->d_rp, h->d_col, h->d_val, nullptr, x, y, nullptr}, alpha, beta);
     return true;
 }
 
@@ -1315,13 +1374,25 @@ spmv_status spmv_set_values(spmv_handle h, const void *val, spmv_dtype t, void *
     DeviceGuard g(h->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (h->nnz == 0) return SPMV_OK;
-    CK(launch_convert(val, t, h->d_val, h->vk, h->nnz, s));
+    // a row-slice copy that served the last values gets the new ones in the same
+    // pass; other copies are laid out again when they are used
+    auto f = h->sells.find(h->sigma);
+    const bool fused = h->family == 5 && f != h->sells.end() && f->second.vals_valid && f->second.diagonal &&
+                       sell_tile_fits(h);
+    if (fused) {
+        const SellParams p =
+            sell_params(f->second, MatRef{h->d_rp, h->d_col, nullptr, nullptr, nullptr, nullptr, nullptr}, 1.0, 0.0);
+        CK(launch_sell_set_values(p, val, t, h->d_val, h->vk, h->max_row, s));
+    } else {
+        CK(launch_convert(val, t, h->d_val, h->vk, h->nnz, s));
+    }
     if (h->mirror32) CK(launch_convert(val, t, h->mirror32->d_val, kF32, h->nnz, s));
     h->valT_valid = false;
     h->valT_requested = false;
     ++h->values_version;
     for (auto &kv : h->slots) kv.second.vals_valid = false;
     for (auto &kv : h->sells) kv.second.vals_valid = false;
+    if (fused) f->second.vals_valid = true;
     return SPMV_OK;
 }
 
@@ -1767,17 +1838,8 @@ spmv_status spmm_apply(spmv_handle h, int32_t nrhs, double alpha, const void *X,
         (t = get_sell(h, kSellSigma, s)) != nullptr) {
         const bool vec = (nrhs % 2 == 0) && (reinterpret_cast<uintptr_t>(X) % 16 == 0) &&
                          (reinterpret_cast<uintptr_t>(Y) % 16 == 0);
-        SellParams b{};
-        b.slices = t->d;
-        b.srows = t->srows;
-        b.cstart = t->cstart;
-        b.vals = t->vals;
-        b.cols = t->cols;
-        b.m = MatRef{h->d_rp, h->d_col, h->d_val, nullptr, nullptr, nullptr, nullptr};
-        b.n_slices = t->n;
-        b.n_ctas = t->n_ctas;
-        b.alpha = alpha;
-        b.beta = beta;
+        const SellParams b =
+            sell_params(*t, MatRef{h->d_rp, h->d_col, h->d_val, nullptr, nullptr, nullptr, nullptr}, alpha, beta);
         for (; c0 + kSellR <= nrhs; c0 += kSellR)
             if (launch_sell_mr(b, static_cast<const double *>(X) + c0, static_cast<double *>(Y) + c0, nrhs, nrhs,
                                vec, s) != cudaSuccess)
@@ -1820,6 +1882,7 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
     if (grad_val && h->nnz > 0 && (!g || !x)) return SPMV_ERR_INVALID_ARG;
     DeviceGuard dg(h->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const bool again = h->valT_requested;  // not the first reverse pass on these values
     if (grad_x && h->n_cols > 0) {
         spmv_status st = ensure_transpose(h, s);
         if (st != SPMV_OK) return st;
@@ -1843,6 +1906,22 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
         const bool ind = !h->valT_valid;
         h->valT_requested = true;
         bool done = false;
+        if (ind) {
+            // new values on diagonal slices: the slices of A^T read them where A's
+            // slices hold them
+            SellOps lops;
+            const int acc = (h->vk == kF32) ? kAccFF : kAccF64;
+            const SellTable *t = nullptr, *a = nullptr;
+            if (sell_ops(h->vk, h->vk, h->vk, acc, &lops) && (t = get_sell_positions(h, s)) != nullptr &&
+                (a = get_sell(h, h->sigma, s)) != nullptr) {
+                SellParams lp =
+                    sell_params(*t, MatRef{h->d_rowT, h->d_colT, h->d_perm, h->d_val, g, grad_x, nullptr}, alpha, 0.0);
+                lp.vals = a->vals;
+                lp.vpos = t->vpos;
+                if (lops.launch_ind(lp, s) != cudaSuccess) return SPMV_ERR_CUDA;
+                done = true;
+            }
+        }
         const double meanT = h->n_cols ? static_cast<double>(h->nnz) / h->n_cols : 0.0;
         if (!ind && h->col_random <= 0.25 && meanT >= kSellMinRowLength) {
             // A^T of a stencil-like matrix with long rows: the sorted row-slice
@@ -1855,20 +1934,8 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
             // without its copy (allocation failed) the slot-major path below runs
             if (h->sell_padT <= kSellMaxPadding && sell_ops(h->vk, h->vk, h->vk, acc, &lops) &&
                 (t = get_sell(h, kSellSigma, s, true)) != nullptr) {
-                SellParams lp{};
-                lp.slices = t->d;
-                lp.srows = t->srows;
-                lp.cstart = t->cstart;
-                lp.vals = t->vals;
-                lp.cols = t->cols;
-                lp.m = MatRef{h->d_rowT, h->d_colT, h->d_valT, nullptr, g, grad_x, nullptr};
-                lp.n_slices = t->n;
-                lp.n_ctas = t->n_ctas;
-                lp.alpha = alpha;
-                lp.beta = 0.0;
-                lp.dorder = t->diagonal ? t->dorder : nullptr;
-                lp.diag = t->diag;
-                lp.dshort = t->slot_rows <= 8LL * t->n;
+                const SellParams lp = sell_params(
+                    *t, MatRef{h->d_rowT, h->d_colT, h->d_valT, nullptr, g, grad_x, nullptr}, alpha, 0.0);
                 if (lops.launch(lp, s) != cudaSuccess) return SPMV_ERR_CUDA;
                 done = true;
             }
@@ -1917,7 +1984,21 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
         }
     }
     if (grad_val && h->nnz > 0) {
-        // warp chunks of kGradValE entries per lane: rows from the row-start bitmasks
+        // Rows of more than 8 entries on average: on A's diagonal slices, when a
+        // forward product or a second reverse pass has built them (27-point 128^3:
+        // FP64 138 against 162 us, FP32 63 against 112).  Else warp chunks of
+        // kGradValE entries per lane, rows from the row-start bitmasks (7-point 160^3
+        // FP64 88 us on either, 5-point 2000^2 FP32 45 against 54-65 on the slices,
+        // whose work per half slice no longer covers its set-up).
+        const SellTable *f = nullptr;
+        if (h->family == 5 && h->nnz > 8LL * h->n_rows && (again || h->sells.count(h->sigma)) && sell_tile_fits(h))
+            f = get_sell(h, h->sigma, s, false, false);
+        if (f && f->diagonal && (reinterpret_cast<uintptr_t>(grad_val) & 15u) == 0) {
+            const SellParams p = sell_params(
+                *f, MatRef{h->d_rp, h->d_col, nullptr, nullptr, x, nullptr, nullptr}, alpha, 0.0);
+            CK(launch_sell_grad_val(p, h->vk, g, grad_val, h->max_row, s));
+            return SPMV_OK;
+        }
         ChunkTable *ct = get_chunks(h, kGradValE, false);
         if (!ct) return SPMV_ERR_ALLOC;
         const int mwp = ((kGradValE + 3) / 4) * 4;

@@ -63,6 +63,9 @@ struct SellParams;
 struct SellOps {
     cudaError_t (*launch)(const SellParams &, cudaStream_t);
     int (*ctas_for)(int32_t n_slices);  // CTAs a launch over n_slices uses
+    // values read through positions (p.vpos; diagonal slices); FP32 storage in
+    // float-float, as the staged kernel that reads values through a permutation
+    cudaError_t (*launch_ind)(const SellParams &, cudaStream_t);
     // y = A x plus the dot x.y reduced into a CG reduction target (FP32
     // storage only; nullptr elsewhere)
     cudaError_t (*launch_dot)(const SellParams &, const RedOut &, cudaStream_t);
@@ -91,6 +94,23 @@ cudaError_t launch_sell_relayout(const void *slices, const int32_t *srows, int32
 // added to count[0] and [1].
 cudaError_t launch_sell_mark_diag(void *dtmp, int32_t n_slices, const int32_t *srows, const int32_t *cols,
                                   void *diag, uint32_t *count, void *dorder, cudaStream_t s);
+
+// vpos[slot] of the nT slices of A^T = position of the slot's value among the
+// values of A's nA slices, -1 in padding (rowpos: n_rows entries of scratch).
+// Every row of A lies in its slices (no long rows) and positions fit in int32.
+cudaError_t launch_sell_vpos(const void *slicesA, const int32_t *srowsA, int32_t nA, const void *slicesT,
+                             const int32_t *srowsT, int32_t nT, const int32_t *rp, const int32_t *rowT,
+                             const int32_t *colT, const int32_t *perm, int32_t *rowpos, int32_t *vpos, cudaStream_t s);
+
+// The longest row of the two launches below (every row lies in the slices).
+int sell_tile_max_row();
+// New values in CRS order (kind sk) into the handle's CRS copy dval (16-byte
+// aligned) and the slices p.vals (kind vk).  max_w: the widest slice.
+cudaError_t launch_sell_set_values(const SellParams &p, const void *val, int sk, void *dval, int vk, int max_w,
+                                   cudaStream_t s);
+// gv[k] = (p.alpha*g[row])*x[col], x = p.m.x, over the slices of p (gv in CRS
+// order, 16-byte aligned).
+cudaError_t launch_sell_grad_val(const SellParams &p, int vk, const void *g, void *gv, int max_w, cudaStream_t s);
 
 cudaError_t launch_rowvec(const KParams &p, const int32_t n_rows, int vk, int xk, int yk, int acc,
                           int T, cudaStream_t s);

@@ -2,6 +2,8 @@
 // relayout kernel: FP64 values and vectors, and FP32 storage with FP32 runs
 // (every row at most 11 entries, so a lane's chain over a row is a run) or FP32
 // runs of one block (4 slot rows) each folded into float-float.
+#include <algorithm>
+
 #include "internal.h"
 #include "sell_kernel.cuh"
 
@@ -11,18 +13,21 @@ bool sell_ops(int vk, int xk, int yk, int acc, SellOps *ops, int32_t max_row) {
     if (vk == kF64 && xk == kF64 && yk == kF64 && acc == kAccF64) {
         ops->launch = &SellKernel<double, double, double, AccF64>::launch;
         ops->ctas_for = &SellKernel<double, double, double, AccF64>::ctas_for;
+        ops->launch_ind = &SellKernel<double, double, double, AccF64>::launch_ind;
         ops->launch_dot = nullptr;
         return true;
     }
     if (vk == kF32 && xk == kF32 && yk == kF32 && acc == kAccFF && max_row <= kFRMaxRun) {
         ops->launch = &SellKernel<float, float, float, AccFR>::launch;
         ops->ctas_for = &SellKernel<float, float, float, AccFR>::ctas_for;
+        ops->launch_ind = &SellKernel<float, float, float, AccFF>::launch_ind;
         ops->launch_dot = &SellKernel<float, float, float, AccFR>::launch_dot;
         return true;
     }
     if (vk == kF32 && xk == kF32 && yk == kF32 && acc == kAccFF) {
         ops->launch = &SellKernel<float, float, float, AccFRF>::launch;
         ops->ctas_for = &SellKernel<float, float, float, AccFRF>::ctas_for;
+        ops->launch_ind = &SellKernel<float, float, float, AccFF>::launch_ind;
         ops->launch_dot = &SellKernel<float, float, float, AccFRF>::launch_dot;
         return true;
     }
@@ -130,15 +135,323 @@ cudaError_t launch_sell_mark_diag(void *dtmp, int32_t n_slices, const int32_t *s
     return cudaGetLastError();
 }
 
-cudaError_t launch_sell_relayout(const void *slices, const int32_t *srows, int32_t n_slices, const int32_t *rp,
-                                 int vk, const void *val, const int32_t *col, void *vals_out, int32_t *cols_out,
-                                 cudaStream_t s) {
-    if (n_slices <= 0) return cudaSuccess;
+// rowpos[r] = position of row r's first slot in a row-slice copy (-1 before: rows
+// outside the slices).
+__global__ void __launch_bounds__(256) k_sell_rowpos(const int2 *__restrict__ slices, const int32_t *__restrict__ srows,
+                                                     int32_t n_slices, int32_t *__restrict__ rowpos) {
+    const int64_t total = static_cast<int64_t>(n_slices) * kSellC;
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    for (int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < total; t += stride) {
+        const int32_t r = srows[t];
+        if (r >= 0) rowpos[r] = slices[t / kSellC].x * kSellC + static_cast<int32_t>(t % kSellC);
+    }
+}
+
+// vpos[slot] of the slices of A^T: where the slot's value is in A's slices (rowpos:
+// the first slot of each row of A; entry perm[k] of A lies in row colT[k]).
+__global__ void __launch_bounds__(256) k_sell_vpos(const int2 *__restrict__ slices, const int32_t *__restrict__ srows,
+                                                   int32_t n_slices, const int32_t *__restrict__ rowT,
+                                                   const int32_t *__restrict__ colT, const int32_t *__restrict__ perm,
+                                                   const int32_t *__restrict__ rp, const int32_t *__restrict__ rowpos,
+                                                   int32_t *__restrict__ vpos) {
+    const int64_t total = static_cast<int64_t>(n_slices) * kSellC;
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    for (int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < total; t += stride) {
+        const int2 d = slices[t / kSellC];
+        if (d.y <= 0) continue;
+        const int32_t row = srows[t];
+        const int32_t k0 = row >= 0 ? rowT[row] : 0;
+        const int32_t len = row >= 0 ? rowT[row + 1] - k0 : 0;
+        for (int j = 0; j < d.y; ++j) {
+            int32_t pos = -1;
+            if (j < len) {
+                const int32_t i = colT[k0 + j];
+                pos = rowpos[i] + (perm[k0 + j] - rp[i]) * kSellC;
+            }
+            vpos[(static_cast<int64_t>(d.x) + j) * kSellC + t % kSellC] = pos;
+        }
+    }
+}
+
+static int slice_grid(int32_t n_slices) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t want = (static_cast<int64_t>(n_slices) * kSellC + 255) / 256;
-    const int grid = static_cast<int>(want < 16LL * sms ? want : 16LL * sms);
+    return static_cast<int>(want < 16LL * sms ? want : 16LL * sms);
+}
+
+cudaError_t launch_sell_vpos(const void *slicesA, const int32_t *srowsA, int32_t nA, const void *slicesT,
+                             const int32_t *srowsT, int32_t nT, const int32_t *rp, const int32_t *rowT,
+                             const int32_t *colT, const int32_t *perm, int32_t *rowpos, int32_t *vpos, cudaStream_t s) {
+    if (nA <= 0 || nT <= 0) return cudaSuccess;
+    k_sell_rowpos<<<slice_grid(nA), 256, 0, s>>>(static_cast<const int2 *>(slicesA), srowsA, nA, rowpos);
+    k_sell_vpos<<<slice_grid(nT), 256, 0, s>>>(static_cast<const int2 *>(slicesT), srowsT, nT, rowT, colT, perm, rp,
+                                               rowpos, vpos);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// CRS order <-> row slices through shared memory.  A warp takes half a slice (32
+// rows of at most kTileMaxW entries, one per lane) and holds its entries in a
+// shared-memory tile, packed as they lie in CRS order: rows that follow each other
+// there form a segment (on a grid nearly always the whole half slice, two across
+// the end of a grid line), and a segment starts at its entries' alignment.  On the
+// CRS side a segment is then one contiguous run, and what goes to CRS order leaves
+// by one bulk copy (cp.async.bulk) per segment, without passing through registers;
+// on the slice side lane l reads or writes row l.  The descriptor, row and row
+// pointers of the following half slices are loaded ahead (a chain of three loads).
+// ---------------------------------------------------------------------------
+constexpr int kTileMaxW = 32;
+
+// The half slices i, i + nw, ... of a warp, each with its descriptor d, the lane's
+// row r (-1: none) and the entries [k0, k1) of that row; f(i, d, r, k0, k1).
+template <typename F>
+__device__ __forceinline__ void each_half_slice(const int4 *__restrict__ dorder, const int32_t *__restrict__ srows,
+                                                int32_t n_slices, const int32_t *__restrict__ rp, int lane, F f) {
+    const int n = 2 * n_slices, nw = gridDim.x * 8;
+    int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= n) return;
+    auto desc_of = [&](int k) { return __ldg(dorder + (k < n ? k >> 1 : n_slices - 1)); };
+    auto row_of = [&](const int4 &d, int k) {
+        return __ldg(srows + static_cast<int64_t>(d.z) * kSellC + (k & 1) * 32 + lane);
+    };
+    int4 d0 = desc_of(i), d1 = desc_of(i + nw), d2 = desc_of(i + 2 * nw);
+    int r0 = row_of(d0, i), r1 = row_of(d1, i + nw);
+    int k0 = r0 >= 0 ? __ldg(rp + r0) : 0, k1 = r0 >= 0 ? __ldg(rp + r0 + 1) : 0;
+    for (; i < n; i += nw) {
+        const int4 d3 = desc_of(i + 3 * nw);
+        const int r2 = row_of(d2, i + 2 * nw);
+        const int n0 = r1 >= 0 ? __ldg(rp + r1) : 0, n1 = r1 >= 0 ? __ldg(rp + r1 + 1) : 0;
+        f(i, d0, r0, k0, k1);
+        d0 = d1;
+        d1 = d2;
+        d2 = d3;
+        r0 = r1;
+        r1 = r2;
+        k0 = n0;
+        k1 = n1;
+    }
+}
+
+// The packing of one half slice's rows into the tile (A entries are 16 bytes).
+template <typename VT>
+struct TilePack {
+    static constexpr int A = 16 / sizeof(VT);
+    int pos;         // tile index of the lane's row
+    unsigned heads;  // lanes whose row starts a segment
+    int kend;        // at a segment's first lane: the end of its entries in CRS order
+    static __host__ __device__ constexpr int entries(int max_w) { return 32 * max_w + 33 * A; }
+    __device__ __forceinline__ TilePack(int w, int k0, int k1, int lane) {
+        const int prev = __shfl_up_sync(0xffffffffu, k1, 1);
+        heads = __ballot_sync(0xffffffffu, lane == 0 || k0 != prev);
+        const unsigned upto = heads & (0xffffffffu >> (31 - lane));
+        const int first = 31 - __clz(upto);  // the segment's first lane
+        const int ks = __shfl_sync(0xffffffffu, k0, first);
+        const int base = first * w + A * (__popc(upto) - 1);
+        pos = base + ((ks - base) & (A - 1)) + (k0 - ks);
+        const unsigned after = lane == 31 ? 0u : heads & ~(0xffffffffu >> (31 - lane));
+        kend = __shfl_sync(0xffffffffu, k1, after ? __ffs(after) - 2 : 31);
+    }
+    // The tile's entries to dst in CRS order (16-byte aligned; whole 16-byte units by
+    // bulk copy, a segment's ragged ends by its first lane).  Every lane calls it
+    // after writing its part; the tile may be written again after drain().
+    __device__ __forceinline__ void store(const VT *tile, VT *dst, int k0, int lane) const {
+        fence_proxy_async_smem();
+        __syncwarp();
+        if ((heads >> lane) & 1u) {
+            const VT *src = tile + pos - k0;  // src[k]: entry k
+            const int a0 = min((k0 + A - 1) & ~(A - 1), kend), a1 = max(a0, kend & ~(A - 1));
+            if (a1 > a0) {
+                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst + a0),
+                             "r"(smem_u32(src + a0)), "r"(static_cast<uint32_t>((a1 - a0) * sizeof(VT)))
+                             : "memory");
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            }
+            for (int k = k0; k < a0; ++k) dst[k] = src[k];
+            for (int k = a1; k < kend; ++k) dst[k] = src[k];
+        }
+    }
+    static __device__ __forceinline__ void drain() {
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        __syncwarp();
+    }
+};
+
+template <typename VT> __device__ __forceinline__ VT value_as(double v) { return narrow<VT>(v); }
+template <typename VT> __device__ __forceinline__ VT value_as(float v) {
+    if constexpr (std::is_same<VT, float>::value) return v;
+    else return widen(v);
+}
+
+// New values: from CRS order (type ST) into the handle's CRS copy dval and into
+// the slices, one read and two writes (27-point 128^3 FP64, 1.34 GB: 225 us, 5.9
+// TB/s; a copy and a layout pass of its own took 314).  Rows of at most kTileMaxW
+// entries.
+template <typename ST, typename VT>
+__global__ void __launch_bounds__(256) k_sell_set_values(const int4 *__restrict__ dorder,
+                                                         const int32_t *__restrict__ srows, int32_t n_slices,
+                                                         const int32_t *__restrict__ rp, const ST *__restrict__ val,
+                                                         VT *__restrict__ dval, VT *__restrict__ vals, int max_w) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31;
+    VT *tile = reinterpret_cast<VT *>(smem) + (threadIdx.x >> 5) * TilePack<VT>::entries(max_w);
+    const uint64_t pol = l2_evict_first_policy();
+    each_half_slice(dorder, srows, n_slices, rp, lane, [&](int i, const int4 &d, int, int k0, int k1) {
+        const TilePack<VT> t(d.y, k0, k1, lane);
+        bool free = false;  // the tile's last bulk copies have read it
+        for (unsigned m = t.heads; m; m &= m - 1) {  // segments, coalesced
+            const int h = __ffs(m) - 1;
+            const int ks = __shfl_sync(0xffffffffu, k0, h), ke = __shfl_sync(0xffffffffu, t.kend, h);
+            VT *out = tile + __shfl_sync(0xffffffffu, t.pos, h) - ks;
+            for (int k = ks + lane; __any_sync(0xffffffffu, k < ke); k += 256) {
+                ST v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = k + 32 * u < ke ? ld_stream_p(val + k + 32 * u, pol) : ST(0);
+                if (!free) TilePack<VT>::drain();
+                free = true;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (k + 32 * u < ke) out[k + 32 * u] = value_as<VT>(v[u]);
+            }
+        }
+        t.store(tile, dval, k0, lane);
+        VT *out = vals + static_cast<int64_t>(d.x) * kSellC + (i & 1) * 32 + lane;
+        const VT *row = tile + t.pos;
+        const int len = k1 - k0;
+#pragma unroll 8
+        for (int j = 0; j < d.y; ++j) out[j * kSellC] = j < len ? row[j] : VT(0);
+        __syncwarp();
+    });
+    TilePack<VT>::drain();
+}
+
+// CNT products of a lane's row along its diagonals.  wait: the tile's last bulk
+// copies may still read it; their end is waited for with the gathers in flight.
+template <int CNT, typename VT>
+__device__ __forceinline__ void grad_val_block(VT *row, VT gr, const int4 *__restrict__ dp, const VT *__restrict__ xr,
+                                               bool wait) {
+    const int4 a = __ldg(dp);
+    int4 b = make_int4(0, 0, 0, 0);
+    if constexpr (CNT > 4) b = __ldg(dp + 1);
+    const int32_t o[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    VT xv[CNT];
+#pragma unroll
+    for (int q = 0; q < CNT; ++q) xv[q] = __ldg(xr + o[q]);
+    if (wait) TilePack<VT>::drain();
+#pragma unroll
+    for (int q = 0; q < CNT; ++q) row[q] = gr * xv[q];
+}
+
+// grad_val[k] = (alpha*g[row]) * x[col[k]] on the row slices: a lane holds its
+// row's g, x is gathered along diagonals (no column indices are read for diagonal
+// slices), and the products leave through the tile in CRS order (gv 16-byte
+// aligned).  Rows of at most kTileMaxW entries.  FP64: the FP64 pipe (one multiply
+// per entry, 93 us on the 27-point 128^3 pattern) is 67 % busy at 136 us (162 on
+// the chunks of k_grad_val_pipe); FP32 60 against 111 us.  Writing each product
+// from the tile by ordinary stores instead of bulk copies: 165 and 76 us.
+template <typename VT>
+__global__ void __launch_bounds__(256) k_sell_grad_val(const SellParams p, const VT *__restrict__ g, VT *__restrict__ gv,
+                                                       int max_w) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31;
+    VT *tile = reinterpret_cast<VT *>(smem) + (threadIdx.x >> 5) * TilePack<VT>::entries(max_w);
+    const VT *__restrict__ x = static_cast<const VT *>(p.m.x);
+    const VT a = static_cast<VT>(p.alpha);
+    const bool scaled = p.alpha != 1.0;
+    each_half_slice(p.dorder, p.srows, p.n_slices, p.m.rp, lane, [&](int i, const int4 &d, int r, int k0, int k1) {
+        VT gr = r >= 0 ? __ldg(g + r) : VT(0);
+        const TilePack<VT> t(d.y, k0, k1, lane);
+        VT *row = tile + t.pos;
+        const int32_t *__restrict__ cb = p.cols + static_cast<int64_t>(d.x) * kSellC + (i & 1) * 32 + lane;
+        const int4 *__restrict__ dp = p.diag + d.w;
+        if (scaled) gr = static_cast<VT>(a * gr);
+        if (d.w >= 0) {
+            int w = d.y;
+            for (; w >= 8; w -= 8, row += 8, dp += 2) grad_val_block<8>(row, gr, dp, x + r, w == d.y);
+            switch (w) {
+                case 7: grad_val_block<7>(row, gr, dp, x + r, w == d.y); break;
+                case 6: grad_val_block<6>(row, gr, dp, x + r, w == d.y); break;
+                case 5: grad_val_block<5>(row, gr, dp, x + r, w == d.y); break;
+                case 4: grad_val_block<4>(row, gr, dp, x + r, w == d.y); break;
+                case 3: grad_val_block<3>(row, gr, dp, x + r, w == d.y); break;
+                case 2: grad_val_block<2>(row, gr, dp, x + r, w == d.y); break;
+                case 1: grad_val_block<1>(row, gr, dp, x + r, w == d.y); break;
+                default: break;
+            }
+        } else {
+            const int len = k1 - k0;
+            TilePack<VT>::drain();
+            for (int j0 = 0; j0 < d.y; j0 += 8) {
+                VT xv[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) xv[q] = j0 + q < len ? __ldg(x + __ldg(cb + (j0 + q) * kSellC)) : VT(0);
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (j0 + q < len) row[j0 + q] = gr * xv[q];
+            }
+        }
+        t.store(tile, gv, k0, lane);
+    });
+    TilePack<VT>::drain();
+}
+
+// Grid of a tile kernel: its resident CTAs, 8 half slices per CTA and turn.
+template <typename K>
+static int tile_grid(K kernel, int32_t n_slices, size_t smem) {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             8 * 8 * TilePack<double>::entries(kTileMaxW)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 256, smem) != cudaSuccess || per_sm <= 0)
+        return 0;
+    const int64_t want = (2 * static_cast<int64_t>(n_slices) + 7) / 8;
+    return static_cast<int>(std::min<int64_t>(want, static_cast<int64_t>(per_sm) * sms));
+}
+
+int sell_tile_max_row() { return kTileMaxW; }
+
+template <typename ST, typename VT>
+static cudaError_t set_values_as(const SellParams &p, const void *val, void *dval, int max_w, cudaStream_t s) {
+    const size_t smem = sizeof(VT) * 8 * TilePack<VT>::entries(max_w);
+    const int grid = tile_grid(k_sell_set_values<ST, VT>, p.n_slices, smem);
+    if (grid <= 0) return cudaErrorInvalidConfiguration;
+    k_sell_set_values<ST, VT><<<grid, 256, smem, s>>>(p.dorder, p.srows, p.n_slices, p.m.rp,
+                                                      static_cast<const ST *>(val), static_cast<VT *>(dval),
+                                                      static_cast<VT *>(const_cast<void *>(p.vals)), max_w);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sell_set_values(const SellParams &p, const void *val, int sk, void *dval, int vk, int max_w,
+                                   cudaStream_t s) {
+    if (p.n_slices <= 0) return cudaSuccess;
+    if (vk == kF64)
+        return sk == kF64 ? set_values_as<double, double>(p, val, dval, max_w, s)
+                          : set_values_as<float, double>(p, val, dval, max_w, s);
+    return sk == kF64 ? set_values_as<double, float>(p, val, dval, max_w, s)
+                      : set_values_as<float, float>(p, val, dval, max_w, s);
+}
+
+template <typename VT>
+static cudaError_t grad_val_as(const SellParams &p, const void *g, void *gv, int max_w, cudaStream_t s) {
+    const size_t smem = sizeof(VT) * 8 * TilePack<VT>::entries(max_w);
+    const int grid = tile_grid(k_sell_grad_val<VT>, p.n_slices, smem);
+    if (grid <= 0) return cudaErrorInvalidConfiguration;
+    k_sell_grad_val<VT><<<grid, 256, smem, s>>>(p, static_cast<const VT *>(g), static_cast<VT *>(gv), max_w);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sell_grad_val(const SellParams &p, int vk, const void *g, void *gv, int max_w, cudaStream_t s) {
+    if (p.n_slices <= 0) return cudaSuccess;
+    return vk == kF64 ? grad_val_as<double>(p, g, gv, max_w, s) : grad_val_as<float>(p, g, gv, max_w, s);
+}
+
+cudaError_t launch_sell_relayout(const void *slices, const int32_t *srows, int32_t n_slices, const int32_t *rp,
+                                 int vk, const void *val, const int32_t *col, void *vals_out, int32_t *cols_out,
+                                 cudaStream_t s) {
+    if (n_slices <= 0) return cudaSuccess;
+    const int grid = slice_grid(n_slices);
     const int2 *d = static_cast<const int2 *>(slices);
     if (vk == kF64)
         k_sell_relayout<double><<<grid, 256, 0, s>>>(d, srows, n_slices, rp, static_cast<const double *>(val), col,

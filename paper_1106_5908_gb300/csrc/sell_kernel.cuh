@@ -51,6 +51,7 @@ struct SellParams {
     const int4 *dorder;    // n_slices: x, y = the descriptor, z = the slice, w = its place in diag (-1: not diagonal)
     const int4 *diag;      // column minus row of each slot row of the diagonal slices, 4 to an element
     bool dshort;           // at most 8 slot rows per slice on average
+    const int32_t *vpos;   // launch_ind: position in vals of each slot's value (-1: padding)
 };
 
 // For i = 0 .. cnt-1 and both rows h of the lane, in that order:
@@ -88,6 +89,11 @@ __device__ __forceinline__ double ld_stream_p(const double *p, uint64_t pol) {
     asm("ld.global.nc.L1::no_allocate.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol));
     return v;
 }
+__device__ __forceinline__ int32_t ld_stream_p(const int32_t *p, uint64_t pol) {
+    int32_t v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+    return v;
+}
 __device__ __forceinline__ float ld_stream_p(const float *p, uint64_t pol) {
     float v;
     asm("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
@@ -97,7 +103,7 @@ __device__ __forceinline__ float ld_stream_p(const float *p, uint64_t pol) {
 // Final store of stored row `row` of m; `old` is y[row] widened, loaded ahead
 // (read only when beta is nonzero).  A poisoned float-float sum is summed again
 // in FP64 from the CRS arrays of m.
-template <typename VT, typename XT, typename YT, typename ACC>
+template <typename VT, bool INDIRECT = false, typename XT, typename YT, typename ACC>
 __device__ __forceinline__ YT sell_store(const MatRef &m, const XT *__restrict__ x, YT *__restrict__ y, int row,
                                          const ACC &a, double alpha, double beta, bool plain, double old) {
     if constexpr ((std::is_same<ACC, AccFF>::value || std::is_same<ACC, AccFR>::value ||
@@ -109,7 +115,7 @@ __device__ __forceinline__ YT sell_store(const MatRef &m, const XT *__restrict__
             return out;
         }
     }
-    const double v = acc_value<VT, false>(a, m, row, x);
+    const double v = acc_value<VT, INDIRECT>(a, m, row, x);
     double out;
     if (plain) out = v;
     else if (beta == 0.0) out = alpha * v;
@@ -322,12 +328,33 @@ __global__ void __launch_bounds__(256) k_sell(const SellParams p, const RedOut o
 // their column indices.
 // ---------------------------------------------------------------------------
 
-// CNT slot rows of a half slice: values at vb (kSellC apart), and their columns
-// row + diagonal (DIAG; 8 diagonals at dp) or as stored (cb).
-template <int CNT, bool DIAG, typename ACC, typename VT, typename XT>
-__device__ __forceinline__ void sell_diag_block(ACC &acc, const VT *__restrict__ vb, const int32_t *__restrict__ cb,
+// Where a half slice's values are: in its own slots (vb), or, IND, at position
+// pb[slot] of another copy's values (the reverse pass: the slices of A^T read the
+// values of A's slices, so new values need no layout in A^T's order).  On a grid
+// the 32 positions of a slot row are nearly consecutive in A's slices, where the
+// permutation of the CRS order put them in 32 places: 27-point 128^3, first pass
+// after new values, FP64 306 -> 132 us, FP32 684 -> 95.
+template <typename VT, bool IND>
+struct SellVals {
+    const VT *__restrict__ v;       // the slots (IND: the other copy's values)
+    const int32_t *__restrict__ p;  // IND: the slots' positions there (-1: padding)
+    __device__ __forceinline__ void skip(int rows) {
+        if constexpr (IND) p += rows * kSellC;
+        else v += rows * kSellC;
+    }
+};
+
+// CNT slot rows of a half slice (kSellC apart): their columns are row + diagonal
+// (DIAG; 8 diagonals at dp) or as stored (cb).
+template <int CNT, bool DIAG, bool IND, typename ACC, typename VT, typename XT>
+__device__ __forceinline__ void sell_diag_block(ACC &acc, const SellVals<VT, IND> &sv, const int32_t *__restrict__ cb,
                                                 const int4 *__restrict__ dp, int row, const XT *__restrict__ x,
                                                 uint64_t pol) {
+    int32_t pos[CNT];
+    if constexpr (IND) {
+#pragma unroll
+        for (int u = 0; u < CNT; ++u) pos[u] = ld_stream_p(sv.p + u * kSellC, pol);
+    }
     int32_t c[CNT];
     if constexpr (DIAG) {
         const int4 a = __ldg(dp);
@@ -342,10 +369,16 @@ __device__ __forceinline__ void sell_diag_block(ACC &acc, const VT *__restrict__
     }
     VT v[CNT];
     XT xv[CNT];
+    if constexpr (!IND) {
 #pragma unroll
-    for (int u = 0; u < CNT; ++u) v[u] = ld_stream_p(vb + u * kSellC, pol);
+        for (int u = 0; u < CNT; ++u) v[u] = ld_stream_p(sv.v + u * kSellC, pol);
+    }
 #pragma unroll
     for (int u = 0; u < CNT; ++u) xv[u] = (DIAG || c[u] >= 0) ? __ldg(x + c[u]) : XT(0);
+    if constexpr (IND) {
+#pragma unroll
+        for (int u = 0; u < CNT; ++u) v[u] = (DIAG || pos[u] >= 0) ? __ldg(sv.v + pos[u]) : VT(0);
+    }
 #pragma unroll
     for (int u = 0; u < CNT; ++u) {
         acc.fma(v[u], xv[u]);
@@ -354,29 +387,29 @@ __device__ __forceinline__ void sell_diag_block(ACC &acc, const VT *__restrict__
 }
 
 // All w slot rows of a half slice.
-template <bool DIAG, typename ACC, typename VT, typename XT>
-__device__ __forceinline__ void sell_diag_row(ACC &acc, int w, const VT *__restrict__ vb,
-                                              const int32_t *__restrict__ cb, const int4 *__restrict__ dp, int row,
-                                              const XT *__restrict__ x, uint64_t pol) {
+template <bool DIAG, bool IND, typename ACC, typename VT, typename XT>
+__device__ __forceinline__ void sell_diag_row(ACC &acc, int w, SellVals<VT, IND> sv, const int32_t *__restrict__ cb,
+                                              const int4 *__restrict__ dp, int row, const XT *__restrict__ x,
+                                              uint64_t pol) {
     for (; w >= 8; w -= 8) {
-        sell_diag_block<8, DIAG>(acc, vb, cb, dp, row, x, pol);
-        vb += 8 * kSellC;
+        sell_diag_block<8, DIAG>(acc, sv, cb, dp, row, x, pol);
+        sv.skip(8);
         if constexpr (DIAG) dp += 2;
         else cb += 8 * kSellC;
     }
     switch (w) {
-        case 7: sell_diag_block<7, DIAG>(acc, vb, cb, dp, row, x, pol); break;
-        case 6: sell_diag_block<6, DIAG>(acc, vb, cb, dp, row, x, pol); break;
-        case 5: sell_diag_block<5, DIAG>(acc, vb, cb, dp, row, x, pol); break;
-        case 4: sell_diag_block<4, DIAG>(acc, vb, cb, dp, row, x, pol); break;
-        case 3: sell_diag_block<3, DIAG>(acc, vb, cb, dp, row, x, pol); break;
-        case 2: sell_diag_block<2, DIAG>(acc, vb, cb, dp, row, x, pol); break;
-        case 1: sell_diag_block<1, DIAG>(acc, vb, cb, dp, row, x, pol); break;
+        case 7: sell_diag_block<7, DIAG>(acc, sv, cb, dp, row, x, pol); break;
+        case 6: sell_diag_block<6, DIAG>(acc, sv, cb, dp, row, x, pol); break;
+        case 5: sell_diag_block<5, DIAG>(acc, sv, cb, dp, row, x, pol); break;
+        case 4: sell_diag_block<4, DIAG>(acc, sv, cb, dp, row, x, pol); break;
+        case 3: sell_diag_block<3, DIAG>(acc, sv, cb, dp, row, x, pol); break;
+        case 2: sell_diag_block<2, DIAG>(acc, sv, cb, dp, row, x, pol); break;
+        case 1: sell_diag_block<1, DIAG>(acc, sv, cb, dp, row, x, pol); break;
         default: break;
     }
 }
 
-template <typename VT, typename XT, typename YT, typename ACC, bool DOT>
+template <typename VT, typename XT, typename YT, typename ACC, bool DOT, bool IND>
 __device__ __forceinline__ void sell_diag_walk(const SellParams &p, double &dsum) {
     constexpr int C = kSellC;
     const int lane = threadIdx.x & 31;
@@ -403,7 +436,7 @@ __device__ __forceinline__ void sell_diag_walk(const SellParams &p, double &dsum
             if ((i & 1) == 0) {
                 const int row = d.x;
                 const ChunkDesc cd{__ldg(p.m.rp + row), __ldg(p.m.rp + row + 1), row, (row + 1) | kChunkLong};
-                long_row<VT, XT, YT, ACC, false>(p.m, cd, x, y, alpha, beta, emode == kEpiPlain, lane);
+                long_row<VT, XT, YT, ACC, IND>(p.m, cd, x, y, alpha, beta, emode == kEpiPlain, lane);
                 if constexpr (DOT) {
                     if (lane == 0) dsum = fma(widen(x[row]), widen(y[row]), dsum);  // lane 0 stored it
                 }
@@ -412,10 +445,11 @@ __device__ __forceinline__ void sell_diag_walk(const SellParams &p, double &dsum
             const int64_t base = static_cast<int64_t>(d.x) * C + (i & 1) * 32 + lane;
             ACC acc;
             acc.zero();
+            SellVals<VT, IND> sv{IND ? vals : vals + base, IND ? p.vpos + base : nullptr};
             if (d.w >= 0)
-                sell_diag_row<true>(acc, d.y, vals + base, static_cast<const int32_t *>(nullptr), p.diag + d.w, r, x, pol);
+                sell_diag_row<true>(acc, d.y, sv, static_cast<const int32_t *>(nullptr), p.diag + d.w, r, x, pol);
             else
-                sell_diag_row<false>(acc, d.y, vals + base, p.cols + base, static_cast<const int4 *>(nullptr), r, x, pol);
+                sell_diag_row<false>(acc, d.y, sv, p.cols + base, static_cast<const int4 *>(nullptr), r, x, pol);
             if (r >= 0) {
                 YT q;
                 if constexpr (std::is_same<ACC, AccF64>::value) {
@@ -425,7 +459,7 @@ __device__ __forceinline__ void sell_diag_walk(const SellParams &p, double &dsum
                     y[r] = q;
                 } else {
                     const double old = emode >= kEpiAdd ? widen(y[r]) : 0.0;
-                    q = sell_store<VT>(p.m, x, y, r, acc, alpha, beta, emode == kEpiPlain, old);
+                    q = sell_store<VT, IND>(p.m, x, y, r, acc, alpha, beta, emode == kEpiPlain, old);
                 }
                 if constexpr (DOT) dsum = fma(widen(__ldg(x + r)), widen(q), dsum);
             }
@@ -443,10 +477,10 @@ __device__ __forceinline__ void sell_diag_walk(const SellParams &p, double &dsum
 template <typename VT, bool SHORT>
 constexpr int kSellDiagCtas = (sizeof(VT) == 8 ? 4 : 5) + (SHORT ? 1 : 0);
 
-template <typename VT, typename XT, typename YT, typename ACC, bool SHORT, bool DOT>
+template <typename VT, typename XT, typename YT, typename ACC, bool SHORT, bool DOT, bool IND = false>
 __global__ void __launch_bounds__(256, (kSellDiagCtas<VT, SHORT>)) k_sell_diag(const SellParams p, const RedOut o) {
     double dsum = 0.0;
-    sell_diag_walk<VT, XT, YT, ACC, DOT>(p, dsum);
+    sell_diag_walk<VT, XT, YT, ACC, DOT, IND>(p, dsum);
     if constexpr (DOT) {
         __shared__ double s_red[32];
         finish(block_sum(dsum, s_red), o, s_red);
@@ -665,7 +699,8 @@ __global__ void __launch_bounds__(256, 2) k_sell_mr(const SellMrParams q) {
 
 // Slot-major copy of the regular slices: row h*32 + l of slice s, holding row
 // r, has entry rp[r] + j at slot (off + j)*64 + h*32 + l for j < len(r), value 0
-// and column -1 after it.  cols_out may be null (values only, after new values).
+// and column -1 after it.  cols_out may be null (values only, after new values),
+// vals_out too (columns only).
 template <typename VT>
 __global__ void __launch_bounds__(256) k_sell_relayout(const int2 *__restrict__ slices,
                                                        const int32_t *__restrict__ srows, int32_t n_slices,
@@ -684,7 +719,7 @@ __global__ void __launch_bounds__(256) k_sell_relayout(const int2 *__restrict__ 
         for (int j = 0; j < d.y; ++j) {
             const int64_t slot = (static_cast<int64_t>(d.x) + j) * kSellC + hl;
             const bool ok = j < len;
-            vals_out[slot] = ok ? val[k0 + j] : VT(0);
+            if (vals_out) vals_out[slot] = ok ? val[k0 + j] : VT(0);
             if (cols_out) cols_out[slot] = ok ? col[k0 + j] : -1;
         }
     }
@@ -716,7 +751,7 @@ struct SellKernel {
         return static_cast<int>(want < lim ? want : lim);
     }
     // k_sell_diag on up to its resident CTAs, 8 half slices per CTA and turn
-    template <bool SHORT, bool DOT>
+    template <bool SHORT, bool DOT, bool IND = false>
     static cudaError_t launch_diag(const SellParams &p, const RedOut &o, cudaStream_t s) {
         static int cached = -1;
         static int cached_dev = -1;
@@ -725,7 +760,7 @@ struct SellKernel {
         if (cached < 0 || cached_dev != dev) {
             int per_sm = 0, sms = 0;
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sell_diag<VT, XT, YT, ACC, SHORT, DOT>, 256,
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sell_diag<VT, XT, YT, ACC, SHORT, DOT, IND>, 256,
                                                               0) != cudaSuccess ||
                 per_sm <= 0)
                 return cudaErrorInvalidConfiguration;
@@ -735,7 +770,7 @@ struct SellKernel {
         const int64_t want = (2 * static_cast<int64_t>(p.n_slices) + 7) / 8;
         const int grid = static_cast<int>(want < cached ? want : cached);
         if (DOT && grid > cg_partials_cap()) return cudaErrorInvalidConfiguration;
-        k_sell_diag<VT, XT, YT, ACC, SHORT, DOT><<<grid, 256, 0, s>>>(p, o);
+        k_sell_diag<VT, XT, YT, ACC, SHORT, DOT, IND><<<grid, 256, 0, s>>>(p, o);
         return cudaGetLastError();
     }
     static cudaError_t launch(const SellParams &p, cudaStream_t s) {
@@ -744,6 +779,13 @@ struct SellKernel {
             return p.dshort ? launch_diag<true, false>(p, RedOut{}, s) : launch_diag<false, false>(p, RedOut{}, s);
         k_sell<VT, XT, YT, ACC, false><<<p.n_ctas, 256, 0, s>>>(p, RedOut{});
         return cudaGetLastError();
+    }
+    // y = A x on diagonal slices whose values are read through positions (p.vpos)
+    static cudaError_t launch_ind(const SellParams &p, cudaStream_t s) {
+        if (p.n_slices <= 0 || p.n_ctas <= 0) return cudaSuccess;
+        if (!p.dorder || !p.vpos) return cudaErrorInvalidValue;
+        return p.dshort ? launch_diag<true, false, true>(p, RedOut{}, s)
+                        : launch_diag<false, false, true>(p, RedOut{}, s);
     }
     // y = A x with the dot x.y reduced into o (the CG step's p.q); needs at least
     // one slice and at most cg_partials_cap() CTAs

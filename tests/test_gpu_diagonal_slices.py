@@ -69,6 +69,38 @@ def test_diagonal_slices_match_the_oracle(n, width, broken, long_rows, dtype):
     assert_bitexact(host(M.apply(dev(xi.astype(ft)))).astype(np.float64), oracle.spmv(*B.astuple(), xi), "integers")
 
 
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("n,width,broken", [(65, 3, 0), (5000, 4, 3), (9000, 7, 5), (70, 10, 0), (8191, 9, 0),
+                                            (5003, 12, 40), (4097, 16, 3), (9001, 32, 2), (6000, 33, 2), (3000, 70, 1)])
+def test_training_steps_match_the_oracle(n, width, broken, dtype):
+    """New values, the forward product and reverse passes on them (the first reads
+    A's slices through positions, the second A^T's own copy), each against the oracle."""
+    from paper_1106_5908_gb300 import Matrix
+    ft, tt = (np.float64, torch.float64) if dtype == "f64" else (np.float32, torch.float32)
+    tol = 1e-13 if dtype == "f64" else 1e-6
+    A = banded(n, width, seed=3 * n + width, broken=broken)
+    M = Matrix.from_csr(A.row_ptr, A.col_idx, A.val.astype(ft), n)
+    M.set_plan(5, 0)
+    x, g = W.uniform(n, 1).astype(ft), W.uniform(n, 2).astype(ft)
+    xd, gd = x.astype(np.float64), g.astype(np.float64)
+    M.apply(dev(x))
+    for step, alpha in enumerate((1.0, -0.5, 1.0)):
+        # values of the other type every second step: converted as they are set
+        raw = np.random.default_rng(step).standard_normal(A.nnz).astype(np.float32)
+        M.set_values(dev(raw) if step % 2 else dev(raw.astype(ft)))
+        val = raw.astype(np.float64)
+        if step == 2:
+            M.set_plan(5, 256)  # other slices: the positions of the values change
+        ref, bound = oracle.spmv(A.row_ptr, A.col_idx, val, xd, with_bound=True)
+        assert_within(host(M.apply(dev(x), alpha=alpha)), alpha * ref, abs(alpha) * bound, tol, f"forward {step}")
+        rgx, rgv, gbound = oracle.backward(A.row_ptr, A.col_idx, val, n, gd, xd, with_bound=True)
+        for rep in range(3):
+            gx, gv = M.backward(dev(g), dev(x), alpha)
+            assert gx.dtype == tt and gv.dtype == tt
+            assert_within(host(gx), alpha * rgx, abs(alpha) * gbound, tol, f"grad_x {step} {rep}")
+            assert_within(host(gv), alpha * rgv, np.abs(alpha * rgv), 1e-6 if dtype == "f32" else 1e-15, f"grad_val {step} {rep}")
+
+
 def test_tuner_takes_grid_stencils():
     """FP64 stencils on a grid of at least 16,384 points run on the row slices
     whatever their row length; a banded matrix without diagonals does not."""
