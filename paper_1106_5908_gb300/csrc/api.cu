@@ -379,7 +379,7 @@ struct DeviceGuard {
 
 }  // namespace
 
-constexpr int32_t kCheckEvery = 8;  // CG iterations between residual read-backs
+constexpr int32_t kCheckEvery = kCgCheckEvery;  // CG iterations between residual read-backs
 
 struct CgWork {
     int64_t n = 0;
@@ -387,6 +387,9 @@ struct CgWork {
     float *r32 = nullptr, *d32 = nullptr, *p32 = nullptr, *q32 = nullptr;
     double *sc = nullptr, *partials = nullptr;
     double *host = nullptr;  // pinned scalars
+    // the one-kernel solve: the barrier marks of one_ctas CTAs, results
+    double *one = nullptr;
+    int32_t one_ctas = 0;
     // kCheckEvery CG iterations captured once and replayed (host launch overhead
     // paid once per block); re-captured when the operands or the plan change
     cudaGraphExec_t inner32 = nullptr;  // FP32 inner CG of the IR solver
@@ -429,6 +432,7 @@ struct spmv_matrix {
     std::map<int, SellTable> sellsT;                    // sigma -> sorted row-slice copy of A^T (reverse pass)
     double sell_padT = -1.0;                            // padding of A^T's slices (computed on first use)
     int32_t sigma = 4096;                               // family 5: rows per sorting window
+    bool planned = false;                               // the caller chose the plan
     bool sell_if_diag = false;                          // family 5 by the tuner for its diagonal slices only
     double sell_pad = 1.0;                              // padding of sorted slices of 4096-row windows
     int32_t *d_rmap = nullptr;                          // output row of each stored row
@@ -926,7 +930,7 @@ void destroy_cg(CgWork &w) {
     if (w.cg64) cudaGraphExecDestroy(w.cg64);
     cudaFree(w.r64); cudaFree(w.p64); cudaFree(w.q64);
     cudaFree(w.r32); cudaFree(w.d32); cudaFree(w.p32); cudaFree(w.q32);
-    cudaFree(w.sc); cudaFree(w.partials);
+    cudaFree(w.sc); cudaFree(w.partials); cudaFree(w.one);
     if (w.host) cudaFreeHost(w.host);
     w = CgWork();
 }
@@ -1155,6 +1159,8 @@ spmv_status ensure_cg(spmv_matrix *h, bool mixed) {
         if (cudaMemset(w.partials, 0, static_cast<size_t>(cg_partials_len()) * 8) != cudaSuccess) return SPMV_ERR_CUDA;
         if (cudaMallocHost(reinterpret_cast<void **>(&w.host), 8 * sizeof(double)) != cudaSuccess) return SPMV_ERR_ALLOC;
         if (dmalloc(&w.r64, n) != cudaSuccess) return SPMV_ERR_ALLOC;
+        CK(cudaDeviceGetAttribute(&w.one_ctas, cudaDevAttrMultiProcessorCount, h->device));
+        if (dmalloc(&w.one, 4 * static_cast<size_t>(w.one_ctas) + 4) != cudaSuccess) return SPMV_ERR_ALLOC;
     }
     if (!mixed && w.p64 == nullptr) {
         if (dmalloc(&w.p64, n) != cudaSuccess) return SPMV_ERR_ALLOC;
@@ -1204,6 +1210,34 @@ spmv_status ensure_mirror32(spmv_matrix *h, cudaStream_t s) {
 }
 
 }  // namespace
+
+// CG on h as one cooperative kernel (launch_cg), when h runs on diagonal row slices
+// (by the tuner, whatever its size) and the vectors of a CTA's rows fit in shared
+// memory.  res: rho, iterations, b.b.  SPMV_ERR_UNSUPPORTED: not this matrix.
+// work: the CG work array of the handle that runs the solve (its partials).
+static spmv_status cg_in_one_kernel(spmv_matrix *h, CgWork &w, const void *b, void *x, void *dir, void *dir2, void *r,
+                                    double tol, int32_t max_iter, double *res, cudaStream_t s) {
+    const bool grid_like = h->col_diag >= kDiagMinShare && h->sell_pad <= kSellMaxPadding && h->acc32 == kAccFF;
+    if (h->n_rows == 0 || h->max_row > kSellLongRow || h->d_rmap ||
+        !(h->planned ? h->family == 5 && h->sigma == kSellSigma : grid_like))
+        return SPMV_ERR_UNSUPPORTED;
+    const int32_t few = (h->n_rows + kSellC - 1) / kSellC;  // at least this many slices
+    if (!cg_kernel_fits(h->vk, few, h->max_row)) return SPMV_ERR_UNSUPPORTED;
+    SellTable *t = get_sell(h, kSellSigma, s);
+    if (!t || !t->diagonal || t->n_long > 0 || !cg_kernel_fits(h->vk, t->n, h->max_row)) return SPMV_ERR_UNSUPPORTED;
+    const SellParams p =
+        sell_params(*t, MatRef{h->d_rp, h->d_col, h->d_val, nullptr, nullptr, nullptr, nullptr}, 1.0, 0.0);
+    double *out = w.one + 4 * static_cast<int64_t>(w.one_ctas);
+    if (launch_cg(p, t->dtmp, h->vk, h->max_row, b, x, dir, dir2, r, tol, max_iter, w.one, out, h->d_err, s) != cudaSuccess) {
+        (void)cudaGetLastError();  // not launched: the kernel-by-kernel path runs
+        return SPMV_ERR_UNSUPPORTED;
+    }
+    CK(cudaMemcpyAsync(w.host, out, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    if (w.host[3] != 0.0) return SPMV_ERR_TIMEOUT;
+    for (int i = 0; i < 3; ++i) res[i] = w.host[i];
+    return SPMV_OK;
+}
 
 // Everything an apply needs (chunk tables) is built before a capture, so no
 // allocation happens while a stream is being captured.
@@ -1471,6 +1505,7 @@ spmv_status spmv_row_histogram(spmv_handle h, int32_t nbins, int64_t *counts) {
 spmv_status spmv_set_plan(spmv_handle h, int32_t family, int32_t param) {
     if (!h || family < 0 || family > 6) return SPMV_ERR_INVALID_ARG;
     h->sell_if_diag = false;
+    h->planned = true;
     if (family == 6) {
         const bool f64 = h->vk == kF64;
         if (param != 0 && !(f64 ? (param == 7 || param == 9) : (param == 9 || param == 15)))
@@ -2392,6 +2427,17 @@ spmv_status spmv_cg(spmv_handle h, const double *b, double *x, double tol, int32
     if (st != SPMV_OK) return st;
     CgWork &w = h->cg;
     const int64_t n = h->n_rows;
+    double bb = 0.0, rho = 0.0;
+    int32_t it = 0;
+    double one[3];
+    st = cg_in_one_kernel(h, w, b, x, w.p64, w.q64, w.r64, tol, max_iter, one, s);
+    if (st != SPMV_OK && st != SPMV_ERR_UNSUPPORTED) return st;
+    const bool solved = st == SPMV_OK;
+    if (solved) {
+        rho = one[0];
+        it = static_cast<int32_t>(one[1]);
+        bb = one[2];
+    } else {
     // x = 0, r = b, p = b, rho = b.b
     CK(cudaMemsetAsync(x, 0, static_cast<size_t>(n) * 8, s));
     CK(cudaMemcpyAsync(w.r64, b, static_cast<size_t>(n) * 8, cudaMemcpyDeviceToDevice, s));
@@ -2399,9 +2445,7 @@ spmv_status spmv_cg(spmv_handle h, const double *b, double *x, double tol, int32
     CK(cg_dot(b, kF64, b, kF64, n, w.partials, w.sc, kOpStore, kScRho, s));
     CK(cudaMemcpyAsync(w.host, w.sc + kScRho, 8, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
-    const double bb = w.host[0];
-    double rho = bb;
-    int32_t it = 0;
+    bb = rho = w.host[0];
     // the residual is read back every kCheckEvery iterations (one host round trip
     // per check, not per iteration); CG may run up to kCheckEvery-1 extra steps
     auto iter = [&](cudaStream_t cs) -> spmv_status {
@@ -2444,6 +2488,7 @@ spmv_status spmv_cg(spmv_handle h, const double *b, double *x, double tol, int32
         CK(cudaMemcpyAsync(w.host, w.sc + kScRho, 8, cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         rho = w.host[0];
+    }
     }
     // true residual in FP64
     CK(cudaMemcpyAsync(w.r64, b, static_cast<size_t>(n) * 8, cudaMemcpyDeviceToDevice, s));
@@ -2501,6 +2546,15 @@ spmv_status spmv_ir_cg(spmv_handle h, const double *b, double *x, double outer_t
         if (outer >= max_outer) break;
         // inner (FP32 storage): CG on A d = r / ||r||
         CK(cg_scale_to32(w.r64, w.r32, 1.0 / rnorm, n, s));
+        double one[3];
+        st = cg_in_one_kernel(A32, w, w.r32, w.d32, w.p32, w.q32, w.r32, inner_tol, max_inner, one, s);
+        if (st == SPMV_OK) {
+            inner_total += static_cast<int32_t>(one[1]);
+            CK(cg_axpy_64_32(x, w.d32, rnorm, n, s));
+            ++outer;
+            continue;
+        }
+        if (st != SPMV_ERR_UNSUPPORTED) return st;
         CK(cudaMemsetAsync(w.d32, 0, static_cast<size_t>(n) * 4, s));
         CK(cudaMemcpyAsync(w.p32, w.r32, static_cast<size_t>(n) * 4, cudaMemcpyDeviceToDevice, s));
         CK(cg_dot(w.r32, kF32, w.r32, kF32, n, w.partials, w.sc, kOpStore, kScRho, s));
