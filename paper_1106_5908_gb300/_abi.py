@@ -100,6 +100,7 @@ def load() -> ctypes.CDLL:
         fn = getattr(lib, name)
         fn.restype = res
         fn.argtypes = args
+        globals()[name] = fn  # later calls go straight to the library
     _lib = lib
     return lib
 
@@ -120,7 +121,7 @@ def _fwd(name):
     def f(*args):
         return getattr(load(), name)(*args)
     f.__name__ = name
-    f.__doc__ = f"Direct call of the C entry point {name} (see include/spmv.h)."
+    f.__doc__ = f"Loads the library, then calls the C entry point {name} (see include/spmv.h)."
     return f
 
 
