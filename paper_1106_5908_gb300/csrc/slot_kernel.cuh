@@ -199,7 +199,7 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
                 epi.store(y, srow, r1 - r0, alpha, beta, emode, lane);
             } else {
                 for (int q = lane; q < r1 - r0; q += 32) {
-                    if constexpr (std::is_same<ACC, AccF64>::value) {
+                    if constexpr (std::is_same<ACC, AccF64>::value && !BATCHED) {
                         const int64_t row = m.rmap ? __ldg(m.rmap + r0 + q) : r0 + q;
                         y[row] = narrow<YT>(epi_apply(srow[q].get(), y + row, alpha, beta, emode));
                     } else {
