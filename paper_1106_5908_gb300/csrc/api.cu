@@ -1856,32 +1856,32 @@ spmv_status spmm_apply(spmv_handle h, int32_t nrhs, double alpha, const void *X,
     if (h->n_rows == 0) return SPMV_OK;
     if (nrhs == 1) return apply_impl(h, alpha, X, kF64, beta, Y, kF64, s);
     int32_t c0 = 0;
-    // Groups of 4 right-hand sides on the sorted row slices (one FMA chain per
-    // row and right-hand side, no carries), when the slices pad little and, for
-    // scattered columns, X fits in L2: each group gathers 32 bytes of a row of X
-    // per entry, which costs a DRAM burst apiece once X is out of L2, where the
-    // tile kernel reads whole rows of X once.  Measured (ms, slices against the
-    // tile kernel): 27-point 128^3 nrhs 4 / 8 / 16 / 32: 0.384 / 0.767 / 1.774 /
-    // 3.566 against 0.589 / 1.155 / 2.242 / 4.261; Hamiltonian-like (X of 134 MB
-    // per 4 right-hand sides) nrhs 4: 0.465 against 0.591, nrhs 8 / 16 / 32:
-    // 1.461 / 3.999 / 8.156 against 1.105 / 2.125 / 4.104.
+    // On the sorted row slices when they pad little: lanes across the right-hand
+    // sides, up to 32 per pass; exactly 4 with a lane per two rows (k_sell_mr) when
+    // neighbouring rows share x in L1, or when X is too large for L2 to keep the
+    // rows of X between its reads either way (Hamiltonian-like: 4.2 M rows, X 134
+    // MB, 461 against 478 us; 300,000 rows 50 against 36; 27-point 101^3 192
+    // against 194, 5-point 1400^2 74 against 80).
     int l2 = 0;
     cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, h->device);
-    const bool x_fits = static_cast<double>(h->n_cols) * nrhs * 8.0 <= 1.25 * l2;
+    const bool scattered = h->col_random > 0.25;
     SellTable *t = nullptr;
-    if (nrhs >= kSellR && h->sell_pad <= kSellMaxPadding && (h->col_random <= 0.25 || x_fits) &&
-        (t = get_sell(h, kSellSigma, s)) != nullptr) {
+    if (h->sell_pad <= kSellMaxPadding && (t = get_sell(h, kSellSigma, s)) != nullptr) {
         const bool vec = (nrhs % 2 == 0) && (reinterpret_cast<uintptr_t>(X) % 16 == 0) &&
                          (reinterpret_cast<uintptr_t>(Y) % 16 == 0);
         const SellParams b =
             sell_params(*t, MatRef{h->d_rp, h->d_col, h->d_val, nullptr, nullptr, nullptr, nullptr}, alpha, beta);
-        for (; c0 + kSellR <= nrhs; c0 += kSellR)
-            if (launch_sell_mr(b, static_cast<const double *>(X) + c0, static_cast<double *>(Y) + c0, nrhs, nrhs,
-                               vec, s) != cudaSuccess)
-                return SPMV_ERR_CUDA;
+        const double *Xd = static_cast<const double *>(X);
+        double *Yd = static_cast<double *>(Y);
+        if (nrhs == kSellR && (!scattered || static_cast<double>(h->n_cols) * nrhs * 8.0 > 0.5 * l2)) {
+            CK(launch_sell_mr(b, Xd, Yd, nrhs, nrhs, vec, s));
+            return SPMV_OK;
+        }
+        for (; c0 < nrhs; c0 += kSellMaxRhs)
+            CK(launch_sell_rhs(b, Xd + c0, Yd + c0, nrhs, nrhs, std::min(kSellMaxRhs, nrhs - c0), vec, scattered, s));
+        return SPMV_OK;
     }
-    // the remaining right-hand sides (all of them without the slices): the tile
-    // kernel, up to 32 per launch
+    // without the slices: the tile kernel, up to 32 per launch
     for (; c0 < nrhs; c0 += 32) {
         const int cnt = std::min(32, nrhs - c0);
         int R = 2;

@@ -80,6 +80,11 @@ bool sell_ops(int vk, int xk, int yk, int acc, SellOps *ops, int32_t max_row = 0
 // ldx and ldy allow 16-byte accesses.
 cudaError_t launch_sell_mr(const SellParams &b, const double *X, double *Y, int64_t ldx, int64_t ldy, bool vec,
                            cudaStream_t s);
+// The same for R <= kSellMaxRhs right-hand sides with lanes across them.  scattered:
+// x gathers find no neighbours in L1.
+constexpr int kSellMaxRhs = 32;
+cudaError_t launch_sell_rhs(const SellParams &b, const double *X, double *Y, int64_t ldx, int64_t ldy, int R, bool vec,
+                            bool scattered, cudaStream_t s);
 // Slot-major copies of the values (and, when cols_out is not null, the column
 // indices) of the regular slices in `slices` (int2[n_slices]; srows: 32 rows per
 // slice) from the CRS arrays rp, val, col.

@@ -43,6 +43,56 @@ cudaError_t launch_sell_mr(const SellParams &b, const double *X, double *Y, int6
     return cudaGetLastError();
 }
 
+// How a pass of R right-hand sides runs: V per lane, L = ceil(R/V) lanes per row, G =
+// 32/L rows at a time.  The FP64 pipe needs V warp FMAs (17 cycles each) per G rows
+// and slot; with scattered columns L1 also looks up a line per row for each of the
+// pass's load instructions; 6 stand for the rest of a slot's work (16 right-hand
+// sides on the 5-point matrix: V = 4 280 us, V = 2 350).  V odd, or rows not 16-byte aligned: one load per
+// right-hand side, else one per two.
+static void rhs_plan(int R, bool vec, bool scattered, int *V_out, bool *vec_out) {
+    double best = 1e30;
+    for (int V = 2; V <= 7; ++V) {
+        const bool pv = vec && V % 2 == 0 && R % V == 0;
+        if (V == 6 && !pv) continue;
+        const int L = (R + V - 1) / V;
+        if (L > 16) continue;
+        const int G = 32 / L;
+        const double fma = 17.0 * V, lines = scattered ? (pv ? V / 2 : V) * G + 4.0 : 0.0;
+        const double cost = ((fma > lines ? fma : lines) + 6.0) / G * (pv ? 1.0 : 1.02);
+        if (cost < best) {
+            best = cost;
+            *V_out = V;
+            *vec_out = pv;
+        }
+    }
+}
+
+cudaError_t launch_sell_rhs(const SellParams &b, const double *X, double *Y, int64_t ldx, int64_t ldy, int R, bool vec,
+                            bool scattered, cudaStream_t s) {
+    if (b.n_slices <= 0 || b.n_ctas <= 0) return cudaSuccess;
+    if (R < 1 || R > kSellMaxRhs) return cudaErrorInvalidValue;
+    int V = 2;
+    bool pv = false;
+    rhs_plan(R, vec, scattered, &V, &pv);
+    const int L = (R + V - 1) / V;
+    const SellRhsParams q{SellMrParams{b, X, Y, ldx, ldy}, R, L, 32 / L};
+    switch (V) {
+        case 2:
+            if (pv) k_sell_rhs<2, true><<<b.n_ctas, 512, 0, s>>>(q);
+            else k_sell_rhs<2, false><<<b.n_ctas, 512, 0, s>>>(q);
+            break;
+        case 3: k_sell_rhs<3, false><<<b.n_ctas, 512, 0, s>>>(q); break;
+        case 4:
+            if (pv) k_sell_rhs<4, true><<<b.n_ctas, 512, 0, s>>>(q);
+            else k_sell_rhs<4, false><<<b.n_ctas, 512, 0, s>>>(q);
+            break;
+        case 5: k_sell_rhs<5, false><<<b.n_ctas, 512, 0, s>>>(q); break;
+        case 6: k_sell_rhs<6, true><<<b.n_ctas, 512, 0, s>>>(q); break;
+        default: k_sell_rhs<7, false><<<b.n_ctas, 512, 0, s>>>(q); break;
+    }
+    return cudaGetLastError();
+}
+
 // One warp per slice of dtmp: the diagonals of a diagonal slice into diag from
 // the slice's place on; place -1 for a slice that is not diagonal.  count[0], [1]:
 // slot rows and number of the diagonal slices.  A row of a diagonal slice has a

@@ -697,6 +697,134 @@ __global__ void __launch_bounds__(256, 2) k_sell_mr(const SellMrParams q) {
     }
 }
 
+// ---------------------------------------------------------------------------
+// Block vectors, lanes across the right-hand sides: a group of L lanes takes a row
+// (V right-hand sides per lane), G = 32/L groups the G next rows of a slice.  One
+// row of X is then one contiguous access per group, whatever the width of the pass,
+// where a lane per row needs a cache line of its own for every 16 bytes; the value
+// and column of a slot are one broadcast load per group.  Each lane runs V chains;
+// blocks of a few slot rows of loads, then their FMAs, and the resident warps (32
+// per SM) keep the FP64 pipe, which bounds it, busy: Hamiltonian-like 4.2 M rows, 16
+// and 32 right-hand sides 1,530 and 3,105 us (2,107 and 4,063 on the tile kernel; one
+// FMA per entry and right-hand side takes 1,448 and 2,896), 5-point 1400^2 280 and 552
+// (594 and 1,315; 262 and 524), 27-point 101^3, 5: 253 (371; 228).  VEC: the rows of X and Y allow 16-byte accesses (R
+// even); otherwise the right-hand sides are loaded one by one and the last lane of a
+// group may hold fewer than V.
+// ---------------------------------------------------------------------------
+struct SellRhsParams {
+    SellMrParams m;  // one pass: X and Y at its first right-hand side
+    int R, L, G;
+};
+
+template <int CNT, int V, bool VEC>
+__device__ __forceinline__ void sell_rhs_block(double (&acc)[V], const double *__restrict__ vb,
+                                               const int32_t *__restrict__ cb, const double *__restrict__ X,
+                                               int64_t ldx, int nv) {
+    int32_t c[CNT];
+    double v[CNT], x[CNT][V];
+#pragma unroll
+    for (int u = 0; u < CNT; ++u) c[u] = __ldg(cb + u * kSellC);
+#pragma unroll
+    for (int u = 0; u < CNT; ++u) v[u] = __ldg(vb + u * kSellC);
+#pragma unroll
+    for (int u = 0; u < CNT; ++u) {
+        const double *xp = X + static_cast<int64_t>(c[u]) * ldx;
+        if constexpr (VEC) {
+#pragma unroll
+            for (int r = 0; r < V; r += 2) {
+                const double2 t = c[u] >= 0 ? __ldg(reinterpret_cast<const double2 *>(xp + r)) : make_double2(0.0, 0.0);
+                x[u][r] = t.x;
+                x[u][r + 1] = t.y;
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < V; ++r) x[u][r] = (c[u] >= 0 && r < nv) ? __ldg(xp + r) : 0.0;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < CNT; ++u)
+#pragma unroll
+        for (int r = 0; r < V; ++r) acc[r] = fma(v[u], x[u][r], acc[r]);
+}
+
+template <int V, bool VEC>
+__global__ void __launch_bounds__(512, 2) k_sell_rhs(const SellRhsParams q) {
+    constexpr int C = kSellC;
+    const SellParams &p = q.m.b;
+    const int lane = threadIdx.x & 31, L = q.L, G = q.G;
+    if (static_cast<int>(blockIdx.x) >= p.n_ctas) return;
+    const int s0 = __ldg(p.cstart + blockIdx.x), n = __ldg(p.cstart + blockIdx.x + 1);
+    const int U = (C + G - 1) / G;  // units of G rows per slice
+    const int g = lane / L;
+    int c = (lane - g * L) * V;     // first right-hand side of the lane
+    const int nv = g < G ? min(V, q.R - c) : 0;
+    if (nv <= 0) c = 0;             // an idle lane reads what its group's first lane reads
+    const double *__restrict__ vals = static_cast<const double *>(p.vals);
+    const double *__restrict__ X = q.m.X + c;
+    const int64_t ldx = q.m.ldx, ldy = q.m.ldy;
+    const double alpha = p.alpha, beta = p.beta;
+    const int emode = epi_mode(alpha, beta);
+    for (int u = threadIdx.x >> 5; u < (n - s0) * U; u += 16) {
+        const int s = s0 + u / U, b = u % U;
+        const int2 d = __ldg(p.slices + s);
+        double acc[V];
+#pragma unroll
+        for (int r = 0; r < V; ++r) acc[r] = 0.0;
+        int row = -1;
+        if (d.y < 0) {
+            // a long row: the groups stride its entries, group 0 sums them in order
+            if (b) continue;
+            const int k1 = __ldg(p.m.rp + d.x + 1);
+            if (g < G)
+                for (int k = __ldg(p.m.rp + d.x) + g; k < k1; k += G) {
+                    const double v = __ldg(static_cast<const double *>(p.m.vs) + k);
+                    const double *xp = X + static_cast<int64_t>(__ldg(p.m.col + k)) * ldx;
+#pragma unroll
+                    for (int r = 0; r < V; ++r)
+                        if (r < nv) acc[r] = fma(v, __ldg(xp + r), acc[r]);
+                }
+            for (int o = 1; o < G; ++o)
+#pragma unroll
+                for (int r = 0; r < V; ++r) {
+                    const double t = __shfl_sync(0xffffffffu, acc[r], (lane + o * L) & 31);
+                    if (g == 0) acc[r] += t;
+                }
+            if (g == 0) row = d.x;
+        } else {
+            const int i = b * G + g;
+            const bool ok = g < G && i < C;
+            const int64_t base = static_cast<int64_t>(d.x) * C + (ok ? i : 0);
+            if (ok) row = __ldg(p.srows + static_cast<int64_t>(s) * C + i);
+            const double *__restrict__ vb = vals + base;
+            const int32_t *__restrict__ cb = p.cols + base;
+            constexpr int B = V <= 4 ? 4 : V <= 5 ? 3 : 2;  // slot rows in flight (registers)
+            int w = d.y;
+            for (; w >= B; w -= B) {
+                sell_rhs_block<B, V, VEC>(acc, vb, cb, X, ldx, nv);
+                vb += B * C;
+                cb += B * C;
+            }
+            if (B > 3 && w == 3) sell_rhs_block<3, V, VEC>(acc, vb, cb, X, ldx, nv);
+            else if (B > 2 && w == 2) sell_rhs_block<2, V, VEC>(acc, vb, cb, X, ldx, nv);
+            else if (w == 1) sell_rhs_block<1, V, VEC>(acc, vb, cb, X, ldx, nv);
+        }
+        if (row >= 0 && nv > 0) {
+            double *yp = q.m.Y + static_cast<int64_t>(row) * ldy + c;
+#pragma unroll
+            for (int r = 0; r < V; ++r)
+                if (VEC || r < nv) acc[r] = epi_apply(acc[r], yp + r, alpha, beta, emode);
+            if constexpr (VEC) {
+#pragma unroll
+                for (int r = 0; r < V; r += 2) reinterpret_cast<double2 *>(yp)[r / 2] = make_double2(acc[r], acc[r + 1]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < V; ++r)
+                    if (r < nv) yp[r] = acc[r];
+            }
+        }
+    }
+}
+
 // Slot-major copy of the regular slices: row h*32 + l of slice s, holding row
 // r, has entry rp[r] + j at slot (off + j)*64 + h*32 + l for j < len(r), value 0
 // and column -1 after it.  cols_out may be null (values only, after new values),
