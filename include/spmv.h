@@ -89,13 +89,16 @@ void spmv_destroy(spmv_handle h);
  * given by U, its upper triangle with the diagonal: row_ptr[n+1], col_idx[nnz]
  * and val[nnz] as for spmv_create, every entry of row i having a column
  * j >= i (repeated entries are summed; columns need not be sorted), so each
- * off-diagonal value is stored once and serves a_ij and a_ji.  spmv_apply on
- * the handle computes y = alpha*A*x + beta*y with A = U + U_s^T (U_s: U
- * without its diagonal) in two passes of fixed summation order: the row sums
- * of U on the autotuned kernel (with beta), then the row sums of U_s^T added
- * onto y by the warp-chunk kernel that reads each value through its position
- * in U (a transposed index built once here, on the host: rows of U_s^T list
- * their entries by increasing position in U).  Results are deterministic.
+ * off-diagonal value is given once and serves a_ij and a_ji.  spmv_apply on the
+ * handle computes y = alpha*A*x + beta*y with A = U + U_s^T (U_s: U without its
+ * diagonal).  The first apply expands A into device memory (12 bytes per entry of A
+ * beside its plan's copy, and 4 for the place of each value in U) and applies run on
+ * it with its autotuned plan.  After spmv_set_plan, or when A does not fit, an apply
+ * takes two passes of fixed summation order instead: the row sums of U on U's plan
+ * (with beta), then the row sums of U_s^T added onto y by the warp-chunk kernel that
+ * reads each value through its position in U (a transposed index built once here, on
+ * the host: rows of U_s^T list their entries by increasing position in U).  Results
+ * are deterministic.
  * spmv_set_values replaces U's values; spmv_apply (vector types as for
  * spmv_apply, except FP32 storage with an FP64 y), spmv_get_info, spmv_set_plan
  * (for the U pass), spmv_set_accumulator and spmv_destroy accept the handle;

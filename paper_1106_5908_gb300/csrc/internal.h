@@ -133,6 +133,12 @@ cudaError_t launch_rowvec(const KParams &p, const int32_t n_rows, int vk, int xk
 
 // out[k] = val[perm[k]] for k < nnz (values of kind vk: FP64 or FP32).
 cudaError_t launch_permute(const void *val, const int32_t *perm, void *out, int64_t nnz, int vk, cudaStream_t s);
+// The full CRS of a symmetric matrix from its upper triangle (rp, col) and the
+// transposed strictly upper part (rowS, colS, permS); mapF: position of each entry's
+// value among U's.
+cudaError_t launch_expand_sym(int32_t n, const int32_t *rp, const int32_t *col, const int32_t *rowS,
+                              const int32_t *colS, const int32_t *permS, int32_t *rpF, int32_t *colF, int32_t *mapF,
+                              cudaStream_t s);
 // Device-side CRS check; sets *bad to 1 on any violation.
 cudaError_t launch_validate(int32_t n_rows, int32_t n_cols, int64_t nnz, const int32_t *rp, const int32_t *col,
                             int32_t *bad, cudaStream_t s);

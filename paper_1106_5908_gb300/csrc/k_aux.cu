@@ -160,6 +160,44 @@ cudaError_t launch_permute(const void *val, const int32_t *perm, void *out, int6
     return cudaGetLastError();
 }
 
+// Symmetric CRS expanded: row i = row i of the transposed strictly upper part (rowS,
+// colS: columns below i, ascending; permS: positions in U's values), then row i of U.
+// A warp per row.
+__global__ void __launch_bounds__(256) k_expand_sym(int32_t n, const int32_t *__restrict__ rp,
+                                                    const int32_t *__restrict__ col, const int32_t *__restrict__ rowS,
+                                                    const int32_t *__restrict__ colS,
+                                                    const int32_t *__restrict__ permS, int32_t *__restrict__ rpF,
+                                                    int32_t *__restrict__ colF, int32_t *__restrict__ mapF) {
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * 8;
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5); i <= n; i += stride) {
+        const int32_t u0 = rp[i], s0 = rowS[i];
+        if (lane == 0) rpF[i] = u0 + s0;
+        if (i == n) break;
+        const int32_t u1 = rp[i + 1], s1 = rowS[i + 1];
+        for (int32_t k = s0 + lane; k < s1; k += 32) {
+            colF[u0 + k] = colS[k];
+            mapF[u0 + k] = permS[k];
+        }
+        for (int32_t k = u0 + lane; k < u1; k += 32) {
+            colF[s1 + k] = col[k];
+            mapF[s1 + k] = k;
+        }
+    }
+}
+
+cudaError_t launch_expand_sym(int32_t n, const int32_t *rp, const int32_t *col, const int32_t *rowS,
+                              const int32_t *colS, const int32_t *permS, int32_t *rpF, int32_t *colF, int32_t *mapF,
+                              cudaStream_t s) {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t want = (static_cast<int64_t>(n) + 8) / 8;
+    k_expand_sym<<<static_cast<int>(want < 16LL * sms ? want : 16LL * sms), 256, 0, s>>>(n, rp, col, rowS, colS, permS,
+                                                                                        rpF, colF, mapF);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_gather(const double *x, const int32_t *map, double *halo, int64_t n,
                           cudaStream_t s) {
     if (n <= 0) return cudaSuccess;

@@ -119,3 +119,35 @@ def test_symmetric_unsupported_calls():
     assert _abi.spmv_batched_create(ctypes.byref(b), 1, arr) == _abi.SPMV_ERR_UNSUPPORTED
     st = np.zeros(4)
     assert _abi.spmv_cg(h, p(v), p(v), 1e-10, 10, st.ctypes.data_as(ctypes.c_void_p), None) == _abi.SPMV_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("n", [1, 33, 3000, 20000])
+def test_expanded_and_two_pass_products_agree(n, dtype):
+    """The product on the expanded matrix (the default) and in two passes (a plan of
+    the caller's) against the oracle, before and after new values.  FP32 storage with
+    an FP64 result or the FP64 accumulator is refused, as on the two passes."""
+    from paper_1106_5908_gb300 import _abi
+    ft, tol = (np.float64, 1e-13) if dtype == "f64" else (np.float32, 1e-6)
+    U = W.random_symmetric_upper(n, seed=n + 7, max_len=9)
+    x = W.uniform(n, 3).astype(ft)
+    M, two = (sym(U, dtype=torch.float64 if dtype == "f64" else torch.float32) for _ in range(2))
+    two.set_plan(4, 9)
+    for seed in (None, 21, 22):
+        val = U.val.astype(ft) if seed is None else W.uniform(U.nnz, seed).astype(ft)
+        if seed is not None:
+            M.set_values(dev(val))
+            two.set_values(dev(val))
+        ref, bound = oracle.spmv_sym(U.row_ptr, U.col_idx, val.astype(np.float64), x.astype(np.float64),
+                                     with_bound=True)
+        for rep in range(3):  # new values are expanded by the second apply on them
+            for A in (M, two):
+                assert_within(host(A.apply(dev(x))), ref, bound, tol, f"{n} {seed} {rep}")
+    if dtype == "f32" and n > 1:
+        y = torch.zeros(n, dtype=torch.float64, device="cuda")
+        xd = dev(x)
+        assert _abi.spmv_apply(M.handle, 1.0, xd.data_ptr(), _abi.SPMV_F32, 0.0, y.data_ptr(), _abi.SPMV_F64,
+                               None) == _abi.SPMV_ERR_UNSUPPORTED
+        M.set_accumulator("f64")
+        assert _abi.spmv_apply(M.handle, 1.0, xd.data_ptr(), _abi.SPMV_F32, 0.0, y.data_ptr(), _abi.SPMV_F32,
+                               None) == _abi.SPMV_ERR_UNSUPPORTED
