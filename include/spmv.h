@@ -330,8 +330,9 @@ spmv_status spmv_transpose_noalloc(int32_t n_rows, int32_t n_cols, int64_t nnz,
 /* Group count matrix handles (all FP64 or all FP32 storage) into one batch whose
  * apply is a single persistent kernel launch over the warp chunks of every
  * matrix (the slot-major chunk kernel on a concatenated slot-major copy of the
- * members, one per group of members tuned alike), captured once into a CUDA
- * graph and replayed.  spmv_batched_get_member_plan reports each member's
+ * members, one per group of members tuned alike; large grid stencils on diagonal
+ * row slices, a second kernel of the graph), captured once into a CUDA graph and
+ * replayed.  spmv_batched_get_member_plan reports each member's
  * entries per lane.
  * The batch holds its own copy of the values: after spmv_set_values on a member,
  * the next spmv_batched_apply lays that member's values out again (on stream,
@@ -352,7 +353,8 @@ spmv_status spmv_batched_apply(spmv_batch_handle b, double alpha, const void *co
  * persistent grid at launch). */
 spmv_status spmv_batched_get_info(spmv_batch_handle b, int32_t *plan);
 
-/* The entries per lane each member runs with (HOST array of count int32).  The
+/* The entries per lane each member runs with (HOST array of count int32), 0 for a
+ * member on diagonal row slices (grid stencils of at least 32,768 rows).  The
  * batch tunes its members apart from their own row-length histograms (mean row
  * length below 4 entries: 7 per lane, else 9; a single matrix switches at 8,
  * but in a batch a separate group for members of 4-8 entries per row measured

@@ -510,6 +510,14 @@ struct spmv_batch {
     std::vector<int32_t> slot_cnt;  // chunks of each member (mixed batches)
     SlotTable slots9;
     int32_t *d_scmat9 = nullptr;
+    // members on diagonal row slices (member_E 0): the slices in launch order, the
+    // members' tables (structure from the handles' copies, values in d_dvals, member
+    // m's from byte dval_off[m])
+    int2 *d_dlist = nullptr;
+    SellMember *d_dmembers = nullptr;
+    char *d_dvals = nullptr;
+    std::vector<int64_t> dval_off;
+    int32_t n_dlist = 0;
 };
 
 namespace {
@@ -592,6 +600,8 @@ constexpr int32_t kDiagMinSize = 16384;
 // member at E = 9 (FP32 storage: 0.660 against 0.631 ms); the whole batch at
 // E = 7: 0.90 ms.  Members with shorter rows still get a group of their own.
 constexpr double kBatchSlotMeanE9 = 4.0;
+// Members of at least this many rows whose slices are diagonal run on them instead.
+constexpr int32_t kBatchDiagMinSize = 32768;
 
 void autotune(spmv_matrix *h) {
     const double mean = h->n_rows ? static_cast<double>(h->nnz) / h->n_rows : 0.0;
@@ -1439,6 +1449,61 @@ static spmv_status apply_sym(spmv_matrix *h, double alpha, const void *x, int xk
     return ops.launch(wp, ct->n, s) == cudaSuccess ? SPMV_OK : SPMV_ERR_CUDA;
 }
 
+// Member m's values laid out again in the batch's own slices, on s.
+static bool batch_diag_values(spmv_batch *b, int32_t m, cudaStream_t s) {
+    spmv_matrix *h = b->mats[m];
+    const SellTable &t = h->sells.at(kSellSigma);
+    if (launch_sell_relayout(t.d, t.srows, t.n, h->d_rp, h->vk, h->d_val, nullptr, b->d_dvals + b->dval_off[m], nullptr,
+                             s) != cudaSuccess)
+        return false;
+    b->vals_ver[m] = h->values_version;
+    return true;
+}
+
+// The batch's members on diagonal slices (member_E 0): large grid stencils, whose
+// chunks spend more on their rows than on their entries (32 5-point members of 110,000
+// rows on average: 46 against 59 us).
+// False when something failed; members whose slices are not diagonal stay with the
+// chunks.
+static bool batch_diagonals(spmv_batch *b) {
+    const int32_t count = b->count;
+    b->vals_ver.assign(static_cast<size_t>(count), 0);
+    b->dval_off.assign(static_cast<size_t>(count), 0);
+    const size_t vb = b->vk == kF64 ? 8 : 4;
+    std::vector<SellMember> members;
+    std::vector<int2> list;
+    std::vector<int32_t> which;
+    int64_t bytes = 0;
+    for (int32_t m = 0; m < count; ++m) {
+        spmv_matrix *h = b->mats[m];
+        if (h->col_diag < kDiagMinRows || h->sell_pad > kSellMaxPadding || h->n_rows < kBatchDiagMinSize ||
+            h->max_row > (b->vk == kF64 ? kSellLongRow : kFRMaxRun))
+            continue;
+        const SellTable *t = get_sell(h, kSellSigma, nullptr, false, false);
+        if (!t || !t->diagonal || t->n_long > 0) continue;
+        b->member_E[m] = 0;
+        b->dval_off[m] = bytes;
+        for (int32_t k = 0; k < t->n; ++k) list.push_back(make_int2(static_cast<int>(members.size()), k));
+        members.push_back(SellMember{t->dorder, t->srows, t->diag, nullptr, t->cols, m});
+        which.push_back(m);
+        bytes += (t->slot_rows * kSellC * static_cast<int64_t>(vb) + 255) / 256 * 256;
+    }
+    if (members.empty()) return true;
+    if (cudaMalloc(&b->d_dvals, static_cast<size_t>(bytes)) != cudaSuccess) {
+        b->d_dvals = nullptr;
+        return false;
+    }
+    for (size_t i = 0; i < members.size(); ++i) {
+        members[i].vals = b->d_dvals + b->dval_off[which[i]];
+        if (!batch_diag_values(b, which[i], nullptr)) return false;
+    }
+    b->n_dlist = static_cast<int32_t>(list.size());
+    return dmalloc(&b->d_dlist, list.size()) == cudaSuccess && dmalloc(&b->d_dmembers, members.size()) == cudaSuccess &&
+           cudaMemcpy(b->d_dlist, list.data(), sizeof(int2) * list.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
+           cudaMemcpy(b->d_dmembers, members.data(), sizeof(SellMember) * members.size(), cudaMemcpyHostToDevice) ==
+               cudaSuccess;
+}
+
 extern "C" {
 
 const char *spmv_status_string(spmv_status s) {
@@ -2194,6 +2259,15 @@ spmv_status spmv_batched_create(spmv_batch_handle *out, int32_t count, const spm
         (b->member_E[m] == 7 ? any7 : any9) = true;
     }
     SlotOps sops;
+    if (slot_ops_batched(vk, acc, any7 ? 7 : 9, &sops) && !batch_diagonals(b)) {
+        spmv_batched_destroy(b);
+        return SPMV_ERR_ALLOC;
+    }
+    any7 = any9 = false;
+    for (int32_t m = 0; m < count; ++m) {
+        any7 = any7 || b->member_E[m] == 7;
+        any9 = any9 || b->member_E[m] == 9;
+    }
     if (any7 && any9 && slot_ops_batched(vk, acc, 7, &sops) && slot_ops_batched(vk, acc, 9, &sops)) {
         // two groups, one copy each, one launch over both
         b->mixed = true;
@@ -2201,7 +2275,6 @@ spmv_status spmv_batched_create(spmv_batch_handle *out, int32_t count, const spm
         b->E = 7;
         b->slot_off.assign(static_cast<size_t>(count) + 1, 0);
         b->slot_cnt.assign(static_cast<size_t>(count), 0);
-        b->vals_ver.assign(static_cast<size_t>(count), 0);
         const size_t vb = (vk == kF64) ? 8 : 4;
         bool ok = true;
         for (int g = 0; g < 2 && ok; ++g) {
@@ -2260,12 +2333,12 @@ spmv_status spmv_batched_create(spmv_batch_handle *out, int32_t count, const spm
         b->E = ES;
         b->use_slots = true;
         b->slot_off.assign(static_cast<size_t>(count) + 1, 0);
-        b->vals_ver.assign(static_cast<size_t>(count), 0);
         std::vector<ChunkDesc> d;
         std::vector<uint32_t> lm;
         std::vector<int32_t> cm;
         for (int32_t m = 0; m < count; ++m) {
             b->slot_off[m] = static_cast<int32_t>(d.size());
+            if (b->member_E[m] == 0) continue;  // on diagonal slices
             make_slot_chunks(mats[m]->h_rp.data(), mats[m]->n_rows, ES, d, lm, &b->slots.n_long, &b->slots.n_empty);
             cm.resize(d.size(), m);
         }
@@ -2285,10 +2358,11 @@ spmv_status spmv_batched_create(spmv_batch_handle *out, int32_t count, const spm
                                       cudaSuccess);
         for (int32_t m = 0; ok && m < count; ++m) {
             const int64_t off = b->slot_off[m], nch = b->slot_off[m + 1] - off;
+            b->vals_ver[m] = mats[m]->values_version;
+            if (nch == 0) continue;
             ok = launch_slot_relayout(b->slots.d + off, ES, nch * 32 * ES, vk, mats[m]->d_val, mats[m]->d_col,
                                       static_cast<char *>(b->slots.vals) + off * 32 * ES * vb,
                                       b->slots.cols + off * 32 * ES, nullptr) == cudaSuccess;
-            b->vals_ver[m] = mats[m]->values_version;
         }
         ok = ok && cudaDeviceSynchronize() == cudaSuccess;
         b->slots.vals_valid = true;
@@ -2348,6 +2422,9 @@ void spmv_batched_destroy(spmv_batch_handle b) {
     free_slots(b->slots9);
     cudaFree(b->d_scmat);
     cudaFree(b->d_scmat9);
+    cudaFree(b->d_dlist);
+    cudaFree(b->d_dmembers);
+    cudaFree(b->d_dvals);
     cudaFree(b->d_mats);
     cudaFree(b->d_err);
     delete b;
@@ -2377,11 +2454,15 @@ spmv_status spmv_batched_apply(spmv_batch_handle b, double alpha, const void *co
     }
     const int acc = (b->vk == kF32) ? kAccFF : kAccF64;
     if (b->use_slots) {
-        if (b->slots.n == 0 && b->slots9.n == 0) return SPMV_OK;
+        if (b->slots.n == 0 && b->slots9.n == 0 && b->n_dlist == 0) return SPMV_OK;
         // members given new values since the copy: lay their values out again
         const size_t vb = (b->vk == kF64) ? 8 : 4;
         for (int32_t m = 0; m < b->count; ++m)
             if (b->mats[m]->values_version != b->vals_ver[m]) {
+                if (b->member_E[m] == 0) {
+                    if (!batch_diag_values(b, m, s)) return SPMV_ERR_CUDA;
+                    continue;
+                }
                 const int EG = b->mixed ? b->member_E[m] : b->E;
                 const SlotTable &t = (b->mixed && EG == 9) ? b->slots9 : b->slots;
                 const int64_t off = b->slot_off[m];
@@ -2415,12 +2496,25 @@ spmv_status spmv_batched_apply(spmv_batch_handle b, double alpha, const void *co
                 p9.cmat = b->d_scmat9;
                 p9.n_chunks = b->slots9.n;
             }
-            cudaStream_t cap;
+            // the members on diagonal slices as a second branch of the graph: it fills
+            // the SMs that the chunks' last warps leave idle
+            cudaStream_t cap, side = nullptr;
+            cudaEvent_t join = nullptr;
+            const bool fork = b->n_dlist > 0;
             CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
-            cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+            cudaError_t e = cudaSuccess;
+            if (fork) {
+                e = cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking);
+                if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
+            }
+            if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
             if (e == cudaSuccess) {
                 cudaError_t le = cudaSuccess;
-                if (b->mixed) {
+                if (fork) {
+                    le = cudaEventRecord(join, cap);
+                    if (le == cudaSuccess) le = cudaStreamWaitEvent(side, join, 0);
+                }
+                if (le == cudaSuccess && b->mixed) {
                     // the two groups as two kernel nodes of the one graph
                     SlotOps s7, s9;
                     if (!slot_ops_batched(b->vk, acc, 7, &s7) || !slot_ops_batched(b->vk, acc, 9, &s9)) {
@@ -2429,14 +2523,24 @@ spmv_status spmv_batched_apply(spmv_batch_handle b, double alpha, const void *co
                         le = s7.launch(p, cap);
                         if (le == cudaSuccess) le = s9.launch(p9, cap);
                     }
-                } else {
+                } else if (le == cudaSuccess) {
                     le = sops.launch(p, cap);
+                }
+                if (le == cudaSuccess && fork)
+                    le = launch_sell_diag_batch(SellBatchParams{b->d_dlist, b->d_dmembers, b->d_mats, b->n_dlist, alpha,
+                                                                beta}, b->vk, side);
+                if (fork) {  // join, also after an error: the capture must end on `cap`
+                    if (le == cudaSuccess) le = cudaEventRecord(join, side);
+                    const cudaError_t we = cudaStreamWaitEvent(cap, join, 0);
+                    if (le == cudaSuccess) le = we;
                 }
                 e = cudaStreamEndCapture(cap, &b->graph);
                 if (le != cudaSuccess) e = le;
             }
             if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
             cudaStreamDestroy(cap);
+            if (side) cudaStreamDestroy(side);
+            if (join) cudaEventDestroy(join);
             if (e != cudaSuccess) return SPMV_ERR_CUDA;
             b->graph_valid = true;
             b->cur_alpha = alpha;
@@ -2492,7 +2596,7 @@ spmv_status spmv_batched_get_info(spmv_batch_handle b, int32_t *plan) {
 spmv_status spmv_batched_get_member_plan(spmv_batch_handle b, int32_t *entries_per_lane) {
     if (!b || !entries_per_lane) return SPMV_ERR_INVALID_ARG;
     for (int32_t m = 0; m < b->count; ++m)
-        entries_per_lane[m] = b->use_slots ? (b->mixed ? b->member_E[m] : b->E) : b->E;
+        entries_per_lane[m] = b->use_slots ? (b->mixed || b->member_E[m] == 0 ? b->member_E[m] : b->E) : b->E;
     return SPMV_OK;
 }
 

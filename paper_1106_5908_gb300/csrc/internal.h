@@ -57,6 +57,11 @@ bool slot_ops_batched(int vk, int acc, int E, SlotOps *ops);
 cudaError_t launch_slot_relayout(const void *chunks, int E, int64_t n_slots, int vk, const void *val,
                                  const int32_t *col, void *vals_out, int32_t *cols_out, cudaStream_t s);
 
+struct SellBatchParams;
+// The batched launch over members on diagonal slices: FP64, or FP32 storage with FP32
+// runs (rows of at most 11 entries).
+cudaError_t launch_sell_diag_batch(const SellBatchParams &p, int vk, cudaStream_t s);
+
 struct SellParams;
 // One compiled configuration of the sorted row-slice kernel (plan family 5):
 // (F64, F64, F64) with FP64 FMAs and (F32, F32, F32) with float-float sums.

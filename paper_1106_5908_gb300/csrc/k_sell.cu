@@ -43,6 +43,24 @@ cudaError_t launch_sell_mr(const SellParams &b, const double *X, double *Y, int6
     return cudaGetLastError();
 }
 
+template <typename VT, typename ACC>
+static cudaError_t diag_batch_as(const SellBatchParams &p, cudaStream_t s) {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sell_diag_batch<VT, ACC>, 256, 0) != cudaSuccess ||
+        per_sm <= 0)
+        return cudaErrorInvalidConfiguration;
+    const int64_t want = (2 * static_cast<int64_t>(p.n_list) + 7) / 8, lim = static_cast<int64_t>(per_sm) * sms;
+    k_sell_diag_batch<VT, ACC><<<static_cast<int>(want < lim ? want : lim), 256, 0, s>>>(p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sell_diag_batch(const SellBatchParams &p, int vk, cudaStream_t s) {
+    if (p.n_list <= 0) return cudaSuccess;
+    return vk == kF64 ? diag_batch_as<double, AccF64>(p, s) : diag_batch_as<float, AccFR>(p, s);
+}
+
 // How a pass of R right-hand sides runs: V per lane, L = ceil(R/V) lanes per row, G =
 // 32/L rows at a time.  The FP64 pipe needs V warp FMAs (17 cycles each) per G rows
 // and slot; with scattered columns L1 also looks up a line per row for each of the

@@ -470,6 +470,77 @@ __device__ __forceinline__ void sell_diag_walk(const SellParams &p, double &dsum
     }
 }
 
+// The same over the slices of many matrices in one launch (the batch): half slice i
+// is half i & 1 of entry i / 2 of `list`: x = the member, y = the slice in the
+// member's launch order.  The list entry, descriptor and rows of the half slices
+// that follow are loaded ahead, one step of the chain per turn.
+struct SellMember {
+    const int4 *dorder;
+    const int32_t *srows;
+    const int4 *diag;
+    const void *vals;
+    const int32_t *cols;
+    int32_t mat;  // the member's place in the matrix table
+};
+struct SellBatchParams {
+    const int2 *list;
+    const SellMember *members;
+    const MatRef *mats;
+    int32_t n_list;
+    double alpha, beta;
+};
+
+template <typename VT, typename ACC>
+__global__ void __launch_bounds__(256, sizeof(VT) == 8 ? 4 : 5) k_sell_diag_batch(const SellBatchParams p) {
+    constexpr int C = kSellC;
+    const int lane = threadIdx.x & 31;
+    const int n = 2 * p.n_list, nw = gridDim.x * 8;
+    const uint64_t pol = l2_evict_first_policy();
+    const double alpha = p.alpha, beta = p.beta;
+    const int emode = epi_mode(alpha, beta);
+    int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= n) return;
+    auto entry_of = [&](int k) { return __ldg(p.list + (k < n ? k >> 1 : p.n_list - 1)); };
+    auto desc_of = [&](const int2 &e) { return __ldg(p.members[e.x].dorder + e.y); };
+    auto row_of = [&](const int2 &e, const int4 &d, int k) {
+        return __ldg(p.members[e.x].srows + static_cast<int64_t>(d.z) * C + (k & 1) * 32 + lane);
+    };
+    int2 e0 = entry_of(i), e1 = entry_of(i + nw), e2 = entry_of(i + 2 * nw);
+    int4 d0 = desc_of(e0), d1 = desc_of(e1);
+    int r = row_of(e0, d0, i);
+    for (; i < n; i += nw) {
+        const int2 e3 = entry_of(i + 3 * nw);
+        const int4 d2 = desc_of(e2);
+        const int rn = row_of(e1, d1, i + nw);
+        const SellMember &t = p.members[e0.x];
+        const MatRef m = p.mats[t.mat];
+        const VT *__restrict__ x = static_cast<const VT *>(m.x);
+        VT *__restrict__ y = static_cast<VT *>(m.y);
+        const int64_t base = static_cast<int64_t>(d0.x) * C + (i & 1) * 32 + lane;
+        ACC acc;
+        acc.zero();
+        const SellVals<VT, false> sv{static_cast<const VT *>(t.vals) + base, nullptr};
+        if (d0.w >= 0)
+            sell_diag_row<true>(acc, d0.y, sv, static_cast<const int32_t *>(nullptr), t.diag + d0.w, r, x, pol);
+        else
+            sell_diag_row<false>(acc, d0.y, sv, t.cols + base, static_cast<const int4 *>(nullptr), r, x, pol);
+        if (r >= 0) {
+            if constexpr (std::is_same<ACC, AccF64>::value) {
+                y[r] = epi_apply(acc.get(), y + r, alpha, beta, emode);
+            } else {
+                const double old = emode >= kEpiAdd ? widen(y[r]) : 0.0;
+                sell_store<VT>(m, x, y, r, acc, alpha, beta, emode == kEpiPlain, old);
+            }
+        }
+        e0 = e1;
+        e1 = e2;
+        e2 = e3;
+        d0 = d1;
+        d1 = d2;
+        r = rn;
+    }
+}
+
 // CTAs per SM the registers must allow.  Rows of up to 8 entries (SHORT: one
 // block per half slice, so the warps are latency-bound) take one more: 160^3
 // Laplacian FP64 55.3 against 60.3 us, FP32 28.9 against 30.2; longer rows lose

@@ -82,8 +82,15 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
     const uint64_t pol = l2_evict_first_policy();
     const VT *__restrict__ vals = static_cast<const VT *>(p.vals);
     const double alpha = p.alpha, beta = p.beta;
-    auto mat_of = [&](int cc) -> MatRef {
-        if constexpr (BATCHED) return p.mats[p.cmat[cc]];
+    // BATCHED: the member of chunk cc.  It is loaded a turn before the member's
+    // pointers are, so that no address waits for it (32 Hamiltonian-like members,
+    // 38 M entries: 137 -> 126 us).
+    auto member_of = [&](int cc) -> int {
+        if constexpr (BATCHED) return __ldg(p.cmat + (cc < n ? cc : n - 1));
+        else return 0;
+    };
+    auto mat_of = [&](int mi) -> MatRef {
+        if constexpr (BATCHED) return p.mats[mi];
         else return p.m;
     };
     const bool plain = (alpha == 1.0 && beta == 0.0);
@@ -101,8 +108,8 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = ld_stream(b + e * 32, pol);
     };
-    auto xptr_of = [&](int cc) -> const XT * {
-        if constexpr (BATCHED) return static_cast<const XT *>(p.mats[__ldg(p.cmat + cc)].x);
+    auto xptr_of = [&](int mi) -> const XT * {
+        if constexpr (BATCHED) return static_cast<const XT *>(p.mats[mi].x);
         else return static_cast<const XT *>(p.m.x);
     };
     auto gather = [&](const XT *__restrict__ x, const ChunkDesc &d, const int32_t (&cl)[E], XT (&xv)[E]) {
@@ -119,12 +126,15 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
     // descriptor, row starts, column indices
     ChunkDesc dc = load_desc(c);
     uint32_t mc = __ldg(p.lmask + static_cast<int64_t>(c) * 32 + lane);
+    int mic = member_of(c), min1 = member_of(c + nwarps), min2 = member_of(c + 2 * nwarps);
+    YT *yc = nullptr;
+    if constexpr (BATCHED) yc = static_cast<YT *>(p.mats[mic].y);
     XT xc[E];
     VT vc[E];
     {
         int32_t cl[E];
         load_cols(c, cl);
-        gather(xptr_of(c), dc, cl, xc);
+        gather(xptr_of(mic), dc, cl, xc);
         load_vals(c, vc);
     }
     ChunkDesc dn{};
@@ -134,7 +144,7 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
 #pragma unroll
     for (int e = 0; e < E; ++e) cn[e] = 0;
     if (c + nwarps < n) {
-        xpn = xptr_of(c + nwarps);
+        xpn = xptr_of(min1);
         dn = load_desc(c + nwarps);
         mn = __ldg(p.lmask + static_cast<int64_t>(c + nwarps) * 32 + lane);
         load_cols(c + nwarps, cn);
@@ -160,7 +170,7 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
         const XT *xp2 = nullptr;
         int32_t c2l[E];
         if (c2 < n) {
-            xp2 = xptr_of(c2);
+            xp2 = xptr_of(min2);
             d2 = load_desc(c2);
             m2 = __ldg(p.lmask + static_cast<int64_t>(c2) * 32 + lane);
             load_cols(c2, c2l);
@@ -168,10 +178,13 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
 #pragma unroll
             for (int e = 0; e < E; ++e) c2l[e] = 0;
         }
+        const int min3 = member_of(c2 + nwarps);
+        YT *yn = nullptr;  // BATCHED: the next chunk's y
+        if constexpr (BATCHED) yn = static_cast<YT *>(p.mats[min1].y);
         // ---- chunk c ---------------------------------------------------------
-        const MatRef m = mat_of(c);
+        const MatRef m = mat_of(mic);
         const XT *__restrict__ x = static_cast<const XT *>(m.x);
-        YT *__restrict__ y = static_cast<YT *>(m.y);
+        YT *__restrict__ y = BATCHED ? yc : static_cast<YT *>(m.y);
         const int r0 = dc.r0;
         const int r1 = dc.r1f & kChunkRowMask;
         if (dc.r1f & kChunkLong) {
@@ -199,8 +212,8 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
                 epi.store(y, srow, r1 - r0, alpha, beta, emode, lane);
             } else {
                 for (int q = lane; q < r1 - r0; q += 32) {
-                    if constexpr (std::is_same<ACC, AccF64>::value && !BATCHED) {
-                        const int64_t row = m.rmap ? __ldg(m.rmap + r0 + q) : r0 + q;
+                    if constexpr (std::is_same<ACC, AccF64>::value) {
+                        const int64_t row = (!BATCHED && m.rmap) ? __ldg(m.rmap + r0 + q) : r0 + q;
                         y[row] = narrow<YT>(epi_apply(srow[q].get(), y + row, alpha, beta, emode));
                     } else {
                         store_acc<VT, false>(m, x, y, r0 + q, srow[q], alpha, beta, plain);
@@ -214,6 +227,10 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
         dn = d2;
         mn = m2;
         xpn = xp2;
+        yc = yn;
+        mic = min1;
+        min1 = min2;
+        min2 = min3;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             xc[e] = xn[e];

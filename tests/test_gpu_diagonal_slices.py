@@ -116,3 +116,30 @@ def test_tuner_takes_grid_stencils():
     M = Matrix.from_csr(np.arange(0, 5 * n + 1, 5, dtype=np.int32), col.reshape(-1).astype(np.int32),
                         rng.standard_normal(5 * n), n)
     assert M.info()["family"] == 4
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("others", [0, 3])
+def test_batch_members_on_diagonal_slices(others, dtype):
+    """Large grid stencils of a batch run on their diagonal slices beside (or without)
+    chunk members, follow new values and keep their own copy of them."""
+    from paper_1106_5908_gb300 import Batch, Matrix
+    ft, tol = (np.float64, 1e-13) if dtype == "f64" else (np.float32, 1e-6)
+    As = [W.laplace2d(200, 190), W.laplace3d(33), W.laplace2d(181)]
+    As += [W.hamiltonian_like(5000, seed=3), W.laplace2d(60), W.random_csr(700, 700, seed=4, max_len=4)][:others]
+    mats = [Matrix.from_csr(A.row_ptr, A.col_idx, A.val.astype(ft), A.n_cols) for A in As]
+    B = Batch(mats)
+    assert B.info()["member_E"][:3] == [0, 0, 9]  # the last has 32,761 rows
+    xs = [W.uniform(A.n_cols, 50 + m).astype(ft) for m, A in enumerate(As)]
+    y0 = [W.uniform(A.n_rows, 80 + m).astype(ft) for m, A in enumerate(As)]
+    vals = [A.val.astype(ft) for A in As]
+    for rep, (alpha, beta) in enumerate(((1.0, 0.0), (1.0, 0.0), (-1.5, 0.5))):
+        if rep:
+            vals[0] = W.uniform(As[0].nnz, 90 + rep).astype(ft)
+            mats[0].set_values(dev(vals[0]))
+        xd, yd = [dev(x) for x in xs], [dev(y) for y in y0]
+        B.apply(xd, yd, alpha, beta)
+        for m, A in enumerate(As):
+            ref, bound = oracle.spmv(A.row_ptr, A.col_idx, vals[m].astype(np.float64), xs[m].astype(np.float64), alpha,
+                                     beta, y0[m].astype(np.float64), with_bound=True)
+            assert_within(host(yd[m]), ref, bound, tol, f"member {m} rep {rep}")
