@@ -1569,7 +1569,14 @@ spmv_status spmv_set_values(spmv_handle h, const void *val, spmv_dtype t, void *
     } else {
         CK(launch_convert(val, t, h->d_val, h->vk, h->nnz, s));
     }
-    if (h->mirror32) CK(launch_convert(val, t, h->mirror32->d_val, kF32, h->nnz, s));
+    if (h->mirror32) {
+        CK(launch_convert(val, t, h->mirror32->d_val, kF32, h->nnz, s));
+        for (auto &kv : h->mirror32->slots) kv.second.vals_valid = false;
+        for (auto &kv : h->mirror32->sells) kv.second.vals_valid = false;
+    }
+    // captured CG iterations read the copies laid out from the old values: the next
+    // solve runs its first iterations plainly, which lays them out again
+    h->cg.cg64_key = h->cg.inner32_key = -1;
     h->valT_valid = false;
     h->valT_requested = false;
     ++h->values_version;

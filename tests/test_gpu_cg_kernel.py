@@ -90,3 +90,35 @@ def test_zero_right_hand_side_and_new_values():
     x2, st = cg(M, dev(b))
     assert st["converged"]
     assert np.linalg.norm(2.0 * host(x2) - host(x1)) <= 1e-9 * np.linalg.norm(host(x1))
+
+
+@pytest.mark.parametrize("kind", ["grid", "scattered"])
+def test_solvers_follow_new_values(kind):
+    """Both solvers after spmv_set_values, on the one-kernel path and (scattered
+    columns) on the captured iterations, into the same x as before."""
+    from paper_1106_5908_gb300 import Matrix, _abi
+    if kind == "grid":
+        A = W.laplace2d(80)
+        val2 = A.val * 3.0
+    else:
+        H = W.hamiltonian_like(6000, seed=21)
+        rows = np.repeat(np.arange(H.n_rows), np.diff(H.row_ptr.astype(np.int64)))
+        off = rows != H.col_idx
+        rowabs = np.bincount(rows[off], weights=np.abs(H.val[off]), minlength=H.n_rows)
+        v = H.val.copy()
+        v[~off] = rowabs[rows[~off]] + 1.0  # diagonally dominant: SPD
+        A = W.CRS(H.row_ptr, H.col_idx, v, H.n_cols)
+        val2 = A.val.copy()
+        val2[~off] += 40.0  # another matrix, not a multiple of the first
+    M = Matrix.from_csr(A.row_ptr, A.col_idx, A.val, A.n_cols)
+    b, x = dev(W.uniform(A.n_rows, 5)), torch.empty(A.n_rows, dtype=torch.float64, device="cuda")
+    st = np.zeros(4)
+    for val in (A.val, val2):
+        M.set_values(dev(val))
+        for solve in (lambda: _abi.spmv_cg(M.handle, b.data_ptr(), x.data_ptr(), 1e-12, 5000, st.ctypes.data, None),
+                      lambda: _abi.spmv_ir_cg(M.handle, b.data_ptr(), x.data_ptr(), 1e-12, 20, 1e-3, 500, st.ctypes.data,
+                                              None)):
+            torch.cuda.synchronize()
+            assert solve() == _abi.SPMV_OK
+            r = oracle.residual(A.row_ptr, A.col_idx, val, host(b), host(x))
+            assert np.linalg.norm(r) <= 2e-12 * np.linalg.norm(host(b)), (kind, st)
