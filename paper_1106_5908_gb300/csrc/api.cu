@@ -105,7 +105,7 @@ struct SlotTable {
 
 // Sorted row-slice copy of a matrix for plan family 5 (per window sigma).
 struct SellTable {
-    void *meta = nullptr;       // one allocation: the tables d .. diag below
+    void *meta = nullptr;       // one allocation: the tables d, srows, cstart, dtmp, dorder
     int2 *d = nullptr;          // per slice: first slot row and width (width < 0: long row)
     int32_t *srows = nullptr;   // kSellC rows per slice (-1: none)
     int32_t *cstart = nullptr;  // n_ctas + 1: first slice of each CTA of a launch
@@ -118,6 +118,7 @@ struct SellTable {
     bool vals_valid = false;
     // diagonal slices: descriptors with each slice's place in diag (in slice order
     // and in launch order), and the diagonals of the slot rows, padded to 4 per slice
+    // (behind cols)
     int4 *dtmp = nullptr, *dorder = nullptr;
     int4 *diag = nullptr;
     bool diagonal = false;      // enough slices are diagonal for k_sell_diag
@@ -731,19 +732,63 @@ SlotTable *get_slots(spmv_matrix *h, int E, cudaStream_t s, bool transposed = fa
     return &t;
 }
 
-// The tables of a row-slice copy (descriptors, rows, CTA ranges, places of the
-// diagonals) in one allocation and one copy on s.
+// The tables of a row-slice copy built on the device, in one allocation, when the
+// window is the default and no row is long; *done tells whether they were.  Waits for
+// s.  (The 2.1 M-row scattered matrix: first block product 12.6 -> 1.4 ms; first
+// training step on the 27-point 128^3 pattern 37 -> 5.3 ms.)
+bool build_sell(SellTable &t, const int32_t *d_rp, int32_t n_rows, int32_t sigma, bool *done, cudaStream_t s) {
+    static_assert(kSellBuildSigma == kSellSigma && kSellBuildMaxRow == kSellLongRow, "the device's tables");
+    *done = false;
+    if (sigma != kSellBuildSigma) return true;
+    const size_t n = static_cast<size_t>(t.n);
+    // dtmp, dorder, d, srows, cstart + counts, width, off, sums, flag
+    const size_t o_out = sizeof(int4) * n, o_d = 2 * o_out, o_sr = o_d + sizeof(int2) * n,
+                 o_ws = o_sr + 4 * n * kSellC, o_wd = o_ws + 4 * (static_cast<size_t>(t.n_ctas) + 3), o_off = o_wd + 4 * n,
+                 o_sum = o_off + 4 * (n + 1), o_flag = o_sum + 4 * static_cast<size_t>(scan_sums_len(t.n));
+    if (cudaMalloc(&t.meta, o_flag + 4) != cudaSuccess) {
+        t.meta = nullptr;
+        return false;
+    }
+    char *m = static_cast<char *>(t.meta);
+    t.dtmp = reinterpret_cast<int4 *>(m);
+    t.dorder = reinterpret_cast<int4 *>(m + o_out);
+    t.d = reinterpret_cast<int2 *>(m + o_d);
+    t.srows = reinterpret_cast<int32_t *>(m + o_sr);
+    t.cstart = reinterpret_cast<int32_t *>(m + o_ws);
+    int32_t *off = reinterpret_cast<int32_t *>(m + o_off);
+    uint32_t *flag = reinterpret_cast<uint32_t *>(m + o_flag);
+    uint32_t too_long = 0;
+    int32_t rows = 0;
+    if (cudaMemsetAsync(m + o_ws, 0, 4 * (static_cast<size_t>(t.n_ctas) + 3), s) != cudaSuccess ||
+        cudaMemsetAsync(flag, 0, 4, s) != cudaSuccess ||
+        launch_sell_build(d_rp, n_rows, t.n, t.n_ctas, t.srows, reinterpret_cast<int32_t *>(m + o_wd), off,
+                          reinterpret_cast<int32_t *>(m + o_sum), flag, t.d, t.dtmp, t.cstart, s) != cudaSuccess ||
+        cudaMemcpyAsync(&too_long, flag, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaMemcpyAsync(&rows, off + n, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return false;
+    if (too_long) {
+        cudaFree(t.meta);
+        t.meta = nullptr;
+        return true;
+    }
+    t.slot_rows = static_cast<int64_t>(rows) + kSellU;
+    *done = true;
+    return true;
+}
+
+// The tables of a row-slice copy from the host (descriptors, rows, CTA ranges, places
+// of the diagonals) in one allocation and one copy on s.
 bool upload_sell(SellTable &t, const std::vector<int2> &d, const std::vector<int32_t> &sr,
                  const std::vector<int32_t> &ws, cudaStream_t s) {
     std::vector<int4> order(d.size());
-    size_t packed = 2;  // a block of 8 slot rows reads two elements
+    int packed = 0;
     for (size_t i = 0; i < d.size(); ++i) {
-        order[i] = make_int4(d[i].x, d[i].y, static_cast<int>(i), static_cast<int>(packed - 2));
-        packed += d[i].y > 0 ? static_cast<size_t>(d[i].y + 3) / 4 : 0;
+        order[i] = make_int4(d[i].x, d[i].y, static_cast<int>(i), packed);
+        packed += d[i].y > 0 ? (d[i].y + 3) / 4 : 0;
     }
     const size_t o_order = 0, o_d = o_order + sizeof(int4) * order.size(), o_sr = o_d + sizeof(int2) * d.size(),
-                 o_ws = o_sr + 4 * sr.size(), host_end = o_ws + 4 * ws.size() + 8, o_out = (host_end + 15) / 16 * 16,
-                 o_diag = o_out + sizeof(int4) * order.size();
+                 o_ws = o_sr + 4 * sr.size(), host_end = o_ws + 4 * ws.size() + 8, o_out = (host_end + 15) / 16 * 16;
     std::vector<char> host(host_end, 0);  // the last two words: the marking's counts
     if (!d.empty()) {
         std::memcpy(host.data() + o_order, order.data(), sizeof(int4) * order.size());
@@ -751,7 +796,7 @@ bool upload_sell(SellTable &t, const std::vector<int2> &d, const std::vector<int
         std::memcpy(host.data() + o_sr, sr.data(), 4 * sr.size());
     }
     std::memcpy(host.data() + o_ws, ws.data(), 4 * ws.size());
-    if (cudaMalloc(&t.meta, o_diag + sizeof(int4) * packed) != cudaSuccess) {
+    if (cudaMalloc(&t.meta, o_out + sizeof(int4) * order.size()) != cudaSuccess) {
         t.meta = nullptr;
         return false;
     }
@@ -761,9 +806,7 @@ bool upload_sell(SellTable &t, const std::vector<int2> &d, const std::vector<int
     t.d = reinterpret_cast<int2 *>(m + o_d);
     t.srows = reinterpret_cast<int32_t *>(m + o_sr);
     t.cstart = reinterpret_cast<int32_t *>(m + o_ws);
-    t.diag = reinterpret_cast<int4 *>(m + o_diag);
-    return cudaMemcpyAsync(m, host.data(), host.size(), cudaMemcpyHostToDevice, s) == cudaSuccess &&
-           cudaMemsetAsync(t.diag, 0, sizeof(int4) * packed, s) == cudaSuccess;
+    return cudaMemcpyAsync(m, host.data(), host.size(), cudaMemcpyHostToDevice, s) == cudaSuccess;
 }
 
 // Marks the diagonal slices of a row-slice copy whose columns are laid out on s:
@@ -804,19 +847,31 @@ SellTable *get_sell(spmv_matrix *h, int32_t sigma, cudaStream_t s, bool transpos
     };
     auto it = tabs.find(sigma);
     if (it == tabs.end()) {
-        std::vector<int2> d;
-        std::vector<int32_t> sr;
         SellTable t;
-        if (!make_sell_slices(h_rp, nr, sigma, d, sr, &t.n_long, &t.slot_rows)) return nullptr;
-        t.n = static_cast<int32_t>(d.size());
         SellOps o;
         const int acc = (h->vk == kF32) ? kAccFF : kAccF64;
-        t.n_ctas = sell_ops(h->vk, h->vk, h->vk, acc, &o, transposed ? 0x7fffffff : h->max_row) ? o.ctas_for(t.n) : 0;
+        if (!sell_ops(h->vk, h->vk, h->vk, acc, &o, transposed ? 0x7fffffff : h->max_row)) return nullptr;
+        // on the device (slices of a window without long rows), else on the host
+        t.n = static_cast<int32_t>((static_cast<int64_t>(nr) + kSellC - 1) / kSellC);
+        t.n_ctas = o.ctas_for(t.n);
         if (t.n_ctas <= 0) return nullptr;
-        std::vector<int32_t> ws;
-        sell_ranges(d, h_rp, t.n_ctas, ws);
+        bool done = false;
+        bool ok = (!transposed && h->max_row > kSellLongRow) || build_sell(t, d_rp, nr, sigma, &done, s);
+        if (ok && !done) {
+            std::vector<int2> d;
+            std::vector<int32_t> sr, ws;
+            if (!make_sell_slices(h_rp, nr, sigma, d, sr, &t.n_long, &t.slot_rows)) return nullptr;
+            t.n = static_cast<int32_t>(d.size());
+            t.n_ctas = o.ctas_for(t.n);
+            sell_ranges(d, h_rp, t.n_ctas, ws);
+            ok = t.n_ctas > 0 && upload_sell(t, d, sr, ws, s);
+        }
+        // the diagonals (places up to slot_rows / 4 + n on either path) follow the columns
         const size_t nslots = static_cast<size_t>(t.slot_rows) * kSellC;
-        bool ok = upload_sell(t, d, sr, ws, s) && dmalloc(&t.cols, nslots + 4) == cudaSuccess;
+        const size_t ndiag = static_cast<size_t>(t.slot_rows) / 4 + static_cast<size_t>(t.n) + 2;
+        ok = ok && dmalloc(&t.cols, (nslots + 4) + 4 * ndiag) == cudaSuccess;
+        if (ok) t.diag = reinterpret_cast<int4 *>(t.cols + nslots + 4);
+        ok = ok && cudaMemsetAsync(t.diag, 0, sizeof(int4) * ndiag, s) == cudaSuccess;
         ok = ok && (!need_vals || alloc_vals(t));
         // the leading padding rows: column -1 (and value 0)
         ok = ok && cudaMemsetAsync(t.cols, 0xff, static_cast<size_t>(kSellU) * kSellC * 4, s) == cudaSuccess;

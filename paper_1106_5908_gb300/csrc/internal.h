@@ -97,6 +97,18 @@ cudaError_t launch_sell_relayout(const void *slices, const int32_t *srows, int32
                                  int vk, const void *val, const int32_t *col, void *vals_out, int32_t *cols_out,
                                  cudaStream_t s);
 
+// Exclusive scan of n counts into out[0..n]; sums: scan_sums_len(n) entries of scratch.
+cudaError_t launch_scan(const int32_t *in, int64_t n, int32_t *sums, int32_t *out, cudaStream_t s);
+int64_t scan_sums_len(int64_t n);
+// The row-slice tables of windows of kSellBuildSigma rows: slot rows counted from the
+// leading padding on (off: n_slices + 1 entries, off[n_slices] = the slot rows), rows,
+// descriptors, places of the diagonals and CTA ranges.  *too_long is set when a row
+// has more than kSellBuildMaxRow entries (the tables are then not usable).
+constexpr int32_t kSellBuildSigma = 4096;
+constexpr int32_t kSellBuildMaxRow = 128;
+cudaError_t launch_sell_build(const int32_t *rp, int32_t n_rows, int32_t n_slices, int32_t n_ctas, int32_t *srows,
+                              int32_t *width, int32_t *off, int32_t *sums, uint32_t *too_long, void *d, void *dtmp,
+                              int32_t *cstart, cudaStream_t s);
 // Finds the diagonal slices (in every slot row all 64 rows are stored and column -
 // row is one number): their diagonals into diag (int4 elements, from each slice's
 // place dtmp[s].w on), place -1 for the others, and all descriptors into dorder,

@@ -603,6 +603,11 @@ static cudaError_t scan_counts(const int32_t *in, int64_t n, int32_t *sums, int3
     return cudaGetLastError();
 }
 
+cudaError_t launch_scan(const int32_t *in, int64_t n, int32_t *sums, int32_t *out, cudaStream_t s) {
+    return scan_counts(in, n, sums, out, s);
+}
+int64_t scan_sums_len(int64_t n) { return (n + kScanChunk - 1) / kScanChunk + 1; }
+
 // Work layout of the transposed build (int32 entries): column counts
 // (n_cols + 1), the column scan's block sums, the radix histograms, their scan
 // (kRadixHistLen + 1) and its block sums.

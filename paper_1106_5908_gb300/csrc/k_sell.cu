@@ -111,6 +111,133 @@ cudaError_t launch_sell_rhs(const SellParams &b, const double *X, double *Y, int
     return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------
+// The row-slice tables on the device (windows of kSellBuildSigma rows, no row of more
+// than kSellBuildMaxRow entries), the same as the host builds for any window: one CTA
+// sorts a window's rows by length, longest first, ties in row order (a stable counting
+// sort: ranks of equal lengths from a match in each warp, warps and rounds of 256 rows
+// in order); the widths' exclusive scan gives the first slot rows.
+// ---------------------------------------------------------------------------
+constexpr int kBuildBins = kSellBuildMaxRow + 1;
+
+__global__ void __launch_bounds__(256) k_sell_sort(const int32_t *__restrict__ rp, int32_t n_rows,
+                                                   int32_t *__restrict__ srows, int32_t *__restrict__ width,
+                                                   uint32_t *__restrict__ too_long) {
+    constexpr int NW = 8;
+    __shared__ int32_t s_base[kBuildBins];      // next place of each length, longest first
+    __shared__ int32_t s_wc[NW][kBuildBins];    // a round's counts per warp, then its offsets
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int64_t r0 = static_cast<int64_t>(blockIdx.x) * kSellBuildSigma;
+    const int nr = static_cast<int>(min(static_cast<int64_t>(kSellBuildSigma), n_rows - r0));
+    // bin of a row: kSellBuildMaxRow - length (a longer row only sets the flag)
+    auto bin_of = [&](int i) {
+        const int32_t len = __ldg(rp + r0 + i + 1) - __ldg(rp + r0 + i);
+        return max(0, kSellBuildMaxRow - len);
+    };
+    for (int b = t; b < kBuildBins; b += 256) {
+        s_base[b] = 0;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) s_wc[q][b] = 0;
+    }
+    __syncthreads();
+    for (int i = t; i < nr; i += 256) {
+        atomicAdd(&s_base[bin_of(i)], 1);
+        if (__ldg(rp + r0 + i + 1) - __ldg(rp + r0 + i) > kSellBuildMaxRow) atomicOr(too_long, 1u);
+    }
+    __syncthreads();
+    if (w == 0) {  // exclusive scan of the bins
+        int32_t run = 0;
+        for (int b0 = 0; b0 < kBuildBins; b0 += 32) {
+            const int b = b0 + lane;
+            const int32_t v = b < kBuildBins ? s_base[b] : 0;
+            int32_t inc = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t u = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += u;
+            }
+            if (b < kBuildBins) s_base[b] = run + inc - v;
+            run += __shfl_sync(0xffffffffu, inc, 31);
+        }
+    }
+    __syncthreads();
+    for (int i0 = 0; i0 < nr; i0 += 256) {
+        const int i = i0 + t;
+        const bool ok = i < nr;
+        const int b = ok ? bin_of(i) : kBuildBins;
+        const unsigned peers = __match_any_sync(0xffffffffu, b);
+        const int rank = __popc(peers & ((1u << lane) - 1u));
+        if (ok && rank == 0) s_wc[w][b] = __popc(peers);
+        __syncthreads();
+        for (int q = t; q < kBuildBins; q += 256) {
+            int32_t run = s_base[q];
+#pragma unroll
+            for (int u = 0; u < NW; ++u) {
+                const int32_t c = s_wc[u][q];
+                s_wc[u][q] = run;
+                run += c;
+            }
+            s_base[q] = run;
+        }
+        __syncthreads();
+        if (ok) {
+            const int pos = s_wc[w][b] + rank;
+            srows[r0 + pos] = static_cast<int32_t>(r0 + i);
+            if (pos % kSellC == 0) width[(r0 + pos) / kSellC] = kSellBuildMaxRow - b;
+        }
+        __syncthreads();
+        for (int q = t; q < kBuildBins; q += 256)
+#pragma unroll
+            for (int u = 0; u < NW; ++u) s_wc[u][q] = 0;
+        __syncthreads();
+    }
+    // the last slice's missing rows
+    for (int i = nr + t; i < (nr + kSellC - 1) / kSellC * kSellC; i += 256) srows[r0 + i] = -1;
+}
+
+// Descriptors from the scanned widths (off[n_slices] = their sum); a slice's place
+// among the diagonals is off / 4 + slice, which leaves room for its (w + 3) / 4.  The
+// first n_ctas + 1 threads also cut the slices into ranges of equal work (w + 1 slot
+// rows per slice).
+__global__ void __launch_bounds__(256) k_sell_tables(const int32_t *__restrict__ width, const int32_t *__restrict__ off,
+                                                     int32_t n_slices, int32_t n_ctas, int2 *__restrict__ d,
+                                                     int4 *__restrict__ dtmp, int32_t *__restrict__ cstart) {
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    for (int64_t i = i0; i < n_slices; i += stride) {
+        const int32_t o = off[i], w = width[i];
+        d[i] = make_int2(o + kSellU, w);
+        dtmp[i] = make_int4(o + kSellU, w, static_cast<int>(i), o / 4 + static_cast<int>(i));
+    }
+    for (int64_t g = i0; g <= n_ctas; g += stride) {
+        if (g == n_ctas) {
+            cstart[g] = n_slices;
+            continue;
+        }
+        const int64_t target = (static_cast<int64_t>(off[n_slices]) + n_slices) * kSellC * g / n_ctas;
+        int32_t lo = 0, hi = n_slices;  // the first slice with as much work before it
+        while (lo < hi) {
+            const int32_t mid = lo + (hi - lo) / 2;
+            if ((static_cast<int64_t>(off[mid]) + mid) * kSellC < target) lo = mid + 1;
+            else hi = mid;
+        }
+        cstart[g] = lo;
+    }
+}
+
+cudaError_t launch_sell_build(const int32_t *rp, int32_t n_rows, int32_t n_slices, int32_t n_ctas, int32_t *srows,
+                              int32_t *width, int32_t *off, int32_t *sums, uint32_t *too_long, void *d, void *dtmp,
+                              int32_t *cstart, cudaStream_t s) {
+    static_assert(kSellBuildSigma % kSellC == 0, "windows hold whole slices");
+    k_sell_sort<<<(n_rows + kSellBuildSigma - 1) / kSellBuildSigma, 256, 0, s>>>(rp, n_rows, srows, width, too_long);
+    cudaError_t e = launch_scan(width, n_slices, sums, off, s);
+    if (e != cudaSuccess) return e;
+    const int want = (std::max(n_slices, n_ctas + 1) + 255) / 256;
+    k_sell_tables<<<std::min(want, 2048), 256, 0, s>>>(width, off, n_slices, n_ctas, static_cast<int2 *>(d),
+                                                       static_cast<int4 *>(dtmp), cstart);
+    return cudaGetLastError();
+}
+
 // One warp per slice of dtmp: the diagonals of a diagonal slice into diag from
 // the slice's place on; place -1 for a slice that is not diagonal.  count[0], [1]:
 // slot rows and number of the diagonal slices.  A row of a diagonal slice has a
