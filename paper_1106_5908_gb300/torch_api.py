@@ -170,7 +170,8 @@ class Matrix:
             # (empty_like takes a fifth less than empty with a dtype and a device)
             y = (torch.empty_like(x) if out_dtype is None and x.dim() == 1 and x.shape[0] == self.n_rows else
                  torch.empty(self.n_rows, dtype=out_dtype or x.dtype, device=x.device))
-        status = abi.spmv_apply(self._h, alpha, _dptr(x), _DT[x.dtype], beta, _dptr(y), _DT[y.dtype], _stream(stream))
+        status = abi.spmv_apply(self._h, float(alpha), _dptr(x), _DT[x.dtype], float(beta), _dptr(y), _DT[y.dtype],
+                                _stream(stream))
         if status:
             abi.check(status, "spmv_apply")
         return y
