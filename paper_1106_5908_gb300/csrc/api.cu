@@ -949,6 +949,7 @@ SellParams sell_params(const SellTable &t, const MatRef &m, double alpha, double
     p.n_slices = t.n;
     p.alpha = alpha;
     p.beta = beta;
+    p.ff = epi_ff(alpha, beta);
     p.dorder = t.diagonal ? t.dorder : nullptr;
     p.diag = t.diag;
     p.dshort = t.slot_rows <= 8LL * t.n;
@@ -1128,6 +1129,7 @@ spmv_status apply_impl(spmv_matrix *h, double alpha, const void *x, int xk, doub
             sp.n_chunks = tt->n;
             sp.alpha = alpha;
             sp.beta = beta;
+            sp.ff = epi_ff(alpha, beta);
             sp.err = h->d_err;
             return tops.launch(sp, s) == cudaSuccess ? SPMV_OK : SPMV_ERR_CUDA;
         }
@@ -1135,8 +1137,8 @@ spmv_status apply_impl(spmv_matrix *h, double alpha, const void *x, int xk, doub
     SlotOps sops;
     SlotTable *t = nullptr;
     if ((h->family == 4 || h->family == 5 || h->family == 6) &&
-        ((h->d_rmap && slot_ops(h->vk, xk, yk, acc, h->E, true, &sops)) ||
-         slot_ops(h->vk, xk, yk, acc, h->E, false, &sops)) &&
+        (!h->d_rmap || beta == 1.0) &&  // the row-mapped form adds to y
+        slot_ops(h->vk, xk, yk, acc, h->E, h->d_rmap != nullptr, &sops) &&
         (t = get_slots(h, h->E, s)) != nullptr) {
         SlotParams sp{};
         sp.chunks = t->d;
@@ -1147,6 +1149,7 @@ spmv_status apply_impl(spmv_matrix *h, double alpha, const void *x, int xk, doub
         sp.n_chunks = t->n;
         sp.alpha = alpha;
         sp.beta = beta;
+        sp.ff = epi_ff(alpha, beta);
         sp.err = h->d_err;
         return sops.launch(sp, s) == cudaSuccess ? SPMV_OK : SPMV_ERR_CUDA;
     }
@@ -2204,6 +2207,7 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
                 sp.n_chunks = t->n;
                 sp.alpha = alpha;
                 sp.beta = 0.0;
+                sp.ff = epi_ff(alpha, 0.0);
                 sp.err = h->d_err;
                 if (sops.launch(sp, s) != cudaSuccess) return SPMV_ERR_CUDA;
                 done = true;
@@ -2549,6 +2553,7 @@ spmv_status spmv_batched_apply(spmv_batch_handle b, double alpha, const void *co
             p.n_chunks = b->slots.n;
             p.alpha = alpha;
             p.beta = beta;
+            p.ff = epi_ff(alpha, beta);
             SlotParams p9 = p;
             if (b->mixed) {
                 p9.chunks = b->slots9.d;
@@ -2590,7 +2595,7 @@ spmv_status spmv_batched_apply(spmv_batch_handle b, double alpha, const void *co
                 }
                 if (le == cudaSuccess && fork)
                     le = launch_sell_diag_batch(SellBatchParams{b->d_dlist, b->d_dmembers, b->d_mats, b->n_dlist, alpha,
-                                                                beta}, b->vk, side);
+                                                                beta, epi_ff(alpha, beta)}, b->vk, side);
                 if (fork) {  // join, also after an error: the capture must end on `cap`
                     if (le == cudaSuccess) le = cudaEventRecord(join, side);
                     const cudaError_t we = cudaStreamWaitEvent(cap, join, 0);

@@ -9,19 +9,19 @@ namespace spmv {
 
 bool slot_ops_batched(int vk, int acc, int E, SlotOps *ops) {
     if (vk == kF64 && acc == kAccF64 && E == 7) {
-        ops->launch = &SlotKernel<7, double, double, double, AccF64, false, true>::launch;
+        ops->launch = &SlotKernel<7, double, double, double, AccF64, kUpdPlain, true>::launch;
         return true;
     }
     if (vk == kF64 && acc == kAccF64 && E == 9) {
-        ops->launch = &SlotKernel<9, double, double, double, AccF64, false, true>::launch;
+        ops->launch = &SlotKernel<9, double, double, double, AccF64, kUpdPlain, true>::launch;
         return true;
     }
     if (vk == kF32 && acc == kAccFF && E == 7) {
-        ops->launch = &SlotKernel<7, float, float, float, AccFR, false, true>::launch;
+        ops->launch = &SlotKernel<7, float, float, float, AccFR, kUpdPlain, true>::launch;
         return true;
     }
     if (vk == kF32 && acc == kAccFF && E == 9) {
-        ops->launch = &SlotKernel<9, float, float, float, AccFR, false, true>::launch;
+        ops->launch = &SlotKernel<9, float, float, float, AccFR, kUpdPlain, true>::launch;
         return true;
     }
     return false;
@@ -32,14 +32,14 @@ bool slot_ops(int vk, int xk, int yk, int acc, int E, bool pre, SlotOps *ops) {
         // row-mapped products (the split's nonlocal part): FP64, E = 7 (E = 9
         // measured no faster there: split 230.9 against 229.4 us)
         if (vk == kF64 && xk == kF64 && yk == kF64 && acc == kAccF64 && E == 7) {
-            ops->launch = &SlotKernel<7, double, double, double, AccF64, true>::launch;
+            ops->launch = &SlotKernel<7, double, double, double, AccF64, kUpdMap>::launch;
             return true;
         }
         return false;
     }
 #define SPMV_S(VK_, XK_, YK_, ACCK_, E_, VT_, XT_, YT_, ACC_)                                 \
     if (vk == VK_ && xk == XK_ && yk == YK_ && acc == ACCK_ && E == E_) {                     \
-        ops->launch = &SlotKernel<E_, VT_, XT_, YT_, ACC_>::launch;                            \
+        ops->launch = &SlotKernel<E_, VT_, XT_, YT_, ACC_>::launch_any;                          \
         return true;                                                                          \
     }
     SPMV_S(kF64, kF64, kF64, kAccF64, 7, double, double, double, AccF64)

@@ -39,6 +39,7 @@ struct SlotParams {
     const int32_t *cmat;
     int32_t n_chunks;
     double alpha, beta;
+    EpiFF ff;               // alpha and beta for FP32 rows
     int32_t *err;           // device error word (the staged variant's bounded waits)
 };
 
@@ -62,18 +63,19 @@ __device__ __forceinline__ int32_t ld_stream(const int32_t *p, uint64_t pol) {
 // instead of the packed lane words: only FP64 with E = 9 (150.1 against
 // 152.5 us on the Hamiltonian-like matrix; the packed words win elsewhere, e.g.
 // E = 11 154 against 169 us, the split's nonlocal part 256 against 262 us).
-template <int E, typename VT, bool PRE>
+template <int E, typename VT, int UPD>
 struct kSlotScan {
-    static constexpr bool value = std::is_same<VT, double>::value && E == 9 && !PRE;
+    static constexpr bool value = std::is_same<VT, double>::value && E == 9 && UPD < kUpdMap;
 };
 
-// PRE: the row epilogue's operands (row map, old y) are loaded before the FMA
-// chains (row-mapped products: the nonlocal part of the split form).
+// UPD: the form of the update (kUpd*), known at compile time: a test or a predicated-off
+// FP64 multiply per row costs the plain product 2 to 6 % (147 -> 150..155 us).  From
+// kUpdAdd on the row epilogue's operands (old y, row map) are loaded before the FMA chains.
 // BATCHED: chunks of many matrices in one launch; chunk c belongs to matrix
 // cmat[c] of the table mats (its own x, y and CRS arrays).
 // The persistent loop of one warp over chunks c, c + nwarps, ... of p (srow:
 // the warp's row buffer).
-template <int E, typename VT, typename XT, typename YT, typename ACC, bool PRE, bool BATCHED>
+template <int E, typename VT, typename XT, typename YT, typename ACC, int UPD, bool BATCHED>
 __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c, int nwarps) {
     constexpr int SL = 32 * E;
     const int lane = threadIdx.x & 31;
@@ -192,11 +194,14 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
         } else if (dc.r1f & kChunkEmpty) {
             rows_per_lane<VT, XT, YT, ACC, false>(m, r0, r1, x, y, alpha, beta, plain, lane);
         } else {
-            RowEpilogue<YT> epi;
-            if constexpr (PRE) epi.prefetch(y, m.rmap, r0, r1 - r0, emode >= kEpiAdd, lane);
+            RowEpilogue<YT, UPD> epi;
+            if constexpr (UPD >= kUpdAdd) {
+                constexpr bool reads_y = std::is_same<ACC, AccF64>::value;
+                epi.prefetch(y, m.rmap, r0, r1 - r0, reads_y || emode >= kEpiAdd, lane);
+            }
             const int hi = hi_of(dc);
             const uint32_t mbits = mc & ((1u << E) - 1u);
-            if constexpr (kSlotScan<E, VT, PRE>::value) {
+            if constexpr (kSlotScan<E, VT, UPD>::value) {
                 const uint32_t next_bits = __shfl_down_sync(0xffffffffu, mbits, 1);
                 const bool ends = (lane * E + E >= dc.k1 - dc.k0) || (lane < 31 && (next_bits & 1u));
                 chunk_lane<E, VT, XT, ACC>(vc, xc, mbits, 0, hi, ends, r0, srow, lane,
@@ -208,14 +213,23 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
                                                static_cast<int>((mc >> kSlotChainShift) & kSlotChainMask));
             }
             __syncwarp();
-            if constexpr (PRE) {
-                epi.store(y, srow, r1 - r0, alpha, beta, emode, lane);
+            if constexpr (UPD >= kUpdAdd) {
+                epi.template store<VT>(m, x, y, srow, r0, r1 - r0, alpha, beta, p.ff, emode, lane);
             } else {
                 for (int q = lane; q < r1 - r0; q += 32) {
                     if constexpr (std::is_same<ACC, AccF64>::value) {
-                        const int64_t row = (!BATCHED && m.rmap) ? __ldg(m.rmap + r0 + q) : r0 + q;
-                        y[row] = narrow<YT>(epi_apply(srow[q].get(), y + row, alpha, beta, emode));
+                        const double v = srow[q].get();
+                        // (the batch: one compiled kernel for all updates)
+                        if constexpr (BATCHED) y[r0 + q] = epi_apply(v, y + r0 + q, alpha, beta, emode);
+                        else y[r0 + q] = UPD == kUpdScale ? alpha * v : v;
                     } else {
+                        if constexpr (BATCHED) {
+                            float out;
+                            if (!plain && epi_ff_row(p.ff, srow[q], emode >= kEpiAdd ? y[r0 + q] : 0.0f, out)) {
+                                y[r0 + q] = out;
+                                continue;
+                            }
+                        }
                         store_acc<VT, false>(m, x, y, r0 + q, srow[q], alpha, beta, plain);
                     }
                 }
@@ -248,15 +262,15 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
 // 80 it spills: 256 matrices 0.85 against 0.655 ms).
 template <int E, typename VT, bool BATCHED>
 constexpr int slot_min_ctas() {
-    return sizeof(VT) == 8 ? (E <= 11 ? 2 : 1) : ((E <= 9 && !BATCHED) ? 3 : ((E <= 11 && !BATCHED) ? 2 : 1));
+    return sizeof(VT) == 8 ? (E <= 11 ? 2 : 1) : ((E <= 9 && !BATCHED) ? 3 : (!BATCHED ? 2 : 1));
 }
 
-template <int E, typename VT, typename XT, typename YT, typename ACC, bool PRE = false, bool BATCHED = false>
+template <int E, typename VT, typename XT, typename YT, typename ACC, int UPD = kUpdPlain, bool BATCHED = false>
 __global__ void __launch_bounds__(256, (slot_min_ctas<E, VT, BATCHED>())) k_slot(const SlotParams p) {
     static_assert(sizeof(ACC) == 8, "row buffer entries are 8 bytes");
     __shared__ ACC s_rows[8][kWarpRowCap];
     const int wib = threadIdx.x >> 5;
-    slot_loop<E, VT, XT, YT, ACC, PRE, BATCHED>(p, s_rows[wib], blockIdx.x * 8 + wib, gridDim.x * 8);
+    slot_loop<E, VT, XT, YT, ACC, UPD, BATCHED>(p, s_rows[wib], blockIdx.x * 8 + wib, gridDim.x * 8);
 }
 
 // A batch whose members were tuned apart: the chunks of the members given 7
@@ -268,9 +282,9 @@ __global__ void __launch_bounds__(256, (slot_min_ctas<9, VT, true>())) k_slot_mi
     static_assert(sizeof(ACC) == 8, "row buffer entries are 8 bytes");
     __shared__ ACC s_rows[8][kWarpRowCap];
     const int wib = threadIdx.x >> 5;
-    slot_loop<7, VT, XT, YT, ACC, false, true>(p7, s_rows[wib], blockIdx.x * 8 + wib, gridDim.x * 8);
+    slot_loop<7, VT, XT, YT, ACC, kUpdPlain, true>(p7, s_rows[wib], blockIdx.x * 8 + wib, gridDim.x * 8);
     __syncwarp();
-    slot_loop<9, VT, XT, YT, ACC, false, true>(p9, s_rows[wib], blockIdx.x * 8 + wib, gridDim.x * 8);
+    slot_loop<9, VT, XT, YT, ACC, kUpdPlain, true>(p9, s_rows[wib], blockIdx.x * 8 + wib, gridDim.x * 8);
 }
 
 template <typename VT, typename XT, typename YT, typename ACC>
@@ -497,7 +511,7 @@ __global__ void __launch_bounds__(256) k_slot_relayout(const ChunkDesc *__restri
     }
 }
 
-template <int E, typename VT, typename XT, typename YT, typename ACC, bool PRE = false, bool BATCHED = false>
+template <int E, typename VT, typename XT, typename YT, typename ACC, int UPD = kUpdPlain, bool BATCHED = false>
 struct SlotKernel {
     static int grid_limit() {
         static int cached = -1;
@@ -507,19 +521,33 @@ struct SlotKernel {
         if (cached >= 0 && cached_dev == dev) return cached;
         int per_sm = 0, sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_slot<E, VT, XT, YT, ACC, PRE, BATCHED>, 256, 0) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_slot<E, VT, XT, YT, ACC, UPD, BATCHED>, 256, 0) !=
             cudaSuccess)
             return 0;
         cached = per_sm * sms;
         cached_dev = dev;
         return cached;
     }
+    // the kernel compiled for the update.  Hamiltonian-like 4 M rows, one kernel for
+    // all updates against these: -0.75*A*x + 0.5*y FP64 184 -> 161 us, FP32 E = 7 145 ->
+    // 127, E = 11 134 -> 117, E = 15 129 -> 123; y - A*x FP64 184 -> 153
+    static cudaError_t launch_any(const SlotParams &p, cudaStream_t s) {
+        if constexpr (IsFloatPair<ACC>::value) {
+            if (p.beta != 0.0 || p.ff.on) return SlotKernel<E, VT, XT, YT, ACC, kUpdGeneral, false>::launch(p, s);
+        } else {
+            if (p.beta == 1.0 && (p.alpha == 1.0 || p.alpha == -1.0))
+                return SlotKernel<E, VT, XT, YT, ACC, kUpdAdd, false>::launch(p, s);
+            if (p.beta != 0.0) return SlotKernel<E, VT, XT, YT, ACC, kUpdGeneral, false>::launch(p, s);
+            if (p.alpha != 1.0) return SlotKernel<E, VT, XT, YT, ACC, kUpdScale, false>::launch(p, s);
+        }
+        return launch(p, s);
+    }
     static cudaError_t launch(const SlotParams &p, cudaStream_t s) {
         if (p.n_chunks <= 0) return cudaSuccess;
         const int lim = grid_limit();
         if (lim <= 0) return cudaErrorInvalidConfiguration;
         const int want = (p.n_chunks + 7) / 8;
-        k_slot<E, VT, XT, YT, ACC, PRE, BATCHED><<<want < lim ? want : lim, 256, 0, s>>>(p);
+        k_slot<E, VT, XT, YT, ACC, UPD, BATCHED><<<want < lim ? want : lim, 256, 0, s>>>(p);
         return cudaGetLastError();
     }
 };
