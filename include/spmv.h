@@ -117,6 +117,12 @@ spmv_status spmv_create_symmetric(spmv_handle *out, int32_t n, int64_t nnz, cons
  * the same pass; other derived copies are laid out again when they are used. */
 spmv_status spmv_set_values(spmv_handle h, const void *val, spmv_dtype t, void *stream);
 
+/* spmv_set_values followed by y = alpha*A*x (spmv_apply with beta = 0), in one pass
+ * where the new values go to a row-slice copy on diagonals in their own type and the
+ * vectors have it too.  y overlaps neither x nor val. */
+spmv_status spmv_set_values_apply(spmv_handle h, const void *val, spmv_dtype t, double alpha, const void *x,
+                                  spmv_dtype xt, void *y, spmv_dtype yt, void *stream);
+
 /* Shape and plan of a handle.  plan[0..7] receives: kernel family (as for
  * spmv_set_plan), entries per lane or thread segment E (family 5: the sorting
  * window sigma), threads per CTA, number of chunks, tiles or slices, rows per

@@ -29,6 +29,7 @@ SPMV_NOALLOC_MAX_COLS = 1 << 20
 # Every entry point declared in include/spmv.h.
 EXPORTS = (
     "spmv_status_string", "spmv_version", "spmv_create", "spmv_create_symmetric", "spmv_destroy", "spmv_set_values",
+    "spmv_set_values_apply",
     "spmv_get_info", "spmv_row_histogram", "spmv_set_plan", "spmv_set_accumulator", "spmv_apply", "spmv_split_create",
     "spmv_split_destroy", "spmv_split_get_plan", "spmv_apply_split", "spmv_apply_split_vector",
     "spmv_split_get_halo",
@@ -70,6 +71,7 @@ def load() -> ctypes.CDLL:
         "spmv_create_symmetric": (st, [vp, i32, i64, vp, vp, vp, st, ctypes.c_int, vp]),
         "spmv_destroy": (None, [vp]),
         "spmv_set_values": (st, [vp, vp, st, vp]),
+        "spmv_set_values_apply": (st, [vp, vp, st, f64, vp, st, vp, st, vp]),
         "spmv_get_info": (st, [vp, vp, vp, vp, vp]),
         "spmv_row_histogram": (st, [vp, i32, vp]),
         "spmv_set_plan": (st, [vp, i32, i32]),
@@ -130,6 +132,7 @@ spmv_create = _fwd("spmv_create")
 spmv_create_symmetric = _fwd("spmv_create_symmetric")
 spmv_destroy = _fwd("spmv_destroy")
 spmv_set_values = _fwd("spmv_set_values")
+spmv_set_values_apply = _fwd("spmv_set_values_apply")
 spmv_get_info = _fwd("spmv_get_info")
 spmv_row_histogram = _fwd("spmv_row_histogram")
 spmv_set_plan = _fwd("spmv_set_plan")

@@ -1609,11 +1609,10 @@ spmv_status spmv_create(spmv_handle *out, int32_t n_rows, int32_t n_cols, int64_
 
 void spmv_destroy(spmv_handle h) { destroy_matrix(h); }
 
-spmv_status spmv_set_values(spmv_handle h, const void *val, spmv_dtype t, void *stream) {
-    if (!h || (h->nnz > 0 && !val)) return SPMV_ERR_INVALID_ARG;
-    if (t != SPMV_F64 && t != SPMV_F32) return SPMV_ERR_INVALID_ARG;
-    DeviceGuard g(h->device);
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
+// New values for h; y not null: also y = alpha*A*x with them in the same pass where
+// it can be done (*applied).  The vectors have h's value type.
+static spmv_status set_values_impl(spmv_matrix *h, const void *val, spmv_dtype t, double alpha, const void *x, void *y,
+                                   bool *applied, cudaStream_t s) {
     if (h->nnz == 0) return SPMV_OK;
     // a row-slice copy that served the last values gets the new ones in the same
     // pass; other copies are laid out again when they are used
@@ -1621,9 +1620,13 @@ spmv_status spmv_set_values(spmv_handle h, const void *val, spmv_dtype t, void *
     const bool fused = h->family == 5 && f != h->sells.end() && f->second.vals_valid && f->second.diagonal &&
                        sell_tile_fits(h);
     if (fused) {
-        const SellParams p =
-            sell_params(f->second, MatRef{h->d_rp, h->d_col, nullptr, nullptr, nullptr, nullptr, nullptr}, 1.0, 0.0);
+        const bool prod = y && static_cast<int>(t) == h->vk && !h->sym && !h->d_rmap &&
+                          (h->vk == kF64 || h->acc32 == kAccFF);
+        const SellParams p = sell_params(
+            f->second, MatRef{h->d_rp, h->d_col, prod ? val : nullptr, nullptr, prod ? x : nullptr, prod ? y : nullptr, nullptr},
+            alpha, 0.0);
         CK(launch_sell_set_values(p, val, t, h->d_val, h->vk, h->max_row, s));
+        if (applied) *applied = prod;
     } else {
         CK(launch_convert(val, t, h->d_val, h->vk, h->nnz, s));
     }
@@ -1642,6 +1645,27 @@ spmv_status spmv_set_values(spmv_handle h, const void *val, spmv_dtype t, void *
     for (auto &kv : h->sells) kv.second.vals_valid = false;
     if (fused) f->second.vals_valid = true;
     return SPMV_OK;
+}
+
+spmv_status spmv_set_values(spmv_handle h, const void *val, spmv_dtype t, void *stream) {
+    if (!h || (h->nnz > 0 && !val)) return SPMV_ERR_INVALID_ARG;
+    if (t != SPMV_F64 && t != SPMV_F32) return SPMV_ERR_INVALID_ARG;
+    DeviceGuard g(h->device);
+    return set_values_impl(h, val, t, 1.0, nullptr, nullptr, nullptr, static_cast<cudaStream_t>(stream));
+}
+
+spmv_status spmv_set_values_apply(spmv_handle h, const void *val, spmv_dtype t, double alpha, const void *x,
+                                  spmv_dtype xt, void *y, spmv_dtype yt, void *stream) {
+    if (!h || (h->nnz > 0 && !val)) return SPMV_ERR_INVALID_ARG;
+    if (t != SPMV_F64 && t != SPMV_F32) return SPMV_ERR_INVALID_ARG;
+    if ((h->n_rows > 0 && !y) || (h->n_cols > 0 && h->n_rows > 0 && !x)) return SPMV_ERR_INVALID_ARG;
+    DeviceGuard g(h->device);
+    const bool same = static_cast<int>(xt) == h->vk && static_cast<int>(yt) == h->vk;
+    bool applied = false;
+    const spmv_status st =
+        set_values_impl(h, val, t, alpha, x, same ? y : nullptr, &applied, static_cast<cudaStream_t>(stream));
+    if (st != SPMV_OK || applied) return st;
+    return spmv_apply(h, alpha, x, xt, 0.0, y, yt, stream);
 }
 
 spmv_status spmv_get_info(spmv_handle h, int32_t *n_rows, int32_t *n_cols, int64_t *nnz, int32_t *plan) {

@@ -479,26 +479,97 @@ template <typename VT> __device__ __forceinline__ VT value_as(float v) {
     else return widen(v);
 }
 
+// CNT slot rows of a half slice, their values from the lane's row of the tile (len
+// entries): into the slots and into the sum, in sell_diag_block's order.
+template <int CNT, bool DIAG, typename ACC, typename VT>
+__device__ __forceinline__ void set_values_block(ACC &acc, VT *out, const VT *row, int len,
+                                                 const int32_t *__restrict__ cb, const int4 *__restrict__ dp, int r,
+                                                 const VT *__restrict__ x) {
+    int32_t c[CNT];
+    if constexpr (DIAG) {
+        const int4 a = __ldg(dp);
+        int4 b = make_int4(0, 0, 0, 0);
+        if constexpr (CNT > 4) b = __ldg(dp + 1);
+        const int32_t o[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int u = 0; u < CNT; ++u) c[u] = r + o[u];
+    } else {
+#pragma unroll
+        for (int u = 0; u < CNT; ++u) c[u] = __ldg(cb + u * kSellC);
+    }
+    VT xv[CNT];
+#pragma unroll
+    for (int u = 0; u < CNT; ++u) xv[u] = (DIAG || c[u] >= 0) ? __ldg(x + c[u]) : VT(0);
+#pragma unroll
+    for (int u = 0; u < CNT; ++u) {
+        const VT v = u < len ? row[u] : VT(0);
+        out[u * kSellC] = v;
+        acc.fma(v, xv[u]);
+        if (u % kSellU == kSellU - 1 || u == CNT - 1) end_run(acc);
+    }
+}
+
+template <bool DIAG, typename ACC, typename VT>
+__device__ __forceinline__ void set_values_row(ACC &acc, int w, VT *out, const VT *row, int len,
+                                               const int32_t *__restrict__ cb, const int4 *__restrict__ dp, int r,
+                                               const VT *__restrict__ x) {
+    for (; w >= 8; w -= 8) {
+        set_values_block<8, DIAG>(acc, out, row, len, cb, dp, r, x);
+        out += 8 * kSellC;
+        row += 8;
+        len -= 8;
+        if constexpr (DIAG) dp += 2;
+        else cb += 8 * kSellC;
+    }
+    switch (w) {
+        case 7: set_values_block<7, DIAG>(acc, out, row, len, cb, dp, r, x); break;
+        case 6: set_values_block<6, DIAG>(acc, out, row, len, cb, dp, r, x); break;
+        case 5: set_values_block<5, DIAG>(acc, out, row, len, cb, dp, r, x); break;
+        case 4: set_values_block<4, DIAG>(acc, out, row, len, cb, dp, r, x); break;
+        case 3: set_values_block<3, DIAG>(acc, out, row, len, cb, dp, r, x); break;
+        case 2: set_values_block<2, DIAG>(acc, out, row, len, cb, dp, r, x); break;
+        case 1: set_values_block<1, DIAG>(acc, out, row, len, cb, dp, r, x); break;
+        default: break;
+    }
+}
+
 // New values: from CRS order (type ST) into the handle's CRS copy dval and into
 // the slices, one read and two writes (27-point 128^3 FP64, 1.34 GB: 225 us, 5.9
 // TB/s; a copy and a layout pass of its own took 314).  Rows of at most kTileMaxW
-// entries.
-template <typename ST, typename VT>
-__global__ void __launch_bounds__(256) k_sell_set_values(const int4 *__restrict__ dorder,
-                                                         const int32_t *__restrict__ srows, int32_t n_slices,
-                                                         const int32_t *__restrict__ rp, const ST *__restrict__ val,
-                                                         VT *__restrict__ dval, VT *__restrict__ vals, int max_w) {
+// entries.  ACC not void: also y = alpha*A*x with them, the sums of k_sell_diag (a
+// poisoned FP32 row is summed again from val: dval may still be on its way).  Memory
+// bounds the one and the FP64 pipe the other: together 236 us (5.7 TB/s), one after
+// the other 327 (FP32 144 against 180; 7-point 160^3 143 and 183).
+template <typename ST, typename VT, typename ACC>
+__global__ void __launch_bounds__(256) k_sell_set_values(const SellParams p, const ST *__restrict__ val,
+                                                         VT *__restrict__ dval, int max_w) {
     extern __shared__ __align__(16) unsigned char smem[];
+    VT *__restrict__ vals = static_cast<VT *>(const_cast<void *>(p.vals));
+    const VT *__restrict__ x = static_cast<const VT *>(p.m.x);
+    VT *__restrict__ y = static_cast<VT *>(p.m.y);
+    const double alpha = p.alpha;
+    const int emode = epi_mode(alpha, 0.0);
     const int lane = threadIdx.x & 31;
     VT *tile = reinterpret_cast<VT *>(smem) + (threadIdx.x >> 5) * TilePack<VT>::entries(max_w);
     const uint64_t pol = l2_evict_first_policy();
-    each_half_slice(dorder, srows, n_slices, rp, lane, [&](int i, const int4 &d, int, int k0, int k1) {
+    each_half_slice(p.dorder, p.srows, p.n_slices, p.m.rp, lane, [&](int i, const int4 &d, int r, int k0, int k1) {
         const TilePack<VT> t(d.y, k0, k1, lane);
         bool free = false;  // the tile's last bulk copies have read it
         for (unsigned m = t.heads; m; m &= m - 1) {  // segments, coalesced
             const int h = __ffs(m) - 1;
             const int ks = __shfl_sync(0xffffffffu, k0, h), ke = __shfl_sync(0xffffffffu, t.kend, h);
             VT *out = tile + __shfl_sync(0xffffffffu, t.pos, h) - ks;
+            if constexpr (std::is_same<ST, VT>::value) {
+                // asynchronous copies: all of the half slice's values in flight at once (8
+                // to a lane in registers: 268 us with the product)
+                if (!free) TilePack<VT>::drain();
+                free = true;
+                for (int k = ks + lane; k < ke; k += 32)
+                    asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], %2, %3;" ::"r"(smem_u32(out + k)),
+                                 "l"(val + k), "n"(sizeof(VT)), "l"(pol)
+                                 : "memory");
+                continue;
+            }
             for (int k = ks + lane; __any_sync(0xffffffffu, k < ke); k += 256) {
                 ST v[8];
 #pragma unroll
@@ -510,12 +581,30 @@ __global__ void __launch_bounds__(256) k_sell_set_values(const int4 *__restrict_
                     if (k + 32 * u < ke) out[k + 32 * u] = value_as<VT>(v[u]);
             }
         }
+        if constexpr (std::is_same<ST, VT>::value) asm volatile("cp.async.wait_all;" ::: "memory");
         t.store(tile, dval, k0, lane);
         VT *out = vals + static_cast<int64_t>(d.x) * kSellC + (i & 1) * 32 + lane;
         const VT *row = tile + t.pos;
         const int len = k1 - k0;
+        if constexpr (std::is_void<ACC>::value) {
 #pragma unroll 8
-        for (int j = 0; j < d.y; ++j) out[j * kSellC] = j < len ? row[j] : VT(0);
+            for (int j = 0; j < d.y; ++j) out[j * kSellC] = j < len ? row[j] : VT(0);
+        } else {
+            ACC acc;
+            acc.zero();
+            if (d.w >= 0)
+                set_values_row<true>(acc, d.y, out, row, len, static_cast<const int32_t *>(nullptr), p.diag + d.w, r, x);
+            else
+                set_values_row<false>(acc, d.y, out, row, len,
+                                      p.cols + static_cast<int64_t>(d.x) * kSellC + (i & 1) * 32 + lane,
+                                      static_cast<const int4 *>(nullptr), r, x);
+            if (r >= 0) {
+                if constexpr (std::is_same<ACC, AccF64>::value)
+                    y[r] = epi_apply(acc.get(), y + r, alpha, 0.0, emode);
+                else
+                    sell_store<VT>(p.m, x, y, r, acc, alpha, 0.0, p.ff, emode == kEpiPlain, VT(0));
+            }
+        }
         __syncwarp();
     });
     TilePack<VT>::drain();
@@ -607,20 +696,25 @@ static int tile_grid(K kernel, int32_t n_slices, size_t smem) {
 
 int sell_tile_max_row() { return kTileMaxW; }
 
-template <typename ST, typename VT>
+template <typename ST, typename VT, typename ACC = void>
 static cudaError_t set_values_as(const SellParams &p, const void *val, void *dval, int max_w, cudaStream_t s) {
     const size_t smem = sizeof(VT) * 8 * TilePack<VT>::entries(max_w);
-    const int grid = tile_grid(k_sell_set_values<ST, VT>, p.n_slices, smem);
+    const int grid = tile_grid(k_sell_set_values<ST, VT, ACC>, p.n_slices, smem);
     if (grid <= 0) return cudaErrorInvalidConfiguration;
-    k_sell_set_values<ST, VT><<<grid, 256, smem, s>>>(p.dorder, p.srows, p.n_slices, p.m.rp,
-                                                      static_cast<const ST *>(val), static_cast<VT *>(dval),
-                                                      static_cast<VT *>(const_cast<void *>(p.vals)), max_w);
+    k_sell_set_values<ST, VT, ACC>
+        <<<grid, 256, smem, s>>>(p, static_cast<const ST *>(val), static_cast<VT *>(dval), max_w);
     return cudaGetLastError();
 }
 
 cudaError_t launch_sell_set_values(const SellParams &p, const void *val, int sk, void *dval, int vk, int max_w,
                                    cudaStream_t s) {
     if (p.n_slices <= 0) return cudaSuccess;
+    if (p.m.y) {  // with the product: the accumulators of sell_ops
+        if (sk != vk) return cudaErrorInvalidValue;
+        if (vk == kF64) return set_values_as<double, double, AccF64>(p, val, dval, max_w, s);
+        return max_w <= kFRMaxRun ? set_values_as<float, float, AccFR>(p, val, dval, max_w, s)
+                                  : set_values_as<float, float, AccFRF>(p, val, dval, max_w, s);
+    }
     if (vk == kF64)
         return sk == kF64 ? set_values_as<double, double>(p, val, dval, max_w, s)
                           : set_values_as<float, double>(p, val, dval, max_w, s);

@@ -176,6 +176,15 @@ class Matrix:
             abi.check(status, "spmv_apply")
         return y
 
+    def set_values_apply(self, val: torch.Tensor, x: torch.Tensor, alpha: float = 1.0, stream=None) -> torch.Tensor:
+        """set_values(val), then alpha*A*x, in one pass where the layout allows it."""
+        self._values_token = None
+        y = torch.empty(self.n_rows, dtype=x.dtype, device=x.device)
+        abi.check(abi.spmv_set_values_apply(self._h, _dptr(val.contiguous()), _DT[val.dtype], float(alpha), _dptr(x),
+                                            _DT[x.dtype], _dptr(y), _DT[y.dtype], _stream(stream)),
+                  "spmv_set_values_apply")
+        return y
+
     def spmm(self, X: torch.Tensor, Y: Optional[torch.Tensor] = None, alpha: float = 1.0,
              beta: float = 0.0, stream=None) -> torch.Tensor:
         """Block vectors stored interleaved: X (n_cols, nrhs), Y (n_rows, nrhs)."""
@@ -331,10 +340,9 @@ class SpMVFunction(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, val: torch.Tensor, x: torch.Tensor, A: Matrix, alpha: float = 1.0):
-        A.set_values(val.detach())
+        y = A.set_values_apply(val.detach(), x.detach(), alpha)
         ctx.token = object()
         A._values_token = ctx.token  # the handle holds this forward's values
-        y = A.apply(x.detach(), alpha=alpha)
         ctx.save_for_backward(val.detach(), x.detach())
         ctx.A = A
         ctx.alpha = alpha
