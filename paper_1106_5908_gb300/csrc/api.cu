@@ -604,16 +604,20 @@ constexpr double kBatchSlotMeanE9 = 4.0;
 // Members of at least this many rows whose slices are diagonal run on them instead.
 constexpr int32_t kBatchDiagMinSize = 32768;
 
-void autotune(spmv_matrix *h) {
+// Share of far entries (column_randomness) above which columns count as scattered.
+constexpr double kScattered = 0.25;
+
+// slices = false: the row slices are not considered (their padding is not counted).
+void autotune(spmv_matrix *h, bool slices = true) {
     const double mean = h->n_rows ? static_cast<double>(h->nnz) / h->n_rows : 0.0;
     h->max_row = 0;
     for (int32_t i = 0; i < h->n_rows; ++i) h->max_row = std::max(h->max_row, h->h_rp[i + 1] - h->h_rp[i]);
     int T = 1;
     while (T < 32 && T < mean * 0.5) T <<= 1;
     h->T = T;
-    const bool scattered = h->col_random > 0.25;
+    const bool scattered = h->col_random > kScattered;
     h->sigma = kSellSigma;
-    h->sell_pad = h->n_rows > 0 ? sell_padding(h->h_rp.data(), h->n_rows, kSellSigma) : 1.0;
+    h->sell_pad = slices && h->n_rows > 0 ? sell_padding(h->h_rp.data(), h->n_rows, kSellSigma) : 1.0;
     if (h->vk == kF32) {
         h->family = scattered ? 4 : 0;
         h->E = scattered ? 9 : 15;
@@ -1420,7 +1424,16 @@ static spmv_matrix *get_full(spmv_matrix *h, cudaStream_t s) {
     const uint64_t have = h->full ? h->full_version : 0;  // new handles: the values of their creation
     const bool again = h->full_asked == h->values_version;
     h->full_asked = h->values_version;
-    if (have != h->values_version && !again) return nullptr;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return nullptr;
+    if (cap == cudaStreamCaptureStatusNone) {
+        if (have != h->values_version && !again) return nullptr;
+    } else if (!h->full || (have != h->values_version && again)) {
+        // under capture nothing is allocated, and values that the two passes already have
+        // are not laid out anew: they would come with the graph's first run, too late for
+        // an apply before it
+        return nullptr;
+    }
     if (!h->full) {
         const int32_t n = h->n_rows;
         const int64_t ns = h->h_rowT[n], nnz = h->nnz + ns;
@@ -1456,7 +1469,7 @@ static spmv_matrix *get_full(spmv_matrix *h, cudaStream_t s) {
             h->full_off = true;
             return nullptr;
         }
-        autotune(f);
+        autotune(f, f->vk == kF64 && f->col_random <= kScattered);
         if (f->vk == kF32) {
             // float-float sums: the two passes round y twice, but sum half of each row
             // in float-float, so FP32 runs over all of it would be less exact (1.05 M
@@ -2102,7 +2115,7 @@ spmv_status spmm_apply(spmv_handle h, int32_t nrhs, double alpha, const void *X,
     // against 194, 5-point 1400^2 74 against 80).
     int l2 = 0;
     cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, h->device);
-    const bool scattered = h->col_random > 0.25;
+    const bool scattered = h->col_random > kScattered;
     SellTable *t = nullptr;
     if (h->sell_pad <= kSellMaxPadding && (t = get_sell(h, kSellSigma, s)) != nullptr) {
         const bool vec = (nrhs % 2 == 0) && (reinterpret_cast<uintptr_t>(X) % 16 == 0) &&
@@ -2196,7 +2209,7 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
             }
         }
         const double meanT = h->n_cols ? static_cast<double>(h->nnz) / h->n_cols : 0.0;
-        if (!ind && h->col_random <= 0.25 && meanT >= kSellMinRowLength) {
+        if (!ind && h->col_random <= kScattered && meanT >= kSellMinRowLength) {
             // A^T of a stencil-like matrix with long rows: the sorted row-slice
             // kernel on a row-slice copy of A^T (as the tuner picks for a forward
             // product of such a matrix)

@@ -151,3 +151,52 @@ def test_expanded_and_two_pass_products_agree(n, dtype):
         M.set_accumulator("f64")
         assert _abi.spmv_apply(M.handle, 1.0, xd.data_ptr(), _abi.SPMV_F32, 0.0, y.data_ptr(), _abi.SPMV_F32,
                                None) == _abi.SPMV_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("applies_before,new_values", [(1, False), (1, True), (2, True)])
+def test_symmetric_apply_captured(applies_before, new_values):
+    """A captured apply allocates nothing, and applies beside the graph stay right
+    whether or not it has run: on the first values, and with new values that one apply
+    (two passes) or none has used when the capture begins."""
+    U = W.random_symmetric_upper(20000, seed=5, max_len=9)
+    M = sym(U)
+    x = dev(W.uniform(U.n_rows, 3))
+    y = torch.zeros_like(x)
+    val = U.val
+    M.apply(x)
+    if new_values:
+        val = W.uniform(U.nnz, 6)
+        M.set_values(dev(val))
+        for _ in range(applies_before - 1):
+            M.apply(x)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        M.apply(x, y)
+    ref, bound = oracle.spmv_sym(U.row_ptr, U.col_idx, val, host(x), with_bound=True)
+    if not new_values or applies_before > 1:
+        assert_within(host(M.apply(x)), ref, bound, 1e-13, "beside the graph")
+    for _ in range(2):
+        y.zero_()
+        g.replay()
+        assert_within(host(y), ref, bound, 1e-13, "replayed")
+    assert_within(host(M.apply(x)), ref, bound, 1e-13, "after the graph")
+
+
+def test_symmetric_new_values_before_any_apply_captured():
+    U = W.random_symmetric_upper(20000, seed=8, max_len=9)
+    M = sym(U)
+    x = dev(W.uniform(U.n_rows, 3))
+    y = torch.zeros_like(x)
+    val = W.uniform(U.nnz, 9)
+    M.set_values(dev(val))
+    M.apply(x)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        M.apply(x, y)
+    g.replay()
+    ref, bound = oracle.spmv_sym(U.row_ptr, U.col_idx, val, host(x), with_bound=True)
+    assert_within(host(y), ref, bound, 1e-13, "replayed")
+    for _ in range(3):
+        assert_within(host(M.apply(x)), ref, bound, 1e-13, "after the graph")
