@@ -568,17 +568,17 @@ __global__ void __launch_bounds__(256) k_sell_set_values(const SellParams p, con
                     asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], %2, %3;" ::"r"(smem_u32(out + k)),
                                  "l"(val + k), "n"(sizeof(VT)), "l"(pol)
                                  : "memory");
-                continue;
-            }
-            for (int k = ks + lane; __any_sync(0xffffffffu, k < ke); k += 256) {
-                ST v[8];
+            } else {
+                for (int k = ks + lane; __any_sync(0xffffffffu, k < ke); k += 256) {
+                    ST v[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = k + 32 * u < ke ? ld_stream_p(val + k + 32 * u, pol) : ST(0);
-                if (!free) TilePack<VT>::drain();
-                free = true;
+                    for (int u = 0; u < 8; ++u) v[u] = k + 32 * u < ke ? ld_stream_p(val + k + 32 * u, pol) : ST(0);
+                    if (!free) TilePack<VT>::drain();
+                    free = true;
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (k + 32 * u < ke) out[k + 32 * u] = value_as<VT>(v[u]);
+                    for (int u = 0; u < 8; ++u)
+                        if (k + 32 * u < ke) out[k + 32 * u] = value_as<VT>(v[u]);
+                }
             }
         }
         if constexpr (std::is_same<ST, VT>::value) asm volatile("cp.async.wait_all;" ::: "memory");
