@@ -158,7 +158,7 @@ spmv_status spmv_row_histogram(spmv_handle h, int32_t nbins, int64_t *counts);
  *           whose slot rows each lie on one diagonal, as on a grid stencil, run
  *           without column indices); FP64,
  *           and FP32 storage with the default accumulator (FP32 runs: a whole
- *           row when no row exceeds 9 entries, else blocks of 4 entries folded
+ *           row when no row exceeds 11 entries, else blocks of 4 entries folded
  *           into float-float), other combinations run the slot-major kernel;
  *           copy built on first use, values follow spmv_set_values;
  * family 6: the slot-major kernel of family 4 with each chunk's values brought
