@@ -92,6 +92,31 @@ cudaError_t dmalloc(T **p, size_t count) {
     return cudaMalloc(reinterpret_cast<void **>(p), count * sizeof(T));
 }
 
+// The capture that records what is enqueued on s (0: work on s runs).
+unsigned long long capture_id(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(s, &st, &id) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    return st == cudaStreamCaptureStatusActive ? id : 0;
+}
+
+// Whether a derived copy holds the current values.  A layout recorded while a stream
+// is captured runs with the graph, so it counts for the rest of that capture only: a
+// call outside the graph lays the values out itself.
+struct Laid {
+    bool now = false;
+    unsigned long long in_capture = 0;  // the capture that lays them out
+    bool on(cudaStream_t s) const { return now || (in_capture != 0 && in_capture == capture_id(s)); }
+    void set(cudaStream_t s) {
+        const unsigned long long id = capture_id(s);
+        if (id) in_capture = id;
+        else now = true;
+    }
+};
+
 // Slot-major copy of a matrix for plan family 4 (per entries-per-lane E).
 struct SlotTable {
     ChunkDesc *d = nullptr;
@@ -100,7 +125,7 @@ struct SlotTable {
     int32_t *cols = nullptr;    // n * 32E column indices, slot-major
     int32_t n = 0;
     int32_t n_long = 0, n_empty = 0;
-    bool vals_valid = false;
+    Laid laid;
 };
 
 // Sorted row-slice copy of a matrix for plan family 5 (per window sigma).
@@ -115,7 +140,7 @@ struct SellTable {
     int32_t n = 0;
     int32_t n_long = 0;
     int64_t slot_rows = 0;
-    bool vals_valid = false;
+    Laid laid;
     // diagonal slices: descriptors with each slice's place in diag (in slice order
     // and in launch order), and the diagonals of the slot rows, padded to 4 per slice
     // (behind cols)
@@ -444,7 +469,7 @@ struct spmv_matrix {
     // pass on the same values (valT_requested records the first one) and
     // invalidated by spmv_set_values
     void *d_valT = nullptr;
-    bool valT_valid = false;
+    Laid valT;
     bool valT_requested = false;
     std::vector<int32_t> h_rowT;
     std::map<std::pair<int, int>, TileTable> tablesT;
@@ -452,7 +477,7 @@ struct spmv_matrix {
     // each of its values among U's; full_off: it does not fit
     spmv_matrix *full = nullptr;
     int32_t *d_fullmap = nullptr;
-    uint64_t full_version = 0;  // values_version that full's values come from
+    Laid full_laid;             // U's current values in full
     uint64_t full_asked = 0;    // values_version of the last apply
     bool full_off = false;
     // FP32 mirror for IR-CG
@@ -701,6 +726,7 @@ SlotTable *get_slots(spmv_matrix *h, int E, cudaStream_t s, bool transposed = fa
     const void *d_val = transposed ? h->d_valT : h->d_val;
     auto it = tabs.find(E);
     if (it == tabs.end()) {
+        if (capture_id(s)) return nullptr;  // its columns would be laid out by the graph
         std::vector<ChunkDesc> d;
         std::vector<uint32_t> lm;
         SlotTable t;
@@ -723,15 +749,15 @@ SlotTable *get_slots(spmv_matrix *h, int E, cudaStream_t s, bool transposed = fa
             (void)cudaGetLastError();  // a failed allocation must not surface at a later launch check
             return nullptr;
         }
-        t.vals_valid = true;
+        t.laid.now = true;
         it = tabs.emplace(E, t).first;
     }
     SlotTable &t = it->second;
-    if (!t.vals_valid) {
+    if (!t.laid.on(s)) {
         if (launch_slot_relayout(t.d, E, static_cast<int64_t>(t.n) * 32 * E, h->vk, d_val, nullptr, t.vals,
                                  nullptr, s) != cudaSuccess)
             return nullptr;
-        t.vals_valid = true;
+        t.laid.set(s);
     }
     return &t;
 }
@@ -850,6 +876,7 @@ SellTable *get_sell(spmv_matrix *h, int32_t sigma, cudaStream_t s, bool transpos
         return cudaMemsetAsync(t.vals, 0, static_cast<size_t>(kSellU) * kSellC * vb, s) == cudaSuccess;
     };
     auto it = tabs.find(sigma);
+    if ((it == tabs.end() || (need_vals && !it->second.vals)) && capture_id(s)) return nullptr;  // nothing is built
     if (it == tabs.end()) {
         SellTable t;
         SellOps o;
@@ -886,18 +913,18 @@ SellTable *get_sell(spmv_matrix *h, int32_t sigma, cudaStream_t s, bool transpos
             (void)cudaGetLastError();  // a failed allocation must not surface at a later launch check
             return nullptr;
         }
-        t.vals_valid = need_vals;
+        t.laid.now = need_vals;
         it = tabs.emplace(sigma, t).first;
     }
     SellTable &t = it->second;
-    if (need_vals && !t.vals_valid) {
+    if (need_vals && !t.laid.on(s)) {
         if (!t.vals && !alloc_vals(t)) {
             (void)cudaGetLastError();
             return nullptr;
         }
         if (launch_sell_relayout(t.d, t.srows, t.n, d_rp, h->vk, d_val, nullptr, t.vals, nullptr, s) != cudaSuccess)
             return nullptr;
-        t.vals_valid = true;
+        t.laid.set(s);
     }
     return &t;
 }
@@ -912,6 +939,7 @@ SellTable *get_sell_positions(spmv_matrix *h, cudaStream_t s) {
     if (!a.diagonal || a.n_long > 0 || a.slot_rows * kSellC > INT32_MAX) return nullptr;
     SellTable *t = get_sell(h, kSellSigma, s, true, false);
     if (!t || !t->diagonal) return nullptr;
+    if ((!t->vpos || t->vpos_sigma != h->sigma) && capture_id(s)) return nullptr;  // nothing is built
     if (t->vpos && t->vpos_sigma != h->sigma) {  // another plan since: other positions
         cudaFree(t->vpos);
         t->vpos = nullptr;
@@ -1421,18 +1449,15 @@ static spmv_status create_symmetric_index(spmv_matrix *h, const int32_t *col_hos
 // values and one apply 174 against 145 us), so the second apply on them does it.
 static spmv_matrix *get_full(spmv_matrix *h, cudaStream_t s) {
     if (h->full_off) return nullptr;
-    const uint64_t have = h->full ? h->full_version : 0;  // new handles: the values of their creation
+    const bool have = h->full ? h->full_laid.on(s) : h->values_version == 0;  // new handles: the values of their creation
     const bool again = h->full_asked == h->values_version;
     h->full_asked = h->values_version;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return nullptr;
     if (cap == cudaStreamCaptureStatusNone) {
-        if (have != h->values_version && !again) return nullptr;
-    } else if (!h->full || (have != h->values_version && again)) {
-        // under capture nothing is allocated, and values that the two passes already have
-        // are not laid out anew: they would come with the graph's first run, too late for
-        // an apply before it
-        return nullptr;
+        if (!have && !again) return nullptr;
+    } else if (!h->full || (!have && again)) {
+        return nullptr;  // under capture nothing is allocated
     }
     if (!h->full) {
         const int32_t n = h->n_rows;
@@ -1479,14 +1504,14 @@ static spmv_matrix *get_full(spmv_matrix *h, cudaStream_t s) {
             f->sell_if_diag = false;
         }
         h->full = f;
-        h->full_version = h->values_version;
+        h->full_laid.now = true;
     }
     spmv_matrix *f = h->full;
-    if (h->full_version != h->values_version) {
+    if (!h->full_laid.on(s)) {
         if (launch_permute(h->d_val, h->d_fullmap, f->d_val, f->nnz, f->vk, s) != cudaSuccess) return nullptr;
-        for (auto &kv : f->slots) kv.second.vals_valid = false;
-        for (auto &kv : f->sells) kv.second.vals_valid = false;
-        h->full_version = h->values_version;
+        for (auto &kv : f->slots) kv.second.laid = Laid();
+        for (auto &kv : f->sells) kv.second.laid = Laid();
+        h->full_laid.set(s);
     }
     f->acc32 = h->acc32;
     return f;
@@ -1527,7 +1552,7 @@ static bool batch_diag_values(spmv_batch *b, int32_t m, cudaStream_t s) {
     if (launch_sell_relayout(t.d, t.srows, t.n, h->d_rp, h->vk, h->d_val, nullptr, b->d_dvals + b->dval_off[m], nullptr,
                              s) != cudaSuccess)
         return false;
-    b->vals_ver[m] = h->values_version;
+    if (!capture_id(s)) b->vals_ver[m] = h->values_version;
     return true;
 }
 
@@ -1630,7 +1655,7 @@ static spmv_status set_values_impl(spmv_matrix *h, const void *val, spmv_dtype t
     // a row-slice copy that served the last values gets the new ones in the same
     // pass; other copies are laid out again when they are used
     auto f = h->sells.find(h->sigma);
-    const bool fused = h->family == 5 && f != h->sells.end() && f->second.vals_valid && f->second.diagonal &&
+    const bool fused = h->family == 5 && f != h->sells.end() && f->second.laid.on(s) && f->second.diagonal &&
                        sell_tile_fits(h);
     if (fused) {
         const bool prod = y && static_cast<int>(t) == h->vk && !h->sym && !h->d_rmap &&
@@ -1645,18 +1670,19 @@ static spmv_status set_values_impl(spmv_matrix *h, const void *val, spmv_dtype t
     }
     if (h->mirror32) {
         CK(launch_convert(val, t, h->mirror32->d_val, kF32, h->nnz, s));
-        for (auto &kv : h->mirror32->slots) kv.second.vals_valid = false;
-        for (auto &kv : h->mirror32->sells) kv.second.vals_valid = false;
+        for (auto &kv : h->mirror32->slots) kv.second.laid = Laid();
+        for (auto &kv : h->mirror32->sells) kv.second.laid = Laid();
     }
     // captured CG iterations read the copies laid out from the old values: the next
     // solve runs its first iterations plainly, which lays them out again
     h->cg.cg64_key = h->cg.inner32_key = -1;
-    h->valT_valid = false;
+    h->valT = h->full_laid = Laid();
     h->valT_requested = false;
     ++h->values_version;
-    for (auto &kv : h->slots) kv.second.vals_valid = false;
-    for (auto &kv : h->sells) kv.second.vals_valid = false;
-    if (fused) f->second.vals_valid = true;
+    const Laid with = fused ? f->second.laid : Laid();
+    for (auto &kv : h->slots) kv.second.laid = Laid();
+    for (auto &kv : h->sells) kv.second.laid = Laid();
+    if (fused) f->second.laid = with;  // it holds what the CRS copy holds, before and after this call's work
     return SPMV_OK;
 }
 
@@ -2179,17 +2205,17 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
         // pass), and from then on the product runs like a forward product on a
         // slot-major copy of A^T.
         const size_t vb = (h->vk == kF64) ? 8 : 4;
-        if (!h->valT_valid && h->valT_requested && h->nnz > 0) {
+        if (h->valT_requested && h->nnz > 0 && !h->valT.on(s)) {
             if (!h->d_valT && cudaMalloc(&h->d_valT, static_cast<size_t>(h->nnz) * vb) != cudaSuccess) {
                 h->d_valT = nullptr;
                 return SPMV_ERR_ALLOC;
             }
             CK(launch_permute(h->d_val, h->d_perm, h->d_valT, h->nnz, h->vk, s));
-            h->valT_valid = true;
-            for (auto &kv : h->slotsT) kv.second.vals_valid = false;
-            for (auto &kv : h->sellsT) kv.second.vals_valid = false;
+            h->valT.set(s);
+            for (auto &kv : h->slotsT) kv.second.laid = Laid();
+            for (auto &kv : h->sellsT) kv.second.laid = Laid();
         }
-        const bool ind = !h->valT_valid;
+        const bool ind = !h->valT.on(s);
         h->valT_requested = true;
         bool done = false;
         if (ind) {
@@ -2412,7 +2438,7 @@ spmv_status spmv_batched_create(spmv_batch_handle *out, int32_t count, const spm
                                           nullptr) == cudaSuccess;
                 b->vals_ver[m] = mats[m]->values_version;
             }
-            t.vals_valid = true;
+            t.laid.now = true;
         }
         ok = ok && cudaDeviceSynchronize() == cudaSuccess;
         b->h_mats.resize(static_cast<size_t>(count));
@@ -2468,7 +2494,7 @@ spmv_status spmv_batched_create(spmv_batch_handle *out, int32_t count, const spm
                                       b->slots.cols + off * 32 * ES, nullptr) == cudaSuccess;
         }
         ok = ok && cudaDeviceSynchronize() == cudaSuccess;
-        b->slots.vals_valid = true;
+        b->slots.laid.now = true;
         b->h_mats.resize(static_cast<size_t>(count));
         for (int32_t m = 0; m < count; ++m)
             b->h_mats[m] = MatRef{mats[m]->d_rp, mats[m]->d_col, mats[m]->d_val, nullptr, nullptr, nullptr, nullptr};
@@ -2572,7 +2598,7 @@ spmv_status spmv_batched_apply(spmv_batch_handle b, double alpha, const void *co
                 const int64_t nch = b->mixed ? b->slot_cnt[m] : b->slot_off[m + 1] - off;
                 CK(launch_slot_relayout(t.d + off, EG, nch * 32 * EG, b->vk, b->mats[m]->d_val, nullptr,
                                         static_cast<char *>(t.vals) + off * 32 * EG * vb, nullptr, s));
-                b->vals_ver[m] = b->mats[m]->values_version;
+                if (!capture_id(s)) b->vals_ver[m] = b->mats[m]->values_version;
             }
         SlotOps sops;
         if (!b->mixed && !slot_ops_batched(b->vk, acc, b->E, &sops)) return SPMV_ERR_UNSUPPORTED;

@@ -1,0 +1,121 @@
+"""Calls captured right after new values: what the capture records runs with the graph
+only, so a call beside it, before its first run, uses the new values all the same; and
+nothing is built while a stream is captured."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1106_5908_gb300 import workloads as W
+from gpu_util import assert_within, dev, host, need_gpu
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _gpu():
+    need_gpu()
+
+
+def _matrix(kind):
+    if kind == "grid":
+        return W.laplace3d(28)  # 21,952 rows: diagonal slices
+    if kind == "27-point":
+        return W.stencil27(26)
+    return W.hamiltonian_like(20000, seed=4)
+
+
+@pytest.mark.parametrize("kind,plan", [("scattered", None), ("grid", None), ("scattered", (5, 4096)), ("scattered", (6, 9)),
+                                       ("scattered", (0, 15))])
+def test_apply_captured_on_new_values(kind, plan):
+    from paper_1106_5908_gb300 import Matrix
+    A = _matrix(kind)
+    M = Matrix.from_csr(A.row_ptr, A.col_idx, A.val, A.n_cols)
+    if plan:
+        M.set_plan(*plan)
+    x = dev(W.uniform(A.n_cols, 3))
+    y = torch.zeros_like(x)
+    M.apply(x)
+    val = W.uniform(A.nnz, 6)
+    M.set_plan(4, 9)  # leaves the copies of the matrix's own plan behind: they have to be laid out anew
+    M.apply(x)
+    M.set_values(dev(val))
+    if plan or kind == "grid":
+        M.set_plan(*(plan or (5, 4096)))
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        M.apply(x, y)
+        M.apply(x, y, alpha=1.0, beta=1.0)
+    ref, bound = oracle.spmv(A.row_ptr, A.col_idx, val, host(x), with_bound=True)
+    assert_within(host(M.apply(x)), ref, bound, 1e-13, "before the graph's first run")
+    for _ in range(2):
+        g.replay()
+        assert_within(host(y), 2 * ref, 3 * bound, 1e-13, "replayed")
+    assert_within(host(M.apply(x)), ref, bound, 1e-13, "after the graph")
+
+
+@pytest.mark.parametrize("applies", [0, 1, 2])
+def test_symmetric_apply_captured_on_new_values(applies):
+    from paper_1106_5908_gb300 import Matrix
+    U = W.random_symmetric_upper(20000, seed=5, max_len=9)
+    M = Matrix.from_symmetric_upper(U.row_ptr, U.col_idx, U.val)
+    x = dev(W.uniform(U.n_rows, 3))
+    y = torch.zeros_like(x)
+    M.apply(x)
+    val = W.uniform(U.nnz, 6)
+    M.set_values(dev(val))
+    for _ in range(applies):
+        M.apply(x)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        M.apply(x, y)
+    ref, bound = oracle.spmv_sym(U.row_ptr, U.col_idx, val, host(x), with_bound=True)
+    for _ in range(3):
+        assert_within(host(M.apply(x)), ref, bound, 1e-13, "before the graph's first run")
+    y.zero_()
+    g.replay()
+    assert_within(host(y), ref, bound, 1e-13, "replayed")
+    assert_within(host(M.apply(x)), ref, bound, 1e-13, "after the graph")
+
+
+@pytest.mark.parametrize("kind", ["27-point", "scattered"])
+@pytest.mark.parametrize("new_values", [False, True])
+def test_reverse_pass_captured(kind, new_values):
+    """The reverse passes build copies of A^T on the way; captured, they take what is
+    there, with the values laid out once more by the next pass beside the graph."""
+    from paper_1106_5908_gb300 import Matrix
+    A = _matrix(kind)
+    M = Matrix.from_csr(A.row_ptr, A.col_idx, A.val, A.n_cols)
+    x, g = dev(W.uniform(A.n_cols, 3)), dev(W.uniform(A.n_rows, 4))
+    M.backward(g, x)
+    M.backward(g, x)
+    val, vd = A.val, dev(W.uniform(A.nnz, 8))
+    torch.cuda.synchronize()
+    if new_values:
+        val = host(vd)
+        M.set_values(vd)
+        M.backward(g, x)
+        torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        gx, gv = M.backward(g, x)
+        if not new_values:  # and a first pass on values set in the graph
+            M.set_values(vd)
+            gx2, gv2 = M.backward(g, x)
+    T = oracle.transpose(A.row_ptr, A.col_idx, A.n_cols)
+
+    def check(got, v, what):
+        ref, bound = oracle.spmv(T[0], T[1], v[T[2]], host(g), with_bound=True)
+        assert_within(host(got[0]), ref, bound, 1e-13, what)
+        rows = np.repeat(np.arange(A.n_rows), np.diff(A.row_ptr.astype(np.int64)))
+        assert np.array_equal(host(got[1]), host(g)[rows] * host(x)[A.col_idx]), what
+
+    check(M.backward(g, x), val, "before the graph's first run")
+    graph.replay()
+    check((gx, gv), val, "replayed")
+    if not new_values:
+        check((gx2, gv2), host(vd), "replayed, new values")
+    M.set_values(vd)
+    check(M.backward(g, x), host(vd), "after the graph")
