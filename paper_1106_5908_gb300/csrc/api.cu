@@ -1781,47 +1781,26 @@ spmv_status spmv_row_histogram(spmv_handle h, int32_t nbins, int64_t *counts) {
 
 spmv_status spmv_set_plan(spmv_handle h, int32_t family, int32_t param) {
     if (!h || family < 0 || family > 6) return SPMV_ERR_INVALID_ARG;
-    h->sell_if_diag = false;
+    // a refused parameter leaves the handle as it was
+    const bool f64 = h->vk == kF64;
+    bool ok = param == 0;
+    switch (family) {
+        case 0: ok = ok || param == 7 || param == 8 || param == 15 || param == 16; break;
+        case 1: ok = ok || (param >= 1 && param <= 32 && !(param & (param - 1))); break;
+        case 2: ok = ok || (param >= 3 && param <= 31 && param % 2 != 0); break;
+        case 3: ok = ok || param == 7 || param == 11 || param == 15; break;
+        case 4: ok = ok || param == 7 || param == 9 || param == 11 || param == 15; break;
+        case 5: ok = ok || (param >= 32 && param <= (1 << 20) && !(param & (param - 1))); break;
+        default: ok = ok || param == 9 || param == (f64 ? 7 : 15); break;
+    }
+    if (!ok) return SPMV_ERR_INVALID_ARG;
+    constexpr int kDefaultE[7] = {16, 0, 15, 7, 9, 0, 9};
+    h->family = family;
     h->planned = true;
-    if (family == 6) {
-        const bool f64 = h->vk == kF64;
-        if (param != 0 && !(f64 ? (param == 7 || param == 9) : (param == 9 || param == 15)))
-            return SPMV_ERR_INVALID_ARG;
-        h->family = 6;
-        h->E = param ? param : 9;
-        return SPMV_OK;
-    }
-    if (family == 5) {
-        if (param != 0 && (param < 32 || param > (1 << 20) || (param & (param - 1)))) return SPMV_ERR_INVALID_ARG;
-        h->family = 5;
-        h->sigma = param ? param : 4096;
-        return SPMV_OK;
-    }
-    if (family == 4) {
-        if (param != 0 && param != 7 && param != 9 && param != 11 && param != 15) return SPMV_ERR_INVALID_ARG;
-        h->family = 4;
-        h->E = param ? param : (h->vk == kF32 ? 15 : 9);
-        return SPMV_OK;
-    }
-    if (family == 3) {
-        if (param != 0 && param != 7 && param != 11 && param != 15) return SPMV_ERR_INVALID_ARG;
-        h->family = 3;
-        h->E = param ? param : 7;
-        return SPMV_OK;
-    }
-    if (family == 0) {
-        if (param != 0 && param != 7 && param != 8 && param != 15 && param != 16) return SPMV_ERR_INVALID_ARG;
-        h->family = 0;
-        h->E = param ? param : 16;
-    } else if (family == 2) {
-        if (param != 0 && (param < 3 || param > 31 || param % 2 == 0)) return SPMV_ERR_INVALID_ARG;
-        h->family = 2;
-        h->E = param ? param : 15;
-    } else {
-        if (param != 0 && (param < 1 || param > 32 || (param & (param - 1)))) return SPMV_ERR_INVALID_ARG;
-        h->family = 1;
-        if (param) h->T = param;
-    }
+    h->sell_if_diag = false;
+    if (family == 5) h->sigma = param ? param : 4096;
+    else if (family == 1) h->T = param ? param : h->T;
+    else h->E = param ? param : (family == 4 && !f64 ? 15 : kDefaultE[family]);
     return SPMV_OK;
 }
 
