@@ -1124,16 +1124,33 @@ spmv_status prepare_run(spmv_matrix *h, int xk, int yk, int R, int E, bool trans
     return SPMV_OK;
 }
 
+// A plan taken for its diagonal slices only (sell_if_diag), from a sample of the rows,
+// is settled when the slices are known: too few diagonal ones, and the handle runs on
+// the slot-major kernel and gives the copy back, unless other calls had built it.
+void settle_plan(spmv_matrix *h, cudaStream_t s) {
+    if (!h->sell_if_diag) return;
+    const bool had = h->sells.count(h->sigma) != 0;
+    const SellTable *t = get_sell(h, h->sigma, s, false, false);
+    if (!t) return;  // not built now: asked again by the next call
+    h->sell_if_diag = false;
+    if (t->diagonal) return;
+    h->family = 4;  // E as the tuner chose it
+    if (had) return;
+    free_sell(h->sells[h->sigma]);
+    h->sells.erase(h->sigma);
+}
+
 // The row-slice launch of h for these operands (plan family 5, no row map):
 // its compiled configuration and parameters, with the slice copy built on first
 // use; false when h does not run on the row slices here.
 bool sell_launch_of(spmv_matrix *h, double alpha, const void *x, int xk, double beta, void *y, int yk,
                     cudaStream_t s, SellOps *ops, SellParams *lp) {
     if (h->family != 5 || h->d_rmap) return false;
+    settle_plan(h, s);
+    if (h->family != 5 || h->sell_if_diag) return false;
     const int acc = (h->vk == kF32) ? h->acc32 : kAccF64;
     SellTable *lt = nullptr;
     if (!sell_ops(h->vk, xk, yk, acc, ops, h->max_row) || (lt = get_sell(h, h->sigma, s)) == nullptr) return false;
-    if (h->sell_if_diag && !lt->diagonal) return false;  // few diagonal slices after all: the slot-major kernel
     *lp = sell_params(*lt, MatRef{h->d_rp, h->d_col, h->d_val, nullptr, x, y, nullptr}, alpha, beta);
     return true;
 }
@@ -1332,8 +1349,10 @@ static spmv_status cg_in_one_kernel(spmv_matrix *h, CgWork &w, const void *b, vo
         return SPMV_ERR_UNSUPPORTED;
     const int32_t few = (h->n_rows + kSellC - 1) / kSellC;  // at least this many slices
     if (!cg_kernel_fits(h->vk, few, h->max_row)) return SPMV_ERR_UNSUPPORTED;
-    SellTable *t = get_sell(h, kSellSigma, s);
-    if (!t || !t->diagonal || t->n_long > 0 || !cg_kernel_fits(h->vk, t->n, h->max_row)) return SPMV_ERR_UNSUPPORTED;
+    SellTable *t = get_sell(h, kSellSigma, s, false, false);
+    if (!t || !t->diagonal || t->n_long > 0 || !cg_kernel_fits(h->vk, t->n, h->max_row) ||
+        !(t = get_sell(h, kSellSigma, s)))
+        return SPMV_ERR_UNSUPPORTED;
     const SellParams p =
         sell_params(*t, MatRef{h->d_rp, h->d_col, h->d_val, nullptr, nullptr, nullptr, nullptr}, 1.0, 0.0);
     double *out = w.one + 4 * static_cast<int64_t>(w.one_ctas);
@@ -1714,6 +1733,7 @@ spmv_status spmv_get_info(spmv_handle h, int32_t *n_rows, int32_t *n_cols, int64
     if (nnz) *nnz = h->nnz;
     if (plan) {
         DeviceGuard g(h->device);
+        settle_plan(h, nullptr);
         const int acc = (h->vk == kF32) ? h->acc32 : kAccF64;
         int32_t E = h->E, nunits = 0, rowcap = 0, nlong = 0, threads = 256;
         if (h->family == 2) {
