@@ -296,7 +296,8 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const CgParams q) {
         if (d.w >= 0 && lane < (d.y + 3) / 4) s_dg[own * ndg + lane] = __ldg(q.diag + d.w + lane);
         const int i = l * 32 + lane;
         s_row[i] = row;
-        const T b = row >= 0 ? __ldg(static_cast<const T *>(q.b) + row) : T(0);
+        // an ordinary load: b may be r, which this kernel writes
+        const T b = row >= 0 ? static_cast<const T *>(q.b)[row] : T(0);
         if constexpr (XG) {
             if (row >= 0) x[row] = T(0);
         } else {

@@ -1,0 +1,21 @@
+"""Rules of the one-kernel CG that no result shows reliably, read from its source."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1106_5908_gb300", "csrc")
+
+
+def _source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def test_vectors_never_through_the_read_only_path():
+    """The kernel writes p, p2, r and x, and b may be r: none of them is loaded by __ldg,
+    whose lines nothing invalidates while the kernel runs."""
+    args = re.findall(r"__ldg\(((?:[^()]|\([^()]*\)|\((?:[^()]|\([^()]*\))*\))*)\)", _source("k_cg.cu"))
+    assert len(args) > 5
+    for arg in args:
+        assert re.match(r"(q\.(order|srows|diag)|cb|m\.(rp|col)|src|static_cast<const T \*>\(m\.vs\))(\W|$)", arg.strip()), arg
+    # src is a row of the matrix values
+    assert re.search(r"const T \*src = vals \+", _source("k_cg.cu"))
