@@ -227,8 +227,9 @@ __device__ __forceinline__ T cg_result(const ACC &a, const MatRef &m, int row, c
     }
 }
 
-// Thread sums of products: FP64 FMAs, or float-float for FP32 vectors (off the
-// FP64 pipe; out of FP32's range the caller sums the thread's terms again).
+// Thread sums of r.r: FP64 FMAs, or float-float for FP32 vectors, as the vector kernels
+// of the other path (off the FP64 pipe; out of FP32's range the caller sums the thread's
+// terms again).
 template <typename T> struct DotAcc { using type = AccF64; };
 template <> struct DotAcc<float> { using type = AccFF; };
 __device__ __forceinline__ bool dot_poisoned(const AccF64 &) { return false; }
@@ -323,8 +324,8 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const CgParams q) {
     while (ok && it < q.max_iter && sqrt(rho) > q.tol * sqrt(bb)) {
         const int stop = min(q.max_iter, it + kCgCheckEvery);
         for (; ok && it < stop; ++it) {
-            // q = A p, p.q
-            Dot pq;
+            // q = A p, p.q (in FP64, of exact products for FP32 vectors too)
+            AccF64 pq;
             pq.zero();
             const CgVec<FUSE, T> pv{p, r, be};
             for (int l = warp; l < cnt; l += nw) {
@@ -349,16 +350,8 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const CgParams q) {
                     pq.fma(pr, y);
                 }
             }
-            double t = pq.get();
-            if (dot_poisoned(pq)) {
-                t = 0.0;
-                for (int l = warp; l < cnt; l += nw) {
-                    const int i = l * 32 + lane, row = s_row[i];
-                    if (row >= 0) t = fma(widen(FUSE ? s_p[i] : p[row]), widen(s_q[i]), t);
-                }
-            }
             double tot;
-            ok = grid.sum<false>(t, [rho](double pq) { return pq != 0.0 ? rho / pq : 0.0; }, &tot, &step);
+            ok = grid.sum<false>(pq.get(), [rho](double pq) { return pq != 0.0 ? rho / pq : 0.0; }, &tot, &step);
             if (!ok) break;
             // x += alpha p, r -= alpha q, r.r (a zero direction takes no step)
             const T a = step_scale(step, static_cast<T *>(nullptr));
@@ -376,7 +369,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const CgParams q) {
                     rr.fma(ri, ri);
                 }
             }
-            t = rr.get();
+            double t = rr.get();
             if (dot_poisoned(rr)) {
                 t = 0.0;
                 for (int l = warp; l < cnt; l += nw) {

@@ -19,3 +19,11 @@ def test_vectors_never_through_the_read_only_path():
         assert re.match(r"(q\.(order|srows|diag)|cb|m\.(rp|col)|src|static_cast<const T \*>\(m\.vs\))(\W|$)", arg.strip()), arg
     # src is a row of the matrix values
     assert re.search(r"const T \*src = vals \+", _source("k_cg.cu"))
+
+
+def test_step_length_summed_in_fp64():
+    """p.q is summed by FP64 FMAs of exact products whatever the vectors' type, as the
+    product kernels that fuse it do."""
+    src = _source("k_cg.cu")
+    assert re.search(r"\bAccF64 pq;", src) and "pq.fma(pr, y)" in src
+    assert "dsum = fma(widen(__ldg(x + r)), widen(q), dsum)" in _source("sell_kernel.cuh")
