@@ -1340,6 +1340,8 @@ spmv_status ensure_mirror32(spmv_matrix *h, cudaStream_t s) {
 // CG on h as one cooperative kernel (launch_cg), when h runs on diagonal row slices
 // (by the tuner, whatever its size) and the vectors of a CTA's rows fit in shared
 // memory.  res: rho, iterations, b.b.  SPMV_ERR_UNSUPPORTED: not this matrix.
+// SPMV_ERR_TIMEOUT: a grid barrier gave up (the GPU taken away for a second between two
+// barriers), and x, dir, dir2 and r are void; the callers solve on the other path then.
 // work: the CG work array of the handle that runs the solve (its partials).
 static spmv_status cg_in_one_kernel(spmv_matrix *h, CgWork &w, const void *b, void *x, void *dir, void *dir2, void *r,
                                     double tol, int32_t max_iter, double *res, cudaStream_t s) {
@@ -1356,7 +1358,7 @@ static spmv_status cg_in_one_kernel(spmv_matrix *h, CgWork &w, const void *b, vo
     const SellParams p =
         sell_params(*t, MatRef{h->d_rp, h->d_col, h->d_val, nullptr, nullptr, nullptr, nullptr}, 1.0, 0.0);
     double *out = w.one + 4 * static_cast<int64_t>(w.one_ctas);
-    if (launch_cg(p, t->dtmp, h->vk, h->max_row, b, x, dir, dir2, r, tol, max_iter, w.one, out, h->d_err, s) != cudaSuccess) {
+    if (launch_cg(p, t->dtmp, h->vk, h->max_row, b, x, dir, dir2, r, tol, max_iter, w.one, out, s) != cudaSuccess) {
         (void)cudaGetLastError();  // not launched: the kernel-by-kernel path runs
         return SPMV_ERR_UNSUPPORTED;
     }
@@ -2748,7 +2750,7 @@ spmv_status spmv_cg(spmv_handle h, const double *b, double *x, double tol, int32
     int32_t it = 0;
     double one[3];
     st = cg_in_one_kernel(h, w, b, x, w.p64, w.q64, w.r64, tol, max_iter, one, s);
-    if (st != SPMV_OK && st != SPMV_ERR_UNSUPPORTED) return st;
+    if (st != SPMV_OK && st != SPMV_ERR_UNSUPPORTED && st != SPMV_ERR_TIMEOUT) return st;
     const bool solved = st == SPMV_OK;
     if (solved) {
         rho = one[0];
@@ -2848,7 +2850,7 @@ spmv_status spmv_ir_cg(spmv_handle h, const double *b, double *x, double outer_t
     int32_t outer = 0;
     int64_t inner_total = 0;
     double relres = 0.0;
-    bool converged = false;
+    bool converged = false, one_kernel = true;
     for (;;) {
         // outer (FP64): r = b - A x, ||r||
         CK(cudaMemcpyAsync(w.r64, b, static_cast<size_t>(n) * 8, cudaMemcpyDeviceToDevice, s));
@@ -2864,14 +2866,20 @@ spmv_status spmv_ir_cg(spmv_handle h, const double *b, double *x, double outer_t
         // inner (FP32 storage): CG on A d = r / ||r||
         CK(cg_scale_to32(w.r64, w.r32, 1.0 / rnorm, n, s));
         double one[3];
-        st = cg_in_one_kernel(A32, w, w.r32, w.d32, w.p32, w.q32, w.r32, inner_tol, max_inner, one, s);
+        st = one_kernel ? cg_in_one_kernel(A32, w, w.r32, w.d32, w.p32, w.q32, w.r32, inner_tol, max_inner, one, s)
+                        : SPMV_ERR_UNSUPPORTED;
         if (st == SPMV_OK) {
             inner_total += static_cast<int32_t>(one[1]);
             CK(cg_axpy_64_32(x, w.d32, rnorm, n, s));
             ++outer;
             continue;
         }
-        if (st != SPMV_ERR_UNSUPPORTED) return st;
+        if (st == SPMV_ERR_TIMEOUT) {  // no second wait in this call
+            one_kernel = false;
+            CK(cg_scale_to32(w.r64, w.r32, 1.0 / rnorm, n, s));
+        } else if (st != SPMV_ERR_UNSUPPORTED) {
+            return st;
+        }
         CK(cudaMemsetAsync(w.d32, 0, static_cast<size_t>(n) * 4, s));
         CK(cudaMemcpyAsync(w.p32, w.r32, static_cast<size_t>(n) * 4, cudaMemcpyDeviceToDevice, s));
         CK(cg_dot(w.r32, kF32, w.r32, kF32, n, w.partials, w.sc, kOpStore, kScRho, s));

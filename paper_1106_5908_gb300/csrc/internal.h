@@ -139,11 +139,12 @@ cudaError_t launch_sell_grad_val(const SellParams &p, int vk, const void *g, voi
 // widest slice), tested for ||r|| <= tol*||b|| every kCgCheckEvery iterations.
 // vk: kind of the values and vectors; dir, dir2, r: n entries of scratch each (r may
 // be b, which is then overwritten); work: 4 * SMs
-// doubles, 16-byte aligned; out (4 doubles): r.r, iterations, b.b, 1 after a barrier timed out.
+// doubles, 16-byte aligned; out (4 doubles): r.r, iterations, b.b, 1 after a barrier timed
+// out (the GPU taken away for a second between two barriers): x, dir and r are then void.
 constexpr int32_t kCgCheckEvery = 8;
 bool cg_kernel_fits(int vk, int32_t n_slices, int max_w);
 cudaError_t launch_cg(const SellParams &p, const int4 *order, int vk, int max_w, const void *b, void *x, void *dir,
-                      void *dir2, void *r, double tol, int32_t max_iter, double *work, double *out, int32_t *err, cudaStream_t s);
+                      void *dir2, void *r, double tol, int32_t max_iter, double *work, double *out, cudaStream_t s);
 
 cudaError_t launch_rowvec(const KParams &p, const int32_t n_rows, int vk, int xk, int yk, int acc,
                           int T, cudaStream_t s);

@@ -257,7 +257,6 @@ struct CgParams {
     double *out;            // rho, iterations, b.b, 1 after a timeout
     double tol;
     int32_t max_iter;
-    int32_t *err;
 };
 
 // VSM: the matrix values are kept in shared memory too.  FUSE: two barriers (above).
@@ -402,15 +401,12 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const CgParams q) {
         }
     }
     if (threadIdx.x == 0) {
-        if (!ok) set_error(q.err, kDevErrTimeout);
-        if (blockIdx.x == 0 || !ok) {
-            if (ok) {
-                q.out[0] = rho;
-                q.out[1] = it;
-                q.out[2] = bb;
-            } else {
-                q.out[3] = 1.0;
-            }
+        if (!ok) {
+            q.out[3] = 1.0;
+        } else if (blockIdx.x == 0) {
+            q.out[0] = rho;
+            q.out[1] = it;
+            q.out[2] = bb;
         }
     }
 }
@@ -483,7 +479,7 @@ bool cg_kernel_fits(int vk, int32_t n_slices, int max_w) {
 }
 
 cudaError_t launch_cg(const SellParams &p, const int4 *order, int vk, int max_w, const void *b, void *x, void *dir,
-                      void *dir2, void *r, double tol, int32_t max_iter, double *work, double *out, int32_t *err, cudaStream_t s) {
+                      void *dir2, void *r, double tol, int32_t max_iter, double *work, double *out, cudaStream_t s) {
     CgPlan pl;
     if (!cg_plan(vk, 2 * p.n_slices, max_w, &pl)) return cudaErrorInvalidConfiguration;
     CgParams q{};
@@ -505,7 +501,6 @@ cudaError_t launch_cg(const SellParams &p, const int4 *order, int vk, int max_w,
     q.out = out;
     q.tol = tol;
     q.max_iter = max_iter;
-    q.err = err;
     cudaError_t e = cudaMemsetAsync(work, 0xff, 4 * sizeof(*q.slots) * pl.grid, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(out, 0, 4 * sizeof(double), s);
     if (e != cudaSuccess) return e;

@@ -27,3 +27,17 @@ def test_step_length_summed_in_fp64():
     src = _source("k_cg.cu")
     assert re.search(r"\bAccF64 pq;", src) and "pq.fma(pr, y)" in src
     assert "dsum = fma(widen(__ldg(x + r)), widen(q), dsum)" in _source("sell_kernel.cuh")
+
+
+def test_timeouts_are_solved_on_the_other_path():
+    """A grid barrier that gave up ends neither solver: both go on to the kernel-by-kernel
+    path (the mixed one with its right-hand side formed anew), and the kernel leaves no
+    error word behind."""
+    src = _source("api.cu")
+    calls = [m.end() for m in re.finditer(r"st = (?:one_kernel \? )?cg_in_one_kernel\(", src)]
+    assert len(calls) == 2
+    plain, mixed = (src[c:c + 900] for c in calls)
+    assert "st != SPMV_ERR_UNSUPPORTED && st != SPMV_ERR_TIMEOUT) return st;" in plain
+    retry = mixed[mixed.index("if (st == SPMV_ERR_TIMEOUT)"):]
+    assert "cg_scale_to32(w.r64, w.r32" in retry[:retry.index("}")]
+    assert "set_error" not in _source("k_cg.cu")
