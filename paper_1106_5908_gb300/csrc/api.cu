@@ -631,6 +631,8 @@ constexpr int32_t kBatchDiagMinSize = 32768;
 
 // Share of far entries (column_randomness) above which columns count as scattered.
 constexpr double kScattered = 0.25;
+// Rows from which 2 or 3 right-hand sides run on the row slices (spmm_apply).
+constexpr int32_t kRhsFew = 65536, kRhsFewScattered = 262144;
 
 // slices = false: the row slices are not considered (their padding is not counted).
 void autotune(spmv_matrix *h, bool slices = true) {
@@ -2140,26 +2142,37 @@ spmv_status spmm_apply(spmv_handle h, int32_t nrhs, double alpha, const void *X,
     // rows of X between its reads either way (Hamiltonian-like: 4.2 M rows, X 134
     // MB, 461 against 478 us; 300,000 rows 50 against 36; 27-point 101^3 192
     // against 194, 5-point 1400^2 74 against 80).
+    // Not for 2 or 3 right-hand sides on few rows: a warp then walks 16 or 32 whole rows
+    // at the latency of its loads, where the tile kernel cuts the entries evenly (3:
+    // 27-point 25^3 15.7 against 7.9 us, 32^3 17.6 / 13.9, 40^3 17.6 / 21.3; scattered
+    // 30,000 rows 13.1 / 8.2, 130,000 23.0 / 22.1, 260,000 30.7 / 39.7).
+    // Nor with rows outside the slices (long_row): one warp and its lane groups walk
+    // such a row, which the tile kernel gives a CTA (3,000 rows, 3 of them of 1,500
+    // entries: 3 right-hand sides 47 against 10 us, 32 468 against 164).  Groups of 4
+    // stay on k_sell_mr there, whose 32 lanes share the row, while X fits in L2.
     int l2 = 0;
     cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, h->device);
     const bool scattered = h->col_random > kScattered;
+    const bool long_rows = h->max_row > kSellLongRow;
+    const double x_bytes = static_cast<double>(h->n_cols) * nrhs * 8.0;
+    const bool slices = nrhs < kSellR ? !long_rows && h->n_rows >= (scattered ? kRhsFewScattered : kRhsFew)
+                                      : !long_rows || !scattered || x_bytes <= 1.25 * l2;
     SellTable *t = nullptr;
-    if (h->sell_pad <= kSellMaxPadding && (t = get_sell(h, kSellSigma, s)) != nullptr) {
+    if (slices && h->sell_pad <= kSellMaxPadding && (t = get_sell(h, kSellSigma, s)) != nullptr) {
         const bool vec = (nrhs % 2 == 0) && (reinterpret_cast<uintptr_t>(X) % 16 == 0) &&
                          (reinterpret_cast<uintptr_t>(Y) % 16 == 0);
         const SellParams b =
             sell_params(*t, MatRef{h->d_rp, h->d_col, h->d_val, nullptr, nullptr, nullptr, nullptr}, alpha, beta);
         const double *Xd = static_cast<const double *>(X);
         double *Yd = static_cast<double *>(Y);
-        if (nrhs == kSellR && (!scattered || static_cast<double>(h->n_cols) * nrhs * 8.0 > 0.5 * l2)) {
-            CK(launch_sell_mr(b, Xd, Yd, nrhs, nrhs, vec, s));
-            return SPMV_OK;
+        if (long_rows || (nrhs == kSellR && (!scattered || x_bytes > 0.5 * l2))) {
+            for (; c0 + kSellR <= nrhs; c0 += kSellR) CK(launch_sell_mr(b, Xd + c0, Yd + c0, nrhs, nrhs, vec, s));
+        } else {
+            for (; c0 < nrhs; c0 += kSellMaxRhs)
+                CK(launch_sell_rhs(b, Xd + c0, Yd + c0, nrhs, nrhs, std::min(kSellMaxRhs, nrhs - c0), vec, scattered, s));
         }
-        for (; c0 < nrhs; c0 += kSellMaxRhs)
-            CK(launch_sell_rhs(b, Xd + c0, Yd + c0, nrhs, nrhs, std::min(kSellMaxRhs, nrhs - c0), vec, scattered, s));
-        return SPMV_OK;
     }
-    // without the slices: the tile kernel, up to 32 per launch
+    // what is left (all of it without the slices): the tile kernel, up to 32 per launch
     for (; c0 < nrhs; c0 += 32) {
         const int cnt = std::min(32, nrhs - c0);
         int R = 2;

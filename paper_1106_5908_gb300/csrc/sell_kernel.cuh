@@ -786,7 +786,8 @@ __global__ void __launch_bounds__(256, 2) k_sell_mr(const SellMrParams q) {
 // per SM) keep the FP64 pipe, which bounds it, busy: Hamiltonian-like 4.2 M rows, 16
 // and 32 right-hand sides 1,530 and 3,105 us (2,107 and 4,063 on the tile kernel; one
 // FMA per entry and right-hand side takes 1,448 and 2,896), 5-point 1400^2 280 and 552
-// (594 and 1,315; 262 and 524), 27-point 101^3, 5: 253 (371; 228).  VEC: the rows of X and Y allow 16-byte accesses (R
+// (594 and 1,315; 262 and 524), 27-point 101^3, 5: 253 (371; 228).  Every row lies in a
+// slice (no long rows).  VEC: the rows of X and Y allow 16-byte accesses (R
 // even); otherwise the right-hand sides are loaded one by one and the last lane of a
 // group may hold fewer than V.
 // ---------------------------------------------------------------------------
@@ -850,43 +851,22 @@ __global__ void __launch_bounds__(512, 2) k_sell_rhs(const SellRhsParams q) {
 #pragma unroll
         for (int r = 0; r < V; ++r) acc[r] = 0.0;
         int row = -1;
-        if (d.y < 0) {
-            // a long row: the groups stride its entries, group 0 sums them in order
-            if (b) continue;
-            const int k1 = __ldg(p.m.rp + d.x + 1);
-            if (g < G)
-                for (int k = __ldg(p.m.rp + d.x) + g; k < k1; k += G) {
-                    const double v = __ldg(static_cast<const double *>(p.m.vs) + k);
-                    const double *xp = X + static_cast<int64_t>(__ldg(p.m.col + k)) * ldx;
-#pragma unroll
-                    for (int r = 0; r < V; ++r)
-                        if (r < nv) acc[r] = fma(v, __ldg(xp + r), acc[r]);
-                }
-            for (int o = 1; o < G; ++o)
-#pragma unroll
-                for (int r = 0; r < V; ++r) {
-                    const double t = __shfl_sync(0xffffffffu, acc[r], (lane + o * L) & 31);
-                    if (g == 0) acc[r] += t;
-                }
-            if (g == 0) row = d.x;
-        } else {
-            const int i = b * G + g;
-            const bool ok = g < G && i < C;
-            const int64_t base = static_cast<int64_t>(d.x) * C + (ok ? i : 0);
-            if (ok) row = __ldg(p.srows + static_cast<int64_t>(s) * C + i);
-            const double *__restrict__ vb = vals + base;
-            const int32_t *__restrict__ cb = p.cols + base;
-            constexpr int B = V <= 4 ? 4 : V <= 5 ? 3 : 2;  // slot rows in flight (registers)
-            int w = d.y;
-            for (; w >= B; w -= B) {
-                sell_rhs_block<B, V, VEC>(acc, vb, cb, X, ldx, nv);
-                vb += B * C;
-                cb += B * C;
-            }
-            if (B > 3 && w == 3) sell_rhs_block<3, V, VEC>(acc, vb, cb, X, ldx, nv);
-            else if (B > 2 && w == 2) sell_rhs_block<2, V, VEC>(acc, vb, cb, X, ldx, nv);
-            else if (w == 1) sell_rhs_block<1, V, VEC>(acc, vb, cb, X, ldx, nv);
+        const int i = b * G + g;
+        const bool ok = g < G && i < C;
+        const int64_t base = static_cast<int64_t>(d.x) * C + (ok ? i : 0);
+        if (ok) row = __ldg(p.srows + static_cast<int64_t>(s) * C + i);
+        const double *__restrict__ vb = vals + base;
+        const int32_t *__restrict__ cb = p.cols + base;
+        constexpr int B = V <= 4 ? 4 : V <= 5 ? 3 : 2;  // slot rows in flight (registers)
+        int w = d.y;
+        for (; w >= B; w -= B) {
+            sell_rhs_block<B, V, VEC>(acc, vb, cb, X, ldx, nv);
+            vb += B * C;
+            cb += B * C;
         }
+        if (B > 3 && w == 3) sell_rhs_block<3, V, VEC>(acc, vb, cb, X, ldx, nv);
+        else if (B > 2 && w == 2) sell_rhs_block<2, V, VEC>(acc, vb, cb, X, ldx, nv);
+        else if (w == 1) sell_rhs_block<1, V, VEC>(acc, vb, cb, X, ldx, nv);
         if (row >= 0 && nv > 0) {
             double *yp = q.m.Y + static_cast<int64_t>(row) * ldy + c;
 #pragma unroll
