@@ -141,6 +141,7 @@ struct SellTable {
     int32_t n_long = 0;
     int64_t slot_rows = 0;
     Laid laid;
+    bool read = false;          // something has read the values since the last new ones
     // diagonal slices: descriptors with each slice's place in diag (in slice order
     // and in launch order), and the diagonals of the slot rows, padded to 4 per slice
     // (behind cols)
@@ -928,6 +929,7 @@ SellTable *get_sell(spmv_matrix *h, int32_t sigma, cudaStream_t s, bool transpos
             return nullptr;
         t.laid.set(s);
     }
+    t.read = t.read || need_vals;
     return &t;
 }
 
@@ -1675,18 +1677,21 @@ void spmv_destroy(spmv_handle h) { destroy_matrix(h); }
 static spmv_status set_values_impl(spmv_matrix *h, const void *val, spmv_dtype t, double alpha, const void *x, void *y,
                                    bool *applied, cudaStream_t s) {
     if (h->nnz == 0) return SPMV_OK;
-    // a row-slice copy that served the last values gets the new ones in the same
-    // pass; other copies are laid out again when they are used
+    // a row-slice copy that served the last values, or serves this product, gets the new
+    // ones in the same pass (27-point 128^3: 226 us where the CRS copy alone takes 136);
+    // other copies are laid out again when they are used
     auto f = h->sells.find(h->sigma);
-    const bool fused = h->family == 5 && f != h->sells.end() && f->second.laid.on(s) && f->second.diagonal &&
-                       sell_tile_fits(h);
+    const bool slices = h->family == 5 && f != h->sells.end() && f->second.laid.on(s) && f->second.diagonal &&
+                        sell_tile_fits(h);
+    const bool prod = slices && y && static_cast<int>(t) == h->vk && !h->sym && !h->d_rmap &&
+                      (h->vk == kF64 || h->acc32 == kAccFF);
+    const bool fused = slices && (prod || f->second.read);
     if (fused) {
-        const bool prod = y && static_cast<int>(t) == h->vk && !h->sym && !h->d_rmap &&
-                          (h->vk == kF64 || h->acc32 == kAccFF);
         const SellParams p = sell_params(
             f->second, MatRef{h->d_rp, h->d_col, prod ? val : nullptr, nullptr, prod ? x : nullptr, prod ? y : nullptr, nullptr},
             alpha, 0.0);
         CK(launch_sell_set_values(p, val, t, h->d_val, h->vk, h->max_row, s));
+        f->second.read = prod;
         if (applied) *applied = prod;
     } else {
         CK(launch_convert(val, t, h->d_val, h->vk, h->nnz, s));
@@ -2234,12 +2239,19 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
         bool done = false;
         if (ind) {
             // new values on diagonal slices: the slices of A^T read them where A's
-            // slices hold them
+            // slices hold them.  With rows of up to 8 entries on average only when a
+            // product has laid them out there: doing it for this pass alone costs what
+            // the pass then saves (new values and a reverse pass: 7-point 160^3 290
+            // against 257 us through the permutation, 5-point 2000^2 210 / 195; 27-point
+            // 128^3 500 against 606)
             SellOps lops;
             const int acc = (h->vk == kF32) ? kAccFF : kAccF64;
             const SellTable *t = nullptr, *a = nullptr;
-            if (sell_ops(h->vk, h->vk, h->vk, acc, &lops) && (t = get_sell_positions(h, s)) != nullptr &&
-                (a = get_sell(h, h->sigma, s)) != nullptr) {
+            if (sell_ops(h->vk, h->vk, h->vk, acc, &lops) && (t = get_sell_positions(h, s)) != nullptr) {
+                const SellTable &own = h->sells.at(h->sigma);
+                a = h->nnz > 8LL * h->n_rows ? get_sell(h, h->sigma, s) : own.vals && own.laid.on(s) ? &own : nullptr;
+            }
+            if (a) {
                 SellParams lp =
                     sell_params(*t, MatRef{h->d_rowT, h->d_colT, h->d_perm, h->d_val, g, grad_x, nullptr}, alpha, 0.0);
                 lp.vals = a->vals;
