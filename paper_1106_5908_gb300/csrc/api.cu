@@ -119,6 +119,7 @@ struct Laid {
 
 // Slot-major copy of a matrix for plan family 4 (per entries-per-lane E).
 struct SlotTable {
+    void *block = nullptr;      // one allocation that holds the four arrays (a handle's own copy)
     ChunkDesc *d = nullptr;
     uint32_t *lmask = nullptr;  // 32 words per chunk
     void *vals = nullptr;       // n * 32E values, slot-major
@@ -226,53 +227,69 @@ void free_chunks(ChunkTable &ct) {
 // the chunk's first entry itself (no alignment), with one word per lane: the row
 // starts in its E slots (bits 0..E-1), the rows starting before them (bits
 // kSlotPreShift..) and whether its last slot ends a row or the chunk (kSlotEnds).
-void make_slot_chunks(const int32_t *rp, int32_t n_rows, int E, std::vector<ChunkDesc> &out,
-                      std::vector<uint32_t> &lmask, int32_t *n_long, int32_t *n_empty) {
-    const int64_t SL = 32LL * E;
+template <int E>
+void make_slot_chunks_of(const int32_t *rp, int32_t n_rows, std::vector<ChunkDesc> &out, std::vector<uint32_t> &lmask,
+                         int32_t *n_long, int32_t *n_empty) {
+    constexpr int64_t SL = 32LL * E;
+    if (out.empty() && n_rows > 0) {
+        const size_t guess = static_cast<size_t>((rp[n_rows] - rp[0]) / SL + n_rows / kWarpRowCap);
+        out.reserve(guess + guess / 8 + 8);
+        lmask.reserve(32 * (guess + guess / 8 + 8));
+    }
     int32_t r = 0;
     while (r < n_rows) {
         const int32_t k0 = rp[r];
-        const size_t mo = lmask.size();
-        lmask.resize(mo + 32, 0u);
+        uint32_t w[32] = {0};
         if (static_cast<int64_t>(rp[r + 1]) - k0 > SL) {
             out.push_back(ChunkDesc{k0, rp[r + 1], r, (r + 1) | kChunkLong});
+            lmask.insert(lmask.end(), w, w + 32);
             ++*n_long;
             ++r;
             continue;
         }
-        bool empty = (rp[r + 1] == rp[r]);
-        int32_t r1 = r + 1;
-        while (r1 < n_rows && r1 - r < kWarpRowCap && static_cast<int64_t>(rp[r1 + 1]) - k0 <= SL) {
-            empty = empty || (rp[r1 + 1] == rp[r1]);
+        // a row's start is marked as it joins the chunk (not that of an empty row)
+        bool empty = false;
+        int32_t r1 = r, start = k0;
+        while (r1 < n_rows && r1 - r < kWarpRowCap) {
+            const int32_t end = rp[r1 + 1];
+            if (static_cast<int64_t>(end) - k0 > SL) break;
+            const uint32_t sl = static_cast<uint32_t>(start - k0);
+            if (end > start) w[sl / E] |= 1u << (sl % E);
+            else empty = true;
+            start = end;
             ++r1;
         }
-        out.push_back(ChunkDesc{k0, rp[r1], r, r1 | (empty ? kChunkEmpty : 0)});
+        out.push_back(ChunkDesc{k0, start, r, r1 | (empty ? kChunkEmpty : 0)});
         if (empty) ++*n_empty;
-        for (int32_t q = r; q < r1; ++q)
-            if (rp[q + 1] > rp[q]) {
-                const int32_t sl = rp[q] - k0;
-                lmask[mo + sl / E] |= 1u << (sl % E);
-            }
         if (!empty) {
-            const int64_t n_used = static_cast<int64_t>(rp[r1]) - k0;
+            const int n_used = start - k0;
             uint32_t pre = 0;
             int through_run = 0;  // lanes just before this one that lie inside one row
             for (int lane = 0; lane < 32; ++lane) {
-                const uint32_t bits = lmask[mo + lane];
-                const bool active = static_cast<int64_t>(lane) * E < n_used;
-                const bool ends = static_cast<int64_t>(lane + 1) * E >= n_used ||
-                                  (lane < 31 && (lmask[mo + lane + 1] & 1u));
+                const uint32_t bits = w[lane];
+                const bool active = lane * E < n_used;
+                const bool ends = (lane + 1) * E >= n_used || (lane < 31 && (w[lane + 1] & 1u));
                 const bool started = bits != 0u;
                 // a piece of a row begun in an earlier lane ends in this lane
                 const bool pending = active && !(bits & 1u) && (started || ends);
                 const uint32_t chain = pending ? static_cast<uint32_t>(1 + through_run) : 0u;
                 through_run = (active && !ends && !started) ? through_run + 1 : 0;
-                lmask[mo + lane] = bits | (pre << kSlotPreShift) | (ends ? kSlotEnds : 0u) |
-                                   (chain << kSlotChainShift);
+                w[lane] = bits | (pre << kSlotPreShift) | (ends ? kSlotEnds : 0u) | (chain << kSlotChainShift);
                 pre += static_cast<uint32_t>(__builtin_popcount(bits));
             }
         }
+        lmask.insert(lmask.end(), w, w + 32);
         r = r1;
+    }
+}
+
+void make_slot_chunks(const int32_t *rp, int32_t n_rows, int E, std::vector<ChunkDesc> &out,
+                      std::vector<uint32_t> &lmask, int32_t *n_long, int32_t *n_empty) {
+    switch (E) {  // the entries per lane that the kernels are compiled for
+        case 7: return make_slot_chunks_of<7>(rp, n_rows, out, lmask, n_long, n_empty);
+        case 9: return make_slot_chunks_of<9>(rp, n_rows, out, lmask, n_long, n_empty);
+        case 11: return make_slot_chunks_of<11>(rp, n_rows, out, lmask, n_long, n_empty);
+        default: return make_slot_chunks_of<15>(rp, n_rows, out, lmask, n_long, n_empty);
     }
 }
 
@@ -385,12 +402,34 @@ void free_sell(SellTable &t) {
 }
 
 void free_slots(SlotTable &t) {
-    cudaFree(t.d);
-    cudaFree(t.lmask);
-    cudaFree(t.vals);
-    cudaFree(t.cols);
+    cudaFree(t.block);
+    if (!t.block) {
+        cudaFree(t.d);
+        cudaFree(t.lmask);
+        cudaFree(t.vals);
+        cudaFree(t.cols);
+    }
     t = SlotTable();
 }
+
+// Several arrays in one allocation: add() each, alloc(), then take() them in the same
+// order.  (An allocation takes some 30 us: the first apply of a small symmetric matrix
+// 226 -> 146 us.)
+struct Block {
+    std::vector<size_t> at;
+    size_t bytes = 0, next = 0;
+    char *base = nullptr;
+    void add(size_t b) {
+        at.push_back(bytes);
+        bytes += (b + 255) / 256 * 256;
+    }
+    bool alloc() {
+        if (cudaMalloc(&base, std::max<size_t>(bytes, 256)) != cudaSuccess) base = nullptr;
+        return base != nullptr;
+    }
+    template <typename T> void take(T **p) { *p = reinterpret_cast<T *>(base + at[next++]); }
+    void take(void **p) { *p = base + at[next++]; }
+};
 
 struct DeviceGuard {
     int prev = -1;
@@ -436,6 +475,11 @@ struct spmv_matrix {
     int vk = kF64;
     int device = 0;
     bool owns_structure = true;
+    void *block = nullptr;      // holds the arrays below in one allocation (a symmetric handle's full matrix)
+    // values of the CRS arrays as val_of[map_of[k]] (an FP32 full matrix: U's), for rows
+    // that the slot-major kernel sums again
+    const int32_t *map_of = nullptr;
+    const void *val_of = nullptr;
     int32_t *d_rp = nullptr;
     int32_t *d_col = nullptr;
     void *d_val = nullptr;
@@ -475,11 +519,13 @@ struct spmv_matrix {
     std::vector<int32_t> h_rowT;
     std::map<std::pair<int, int>, TileTable> tablesT;
     // symmetric CRS: the full matrix laid out once (get_full) and the position of
-    // each of its values among U's; full_off: it does not fit
+    // each of its values among U's; full_off: two passes for good
     spmv_matrix *full = nullptr;
-    int32_t *d_fullmap = nullptr;
+    int32_t *d_fullmap = nullptr;  // in full's block
+    int32_t *d_slotmap = nullptr;  // the map in the order of the slots that full's products read
+    bool slotmap_inside = false;   // it lies in full's CRS values, which nothing reads then
+    bool crs_in_graph = false;     // a captured graph writes full's CRS values
     Laid full_laid;             // U's current values in full
-    uint64_t full_asked = 0;    // values_version of the last apply
     bool full_off = false;
     // FP32 mirror for IR-CG
     spmv_matrix *mirror32 = nullptr;
@@ -638,8 +684,10 @@ constexpr int32_t kRhsFew = 65536, kRhsFewScattered = 262144;
 // slices = false: the row slices are not considered (their padding is not counted).
 void autotune(spmv_matrix *h, bool slices = true) {
     const double mean = h->n_rows ? static_cast<double>(h->nnz) / h->n_rows : 0.0;
-    h->max_row = 0;
-    for (int32_t i = 0; i < h->n_rows; ++i) h->max_row = std::max(h->max_row, h->h_rp[i + 1] - h->h_rp[i]);
+    const int32_t *rp = h->h_rp.data();
+    int32_t longest = 0;
+    for (int32_t i = 0; i < h->n_rows; ++i) longest = std::max(longest, rp[i + 1] - rp[i]);
+    h->max_row = longest;
     int T = 1;
     while (T < 32 && T < mean * 0.5) T <<= 1;
     h->T = T;
@@ -740,13 +788,26 @@ SlotTable *get_slots(spmv_matrix *h, int E, cudaStream_t s, bool transposed = fa
         t.n = static_cast<int32_t>(d.size());
         const size_t nslots = static_cast<size_t>(t.n) * 32 * E;
         const size_t vb = (h->vk == kF64) ? 8 : 4;
-        bool ok = dmalloc(&t.d, d.size()) == cudaSuccess && dmalloc(&t.lmask, lm.size()) == cudaSuccess &&
-                  cudaMalloc(&t.vals, nslots * vb + 16) == cudaSuccess && dmalloc(&t.cols, nslots + 4) == cudaSuccess;
+        Block b;
+        b.add(sizeof(ChunkDesc) * d.size());
+        b.add(4 * lm.size());
+        b.add(nslots * vb + 16);
+        b.add(4 * (nslots + 4));
+        bool ok = b.alloc();
+        if (ok) {
+            t.block = b.base;
+            b.take(&t.d);
+            b.take(&t.lmask);
+            b.take(&t.vals);
+            b.take(&t.cols);
+        }
         ok = ok && (d.empty() || cudaMemcpy(t.d, d.data(), sizeof(ChunkDesc) * d.size(), cudaMemcpyHostToDevice) ==
                                      cudaSuccess);
         ok = ok && (lm.empty() || cudaMemcpy(t.lmask, lm.data(), 4 * lm.size(), cudaMemcpyHostToDevice) == cudaSuccess);
+        // (waited for: the next product may run on another stream)
         ok = ok && launch_slot_relayout(t.d, E, static_cast<int64_t>(nslots), h->vk, d_val, d_col, t.vals, t.cols,
-                                        s) == cudaSuccess;
+                                        s) == cudaSuccess &&
+             cudaStreamSynchronize(s) == cudaSuccess;
         if (!ok) {
             free_slots(t);
             (void)cudaGetLastError();  // a failed allocation must not surface at a later launch check
@@ -1048,12 +1109,16 @@ void destroy_matrix(spmv_matrix *h) {
     if (!h) return;
     DeviceGuard g(h->device);
     cudaDeviceSynchronize();
-    if (h->owns_structure) {
-        cudaFree(h->d_rp);
-        cudaFree(h->d_col);
+    if (h->block) {
+        cudaFree(h->block);
+    } else {
+        if (h->owns_structure) {
+            cudaFree(h->d_rp);
+            cudaFree(h->d_col);
+        }
+        cudaFree(h->d_val);
+        cudaFree(h->d_err);
     }
-    cudaFree(h->d_val);
-    cudaFree(h->d_err);
     cudaFree(h->d_rowT);
     cudaFree(h->d_colT);
     cudaFree(h->d_perm);
@@ -1070,7 +1135,7 @@ void destroy_matrix(spmv_matrix *h) {
     destroy_cg(h->cg);
     if (h->mirror32) destroy_matrix(h->mirror32);
     if (h->full) destroy_matrix(h->full);
-    cudaFree(h->d_fullmap);
+    if (!h->slotmap_inside) cudaFree(h->d_slotmap);
     delete h;
 }
 
@@ -1199,6 +1264,10 @@ spmv_status apply_impl(spmv_matrix *h, double alpha, const void *x, int xk, doub
         sp.vals = t->vals;
         sp.cols = t->cols;
         sp.m = MatRef{h->d_rp, h->d_col, h->d_val, nullptr, x, y, h->d_rmap};
+        if (h->map_of && t->n_long == 0 && t->n_empty == 0) {
+            sp.m.vs = h->map_of;
+            sp.m.vind = h->val_of;
+        }
         sp.n_chunks = t->n;
         sp.alpha = alpha;
         sp.beta = beta;
@@ -1426,11 +1495,11 @@ static spmv_status capture_graph(F body, cudaGraphExec_t *exec) {
 // diagonal.  The product y = alpha*(U + U_s^T)*x + beta*y runs on the full matrix,
 // expanded on the device once (get_full): reading an entry twice in order costs far
 // less than finding it through its position (Hamiltonian-like, 4.2 M rows: FP64 148
-// against 429 us, FP32 storage 139 against 372; 1.05 M rows 42 against 89, 41 / 67).  With a plan chosen by the caller, or without room for the
-// full matrix, it runs in two passes with a fixed summation order: the row sums of U on the autotuned
-// kernel (with beta), then the row sums of U_s^T (the strictly upper part,
-// transposed) added onto y by the warp-chunk kernel that reads each value
-// through its position in U.
+// against 429 us, FP32 storage 139 against 372; 1.05 M rows 41 against 87, 41 / 66).
+// With a plan chosen by the caller, or without the full matrix, it runs in two passes
+// with a fixed summation order: the row sums of U on the autotuned kernel (with beta),
+// then the row sums of U_s^T (the strictly upper part, transposed) added onto y by the
+// warp-chunk kernel that reads each value through its position in U.
 static spmv_status create_symmetric_index(spmv_matrix *h, const int32_t *col_host, cudaStream_t s) {
     const int32_t n = h->n_rows;
     std::vector<int32_t> rowS(static_cast<size_t>(n) + 1, 0);
@@ -1467,53 +1536,118 @@ static spmv_status create_symmetric_index(spmv_matrix *h, const int32_t *col_hos
     return SPMV_OK;
 }
 
-// The full matrix A = U + U_s^T of a symmetric handle, built on first use from U and
-// the transposed index, with U's current values; null when it does not fit (in
-// memory or in int32 entry numbers).  Null too at the first apply on new values:
-// laying them out costs more than the two passes save once (1.05 M rows FP64: new
-// values and one apply 174 against 145 us), so the second apply on them does it.
+// The slots that full's products read, when every entry has one (no chunks or rows
+// summed from the CRS arrays): their values, how many there are, and their part of the
+// map laid out like them (built on first use; null while a stream is captured, or
+// without room).  Products then never read full's CRS values, whose array takes the map
+// in FP64 (FP32 sums out of range read U's, through the map).
+struct FullSlots {
+    void *vals = nullptr;
+    int64_t n = 0;
+    Laid *laid = nullptr;
+};
+static FullSlots full_slots(spmv_matrix *h, cudaStream_t s) {
+    spmv_matrix *f = h->full;
+    FullSlots r;
+    const auto c = f->slots.find(f->E);
+    const auto l = f->sells.find(f->sigma);
+    const bool chunks = f->family == 4 && c != f->slots.end() && c->second.n_long == 0 && c->second.n_empty == 0;
+    const bool slices = f->family == 5 && l != f->sells.end() && l->second.vals && l->second.n_long == 0;
+    if (chunks) r = FullSlots{c->second.vals, static_cast<int64_t>(c->second.n) * 32 * f->E, &c->second.laid};
+    if (slices) r = FullSlots{l->second.vals, l->second.slot_rows * kSellC, &l->second.laid};
+    if (!r.vals || h->d_slotmap) return r;
+    const bool inside = f->vk == kF64 && 4 * r.n <= 8 * f->nnz && !h->crs_in_graph;
+    if (capture_id(s) || (!inside && cudaMalloc(&h->d_slotmap, 4 * static_cast<size_t>(r.n) + 16) != cudaSuccess)) {
+        h->d_slotmap = nullptr;
+        (void)cudaGetLastError();
+        return FullSlots();
+    }
+    if (inside) h->d_slotmap = static_cast<int32_t *>(f->d_val);
+    h->slotmap_inside = inside;
+    cudaError_t e = chunks ? launch_slot_map(c->second.d, f->E, r.n, h->d_fullmap, h->d_slotmap, s)
+                           : cudaMemsetAsync(h->d_slotmap, 0xff, 4 * static_cast<size_t>(kSellU) * kSellC, s);
+    if (e == cudaSuccess && slices)
+        e = launch_sell_relayout(l->second.d, l->second.srows, l->second.n, f->d_rp, f->vk, nullptr, h->d_fullmap,
+                                 nullptr, h->d_slotmap, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the next values may come on another stream
+    if (e == cudaSuccess) return r;
+    if (!inside) cudaFree(h->d_slotmap);
+    h->d_slotmap = nullptr;
+    h->slotmap_inside = false;
+    return FullSlots();
+}
+
+// U's values in the full matrix: in the slots that the products read, through their map,
+// else in the CRS arrays (1.05 M rows, new values and one apply: FP64 124 us, two passes
+// 143; FP32 87, 110; 27-point 64^3 FP64 65, 59, where the gathers' cache lines bound it).
+static cudaError_t fill_full(spmv_matrix *h, cudaStream_t s) {
+    spmv_matrix *f = h->full;
+    for (auto &kv : f->slots) kv.second.laid = Laid();
+    for (auto &kv : f->sells) kv.second.laid = Laid();
+    const FullSlots t = full_slots(h, s);
+    cudaError_t e = cudaSuccess;
+    if (!t.vals) {
+        e = launch_permute(h->d_val, h->d_fullmap, f->d_val, f->nnz, f->vk, s);
+        h->crs_in_graph = h->crs_in_graph || capture_id(s) != 0;
+    }
+    if (e == cudaSuccess && t.vals) {
+        e = launch_fill_slots(h->d_val, h->d_slotmap, t.vals, t.n, f->vk, s);
+        if (e == cudaSuccess) t.laid->set(s);
+    }
+    return e;
+}
+
+// The full matrix A = U + U_s^T of a symmetric handle, built by the first apply from U and
+// the transposed index, with U's current values; null when it does not fit (in memory or
+// in int32 entry numbers) or the first apply is captured, where nothing is allocated: the
+// handle then keeps to the two passes, so that all its applies sum in one order.
 static spmv_matrix *get_full(spmv_matrix *h, cudaStream_t s) {
     if (h->full_off) return nullptr;
-    const bool have = h->full ? h->full_laid.on(s) : h->values_version == 0;  // new handles: the values of their creation
-    const bool again = h->full_asked == h->values_version;
-    h->full_asked = h->values_version;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return nullptr;
-    if (cap == cudaStreamCaptureStatusNone) {
-        if (!have && !again) return nullptr;
-    } else if (!h->full || (!have && again)) {
-        return nullptr;  // under capture nothing is allocated
-    }
     if (!h->full) {
         const int32_t n = h->n_rows;
         const int64_t ns = h->h_rowT[n], nnz = h->nnz + ns;
-        spmv_matrix *f = nnz < (int64_t(1) << 31) ? new (std::nothrow) spmv_matrix() : nullptr;
+        spmv_matrix *f = nnz < (int64_t(1) << 31) && !capture_id(s) ? new (std::nothrow) spmv_matrix() : nullptr;
         bool ok = f != nullptr;
         if (ok) {
             f->device = h->device;
             f->n_rows = f->n_cols = n;
             f->nnz = nnz;
             f->vk = h->vk;
+            f->acc32 = h->acc32;
             f->col_random = h->col_random;
             f->col_diag = h->col_diag;
             f->h_rp.resize(static_cast<size_t>(n) + 1);
-            for (int32_t i = 0; i <= n; ++i) f->h_rp[i] = h->h_rp[i] + h->h_rowT[i];
+            const int32_t *ru = h->h_rp.data(), *rs = h->h_rowT.data();
+            int32_t *rf = f->h_rp.data();
+            for (int32_t i = 0; i <= n; ++i) rf[i] = ru[i] + rs[i];
             const size_t nrp = static_cast<size_t>(n) + 1 + kRowPad, nent = static_cast<size_t>(nnz) + kEntryPad;
             const size_t vb = h->vk == kF64 ? 8 : 4;
-            ok = dmalloc(&f->d_rp, nrp) == cudaSuccess && dmalloc(&f->d_col, nent) == cudaSuccess &&
-                 cudaMalloc(&f->d_val, nent * vb) == cudaSuccess && dmalloc(&f->d_err, 1) == cudaSuccess &&
-                 dmalloc(&h->d_fullmap, nent) == cudaSuccess &&
-                 cudaMemsetAsync(f->d_err, 0, 4, s) == cudaSuccess &&
+            Block b;
+            b.add(4 * nrp);
+            b.add(4 * nent);
+            b.add(vb * nent);
+            b.add(4);
+            b.add(4 * nent);
+            ok = b.alloc();
+            if (ok) {
+                f->block = b.base;
+                b.take(&f->d_rp);
+                b.take(&f->d_col);
+                b.take(&f->d_val);
+                b.take(&f->d_err);
+                b.take(&h->d_fullmap);
+            }
+            ok = ok && cudaMemsetAsync(f->d_err, 0, 4, s) == cudaSuccess &&
                  cudaMemsetAsync(f->d_rp + n + 1, 0, kRowPad * 4, s) == cudaSuccess &&
                  cudaMemsetAsync(f->d_col + nnz, 0, kEntryPad * 4, s) == cudaSuccess &&
                  cudaMemsetAsync(static_cast<char *>(f->d_val) + nnz * vb, 0, kEntryPad * vb, s) == cudaSuccess &&
                  launch_expand_sym(n, h->d_rp, h->d_col, h->d_rowT, h->d_colT, h->d_perm, f->d_rp, f->d_col,
                                    h->d_fullmap, s) == cudaSuccess &&
-                 launch_permute(h->d_val, h->d_fullmap, f->d_val, nnz, h->vk, s) == cudaSuccess;
+                 launch_permute(h->d_val, h->d_fullmap, f->d_val, nnz, h->vk, s) == cudaSuccess &&
+                 cudaStreamSynchronize(s) == cudaSuccess;  // the next apply may run on another stream
         }
         if (!ok) {
             if (f) destroy_matrix(f);
-            cudaFree(h->d_fullmap);
             h->d_fullmap = nullptr;
             (void)cudaGetLastError();  // a failed allocation must not surface at a later launch check
             h->full_off = true;
@@ -1527,19 +1661,17 @@ static spmv_matrix *get_full(spmv_matrix *h, cudaStream_t s) {
             f->family = 4;
             f->E = 15;
             f->sell_if_diag = false;
+            f->map_of = h->d_fullmap;
+            f->val_of = h->d_val;
         }
         h->full = f;
         h->full_laid.now = true;
     }
-    spmv_matrix *f = h->full;
     if (!h->full_laid.on(s)) {
-        if (launch_permute(h->d_val, h->d_fullmap, f->d_val, f->nnz, f->vk, s) != cudaSuccess) return nullptr;
-        for (auto &kv : f->slots) kv.second.laid = Laid();
-        for (auto &kv : f->sells) kv.second.laid = Laid();
+        if (fill_full(h, s) != cudaSuccess) return nullptr;
         h->full_laid.set(s);
     }
-    f->acc32 = h->acc32;
-    return f;
+    return h->full;
 }
 
 static spmv_status apply_sym(spmv_matrix *h, double alpha, const void *x, int xk, double beta, void *y, int yk,
@@ -1836,6 +1968,7 @@ spmv_status spmv_set_plan(spmv_handle h, int32_t family, int32_t param) {
 spmv_status spmv_set_accumulator(spmv_handle h, int32_t acc) {
     if (!h || (acc != 0 && acc != 1)) return SPMV_ERR_INVALID_ARG;
     h->acc32 = (acc == 0) ? kAccF64 : kAccFF;
+    if (h->full) h->full->acc32 = h->acc32;
     return SPMV_OK;
 }
 

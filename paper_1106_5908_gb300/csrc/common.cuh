@@ -257,7 +257,7 @@ __device__ __forceinline__ double row_sum_exact(const MatRef m, int64_t r, const
     const int kb = __ldg(m.rp + r), ke = __ldg(m.rp + r + 1);
     for (int k = kb; k < ke; ++k) {
         VT v;
-        if constexpr (INDIRECT)
+        if (INDIRECT || m.vind)  // (a full matrix's values stay where the symmetric handle has them)
             v = __ldg(static_cast<const VT *>(m.vind) + __ldg(static_cast<const int32_t *>(m.vs) + k));
         else
             v = __ldg(static_cast<const VT *>(m.vs) + k);

@@ -56,6 +56,9 @@ bool slot_ops_batched(int vk, int acc, int E, SlotOps *ops);
 // indices) of the regular chunks in `chunks` (ChunkDesc[n_slots / (32E)]).
 cudaError_t launch_slot_relayout(const void *chunks, int E, int64_t n_slots, int vk, const void *val,
                                  const int32_t *col, void *vals_out, int32_t *cols_out, cudaStream_t s);
+// The slot-major copy of a map over the entries, -1 in the other slots.
+cudaError_t launch_slot_map(const void *chunks, int E, int64_t n_slots, const int32_t *map, int32_t *map_out,
+                            cudaStream_t s);
 
 struct SellBatchParams;
 // The batched launch over members on diagonal slices: FP64, or FP32 storage with FP32
@@ -151,6 +154,8 @@ cudaError_t launch_rowvec(const KParams &p, const int32_t n_rows, int vk, int xk
 
 // out[k] = val[perm[k]] for k < nnz (values of kind vk: FP64 or FP32).
 cudaError_t launch_permute(const void *val, const int32_t *perm, void *out, int64_t nnz, int vk, cudaStream_t s);
+// out[t] = val[map[t]] for t < n, 0 where map[t] < 0 (map and out 16-byte aligned).
+cudaError_t launch_fill_slots(const void *val, const int32_t *map, void *out, int64_t n, int vk, cudaStream_t s);
 // The full CRS of a symmetric matrix from its upper triangle (rp, col) and the
 // transposed strictly upper part (rowS, colS, permS); mapF: position of each entry's
 // value among U's.

@@ -160,6 +160,48 @@ cudaError_t launch_permute(const void *val, const int32_t *perm, void *out, int6
     return cudaGetLastError();
 }
 
+// Slots filled through their map.  Four slots to a thread: one 16-byte load of the map
+// and four independent gathers (the map of a slot-major copy puts a warp's neighbours E
+// entries apart, so each gather is a sector of its own, found again in L1 by the next
+// slot rows).  1.05 M Hamiltonian-like rows, 13.5 M slots FP64: about 65 us; the CRS values
+// permuted and laid out again about 105.
+template <typename VT>
+__global__ void __launch_bounds__(256) k_fill_slots(const VT *__restrict__ val, const int4 *__restrict__ map,
+                                                    VT *__restrict__ out, int64_t n4, int64_t n) {
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    const int64_t t0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    for (int64_t t = t0; t < n4; t += stride) {
+        const int4 m = __ldg(map + t);
+        const VT a = m.x >= 0 ? __ldg(val + m.x) : VT(0), b = m.y >= 0 ? __ldg(val + m.y) : VT(0);
+        const VT c = m.z >= 0 ? __ldg(val + m.z) : VT(0), d = m.w >= 0 ? __ldg(val + m.w) : VT(0);
+        if constexpr (sizeof(VT) == 8) {
+            reinterpret_cast<double2 *>(out)[2 * t] = make_double2(a, b);
+            reinterpret_cast<double2 *>(out)[2 * t + 1] = make_double2(c, d);
+        } else {
+            reinterpret_cast<float4 *>(out)[t] = make_float4(a, b, c, d);
+        }
+    }
+    for (int64_t t = 4 * n4 + t0; t < n; t += stride) {
+        const int32_t m = __ldg(reinterpret_cast<const int32_t *>(map) + t);
+        out[t] = m >= 0 ? __ldg(val + m) : VT(0);
+    }
+}
+
+cudaError_t launch_fill_slots(const void *val, const int32_t *map, void *out, int64_t n, int vk, cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t want = (n / 4 + 256) / 256;
+    const int grid = static_cast<int>(want < 16LL * sms ? want : 16LL * sms);
+    const int4 *m = reinterpret_cast<const int4 *>(map);
+    if (vk == kF64)
+        k_fill_slots<double><<<grid, 256, 0, s>>>(static_cast<const double *>(val), m, static_cast<double *>(out), n / 4, n);
+    else
+        k_fill_slots<float><<<grid, 256, 0, s>>>(static_cast<const float *>(val), m, static_cast<float *>(out), n / 4, n);
+    return cudaGetLastError();
+}
+
 // Symmetric CRS expanded: row i = row i of the transposed strictly upper part (rowS,
 // colS: columns below i, ascending; permS: positions in U's values), then row i of U.
 // A warp per row.

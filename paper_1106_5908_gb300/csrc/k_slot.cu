@@ -72,22 +72,30 @@ bool slot_ops_tv(int vk, int xk, int yk, int acc, int E, SlotOps *ops) {
     return false;
 }
 
-cudaError_t launch_slot_relayout(const void *chunks, int E, int64_t n_slots, int vk, const void *val,
-                                 const int32_t *col, void *vals_out, int32_t *cols_out, cudaStream_t s) {
+template <typename VT>
+static cudaError_t relayout_as(const void *chunks, int E, int64_t n_slots, const void *val, const int32_t *col,
+                               void *vals_out, int32_t *cols_out, VT pad, cudaStream_t s) {
     if (n_slots <= 0) return cudaSuccess;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t want = (n_slots + 255) / 256;
     const int grid = static_cast<int>(want < 16LL * sms ? want : 16LL * sms);
-    const ChunkDesc *d = static_cast<const ChunkDesc *>(chunks);
-    if (vk == kF64)
-        k_slot_relayout<double><<<grid, 256, 0, s>>>(d, E, n_slots, static_cast<const double *>(val), col,
-                                                     static_cast<double *>(vals_out), cols_out);
-    else
-        k_slot_relayout<float><<<grid, 256, 0, s>>>(d, E, n_slots, static_cast<const float *>(val), col,
-                                                    static_cast<float *>(vals_out), cols_out);
+    k_slot_relayout<VT><<<grid, 256, 0, s>>>(static_cast<const ChunkDesc *>(chunks), E, n_slots,
+                                             static_cast<const VT *>(val), col, static_cast<VT *>(vals_out), cols_out,
+                                             pad);
     return cudaGetLastError();
+}
+
+cudaError_t launch_slot_relayout(const void *chunks, int E, int64_t n_slots, int vk, const void *val,
+                                 const int32_t *col, void *vals_out, int32_t *cols_out, cudaStream_t s) {
+    return vk == kF64 ? relayout_as<double>(chunks, E, n_slots, val, col, vals_out, cols_out, 0.0, s)
+                      : relayout_as<float>(chunks, E, n_slots, val, col, vals_out, cols_out, 0.0f, s);
+}
+
+cudaError_t launch_slot_map(const void *chunks, int E, int64_t n_slots, const int32_t *map, int32_t *map_out,
+                            cudaStream_t s) {
+    return relayout_as<int32_t>(chunks, E, n_slots, map, nullptr, map_out, nullptr, -1, s);
 }
 
 }  // namespace spmv

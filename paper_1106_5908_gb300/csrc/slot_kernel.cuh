@@ -491,12 +491,12 @@ struct SlotKernelTV {
 
 // Slot-major copies of a CRS: slot t = chunk*32E + e*32 + l holds entry
 // k0 + l*E + e of the chunk when the chunk is regular and the entry belongs to
-// it, else zero.  cols_out may be null (values only, after new values).
+// it, else pad.  cols_out may be null (values only, after new values).
 template <typename VT>
 __global__ void __launch_bounds__(256) k_slot_relayout(const ChunkDesc *__restrict__ chunks, int E,
                                                        int64_t n_slots, const VT *__restrict__ val,
                                                        const int32_t *__restrict__ col, VT *__restrict__ vals_out,
-                                                       int32_t *__restrict__ cols_out) {
+                                                       int32_t *__restrict__ cols_out, VT pad) {
     const int64_t SL = 32LL * E;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < n_slots; t += stride) {
@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(256) k_slot_relayout(const ChunkDesc *__restri
         const ChunkDesc d = chunks[cc];
         const int64_t k = static_cast<int64_t>(d.k0) + static_cast<int64_t>(l) * E + e;
         const bool ok = ((d.r1f & (kChunkLong | kChunkEmpty)) == 0) && k < d.k1;
-        vals_out[t] = ok ? val[k] : VT(0);
+        vals_out[t] = ok ? val[k] : pad;
         if (cols_out) cols_out[t] = ok ? col[k] : 0;
     }
 }

@@ -100,8 +100,9 @@ class Matrix:
     def from_symmetric_upper(cls, row_ptr, col_idx, val, dtype: Optional[torch.dtype] = None,
                              device="cuda") -> "Matrix":
         """Symmetric CRS: a symmetric n x n matrix from its upper triangle with
-        the diagonal (host numpy arrays; every column >= its row).  apply()
-        computes y = alpha*A*x + beta*y with each off-diagonal value stored once."""
+        the diagonal (host numpy arrays; every column >= its row), so each
+        off-diagonal value is given, and set, once.  apply() computes
+        y = alpha*A*x + beta*y; the first one expands A in device memory."""
         device = torch.device(device)
         rp = np.ascontiguousarray(row_ptr, dtype=np.int32)
         ci = np.ascontiguousarray(col_idx, dtype=np.int32)
