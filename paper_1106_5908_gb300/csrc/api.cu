@@ -149,8 +149,9 @@ struct SellTable {
     int4 *dtmp = nullptr, *dorder = nullptr;
     int4 *diag = nullptr;
     bool diagonal = false;      // enough slices are diagonal for k_sell_diag
-    int32_t *vpos = nullptr;    // A^T: position of each slot's value in A's copy for window
-    int32_t vpos_sigma = 0;     //      vpos_sigma (built on first use)
+    // A^T: position of each slot's value in A's copy for a window (built on first use;
+    // held for each window of A that reverse passes ran on: captured ones read them)
+    std::map<int32_t, int32_t *> vpos;
 };
 
 struct ChunkTable {
@@ -395,7 +396,7 @@ void sell_ranges(const std::vector<int2> &d, const int32_t *rp, int G, std::vect
 
 void free_sell(SellTable &t) {
     cudaFree(t.meta);
-    cudaFree(t.vpos);
+    for (auto &kv : t.vpos) cudaFree(kv.second);
     cudaFree(t.vals);
     cudaFree(t.cols);
     t = SellTable();
@@ -1004,29 +1005,23 @@ SellTable *get_sell_positions(spmv_matrix *h, cudaStream_t s) {
     if (!a.diagonal || a.n_long > 0 || a.slot_rows * kSellC > INT32_MAX) return nullptr;
     SellTable *t = get_sell(h, kSellSigma, s, true, false);
     if (!t || !t->diagonal) return nullptr;
-    if ((!t->vpos || t->vpos_sigma != h->sigma) && capture_id(s)) return nullptr;  // nothing is built
-    if (t->vpos && t->vpos_sigma != h->sigma) {  // another plan since: other positions
-        cudaFree(t->vpos);
-        t->vpos = nullptr;
+    if (t->vpos.count(h->sigma)) return t;
+    if (capture_id(s)) return nullptr;  // nothing is built
+    const size_t nslots = static_cast<size_t>(t->slot_rows) * kSellC;
+    int32_t *vpos = nullptr, *rowpos = nullptr;
+    bool ok = dmalloc(&vpos, nslots + 4) == cudaSuccess &&
+              dmalloc(&rowpos, static_cast<size_t>(h->n_rows)) == cudaSuccess &&
+              cudaMemsetAsync(vpos, 0xff, static_cast<size_t>(kSellU) * kSellC * 4, s) == cudaSuccess &&
+              launch_sell_vpos(a.d, a.srows, a.n, t->d, t->srows, t->n, h->d_rp, h->d_rowT, h->d_colT, h->d_perm, rowpos,
+                               vpos, s) == cudaSuccess &&
+              cudaStreamSynchronize(s) == cudaSuccess;
+    cudaFree(rowpos);
+    if (!ok) {
+        cudaFree(vpos);
+        (void)cudaGetLastError();
+        return nullptr;
     }
-    if (!t->vpos) {
-        const size_t nslots = static_cast<size_t>(t->slot_rows) * kSellC;
-        int32_t *rowpos = nullptr;
-        bool ok = dmalloc(&t->vpos, nslots + 4) == cudaSuccess &&
-                  dmalloc(&rowpos, static_cast<size_t>(h->n_rows)) == cudaSuccess &&
-                  cudaMemsetAsync(t->vpos, 0xff, static_cast<size_t>(kSellU) * kSellC * 4, s) == cudaSuccess &&
-                  launch_sell_vpos(a.d, a.srows, a.n, t->d, t->srows, t->n, h->d_rp, h->d_rowT, h->d_colT, h->d_perm,
-                                   rowpos, t->vpos, s) == cudaSuccess &&
-                  cudaStreamSynchronize(s) == cudaSuccess;
-        cudaFree(rowpos);
-        if (!ok) {
-            cudaFree(t->vpos);
-            t->vpos = nullptr;
-            (void)cudaGetLastError();
-            return nullptr;
-        }
-        t->vpos_sigma = h->sigma;
-    }
+    t->vpos[h->sigma] = vpos;
     return t;
 }
 
@@ -2388,7 +2383,7 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
                 SellParams lp =
                     sell_params(*t, MatRef{h->d_rowT, h->d_colT, h->d_perm, h->d_val, g, grad_x, nullptr}, alpha, 0.0);
                 lp.vals = a->vals;
-                lp.vpos = t->vpos;
+                lp.vpos = t->vpos.at(h->sigma);
                 if (lops.launch_ind(lp, s) != cudaSuccess) return SPMV_ERR_CUDA;
                 done = true;
             }

@@ -119,3 +119,35 @@ def test_reverse_pass_captured(kind, new_values):
         check((gx2, gv2), host(vd), "replayed, new values")
     M.set_values(vd)
     check(M.backward(g, x), host(vd), "after the graph")
+
+
+def test_captured_reverse_pass_outlives_its_plan():
+    """A first reverse pass on new values reads positions that belong to the window of A's
+    slices; a pass on another window beside the graph leaves the graph's alone."""
+    from paper_1106_5908_gb300 import Matrix
+    A = W.stencil27(26)
+    M = Matrix.from_csr(A.row_ptr, A.col_idx, A.val, A.n_cols)
+    x, g, source = dev(W.uniform(A.n_cols, 3)), dev(W.uniform(A.n_rows, 4)), dev(A.val)
+    T = oracle.transpose(A.row_ptr, A.col_idx, A.n_cols)
+
+    def step():
+        M.set_values(source)
+        M.apply(x)
+        return M.backward(g, x)[0]
+
+    for _ in range(2):
+        step()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        gx = step()
+    for turn, window in enumerate((64, 4096, 1024)):
+        val = W.uniform(A.nnz, 30 + turn)
+        source.copy_(dev(val))
+        ref, bound = oracle.spmv(T[0], T[1], val[T[2]], host(g), with_bound=True)
+        M.set_plan(5, window)
+        for _ in range(2):
+            assert_within(host(step()), ref, bound, 1e-13, f"{window}")
+        gx.zero_()
+        graph.replay()
+        assert_within(host(gx), ref, bound, 1e-13, f"replayed after {window}")
