@@ -679,6 +679,9 @@ constexpr int32_t kBatchDiagMinSize = 32768;
 
 // Share of far entries (column_randomness) above which columns count as scattered.
 constexpr double kScattered = 0.25;
+// Entries from which a reverse pass reads A's slices: grad_x through their positions
+// (rows of up to 8 entries), grad_val (spmv_backward).
+constexpr int64_t kPosMinEntries = 400000, kGradValMinEntries = 2000000;
 // Rows from which 2 or 3 right-hand sides run on the row slices (spmm_apply).
 constexpr int32_t kRhsFew = 65536, kRhsFewScattered = 262144;
 
@@ -1806,13 +1809,17 @@ static spmv_status set_values_impl(spmv_matrix *h, const void *val, spmv_dtype t
     if (h->nnz == 0) return SPMV_OK;
     // a row-slice copy that served the last values, or serves this product, gets the new
     // ones in the same pass (27-point 128^3: 226 us where the CRS copy alone takes 136);
-    // other copies are laid out again when they are used
+    // other copies are laid out again when they are used.  Small grids of short rows get
+    // only product and values in one pass: the tile's chain of loads takes longer than
+    // the copy and the layout one after the other (new values and a product, 5-point
+    // 140^2 FP64 8.3 against 6.2 us, 200^2 8.8 / 7.2, 300^2 9.2 / 10.2; 7-point 25^3 FP32
+    // 9.3 / 7.7, 40^3 8.9 / 9.0; 27-point 12^3 11.0 / 12.7)
     auto f = h->sells.find(h->sigma);
     const bool slices = h->family == 5 && f != h->sells.end() && f->second.laid.on(s) && f->second.diagonal &&
                         sell_tile_fits(h);
     const bool prod = slices && y && static_cast<int>(t) == h->vk && !h->sym && !h->d_rmap &&
                       (h->vk == kF64 || h->acc32 == kAccFF);
-    const bool fused = slices && (prod || f->second.read);
+    const bool fused = slices && (prod || (f->second.read && (h->nnz > 8LL * h->n_rows || h->nnz >= kPosMinEntries)));
     if (fused) {
         const SellParams p = sell_params(
             f->second, MatRef{h->d_rp, h->d_col, prod ? val : nullptr, nullptr, prod ? x : nullptr, prod ? y : nullptr, nullptr},
@@ -2371,13 +2378,19 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
             // product has laid them out there: doing it for this pass alone costs what
             // the pass then saves (new values and a reverse pass: 7-point 160^3 290
             // against 257 us through the permutation, 5-point 2000^2 210 / 195; 27-point
-            // 128^3 500 against 606)
+            // 128^3 500 against 606).  Such rows also need kPosMinEntries entries: a
+            // smaller grid's pass is one chain of loads, which the positions lengthen
+            // (new values, product and reverse pass, FP32: 5-point 100^2 12.7 against
+            // 11.4 us, 200^2 13.3 / 12.2, 300^2 13.8 / 15.0; 27-point 12^3 14.2 / 16.1
+            // for grad_x).
             SellOps lops;
             const int acc = (h->vk == kF32) ? kAccFF : kAccF64;
             const SellTable *t = nullptr, *a = nullptr;
-            if (sell_ops(h->vk, h->vk, h->vk, acc, &lops) && (t = get_sell_positions(h, s)) != nullptr) {
+            const bool longer = h->nnz > 8LL * h->n_rows;
+            if ((longer || h->nnz >= kPosMinEntries) && sell_ops(h->vk, h->vk, h->vk, acc, &lops) &&
+                (t = get_sell_positions(h, s)) != nullptr) {
                 const SellTable &own = h->sells.at(h->sigma);
-                a = h->nnz > 8LL * h->n_rows ? get_sell(h, h->sigma, s) : own.vals && own.laid.on(s) ? &own : nullptr;
+                a = longer ? get_sell(h, h->sigma, s) : own.vals && own.laid.on(s) ? &own : nullptr;
             }
             if (a) {
                 SellParams lp =
@@ -2453,12 +2466,15 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
     if (grad_val && h->nnz > 0) {
         // Rows of more than 8 entries on average: on A's diagonal slices, when a
         // forward product or a second reverse pass has built them (27-point 128^3:
-        // FP64 138 against 162 us, FP32 63 against 112).  Else warp chunks of
-        // kGradValE entries per lane, rows from the row-start bitmasks (7-point 160^3
-        // FP64 88 us on either, 5-point 2000^2 FP32 45 against 54-65 on the slices,
-        // whose work per half slice no longer covers its set-up).
+        // FP64 138 against 162 us, FP32 63 against 112), from kGradValMinEntries
+        // entries on (a half slice is one long chain: 24^3 FP64 6.2 against 3.8 us, FP32
+        // 4.9 / 2.4; 32^3 6.6 / 5.6, 5.0 / 4.5; 48^3 13.0 / 14.1, 6.3 / 8.0).  Else warp
+        // chunks of kGradValE entries per lane, rows from the row-start bitmasks
+        // (7-point 160^3 FP64 88 us on either, 5-point 2000^2 FP32 45 against 54-65 on
+        // the slices, whose work per half slice no longer covers its set-up).
         const SellTable *f = nullptr;
-        if (h->family == 5 && h->nnz > 8LL * h->n_rows && (again || h->sells.count(h->sigma)) && sell_tile_fits(h))
+        if (h->family == 5 && h->nnz > 8LL * h->n_rows && h->nnz >= kGradValMinEntries &&
+            (again || h->sells.count(h->sigma)) && sell_tile_fits(h))
             f = get_sell(h, h->sigma, s, false, false);
         if (f && f->diagonal && (reinterpret_cast<uintptr_t>(grad_val) & 15u) == 0) {
             const SellParams p = sell_params(

@@ -19,12 +19,14 @@ def _gpu():
     need_gpu()
 
 
-@pytest.mark.parametrize("kind", ["5-point", "7-point", "27-point"])
+# below and above the entries from which the reverse passes read A's slices
+@pytest.mark.parametrize("kind,n", [("5-point", 131), ("5-point", 290), ("7-point", 27), ("7-point", 39), ("27-point", 26),
+                                    ("27-point", 44)])
 @pytest.mark.parametrize("dtype", ["f64", "f32"])
 @pytest.mark.parametrize("seed", [1, 2])
-def test_any_order(kind, dtype, seed):
+def test_any_order(kind, n, dtype, seed):
     from paper_1106_5908_gb300 import Matrix
-    A = {"5-point": lambda: W.laplace2d(131), "7-point": lambda: W.laplace3d(27), "27-point": lambda: W.stencil27(26)}[kind]()
+    A = {"5-point": W.laplace2d, "7-point": W.laplace3d, "27-point": W.stencil27}[kind](n)
     ft, tol = (np.float64, 1e-13) if dtype == "f64" else (np.float32, 1e-6)
     T = oracle.transpose(A.row_ptr, A.col_idx, A.n_cols)
     rows = np.repeat(np.arange(A.n_rows), np.diff(A.row_ptr.astype(np.int64)))
