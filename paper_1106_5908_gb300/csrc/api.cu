@@ -171,6 +171,11 @@ void make_chunks(const int32_t *rp, int32_t n_rows, int E, int32_t mat, std::vec
                  int32_t *n_empty) {
     const int64_t SL = 32LL * E;
     const int MW = ((E + 3) / 4) * 4;  // mask words per chunk, rows of 16 bytes
+    if (out.empty() && n_rows > 0) {
+        const size_t guess = static_cast<size_t>((rp[n_rows] - rp[0]) / SL + n_rows / kWarpRowCap);
+        out.reserve(guess + guess / 8 + 8);
+        masks.reserve(MW * (guess + guess / 8 + 8));
+    }
     int32_t r = 0;
     while (r < n_rows) {
         const int32_t k0 = rp[r];
@@ -414,8 +419,7 @@ void free_slots(SlotTable &t) {
 }
 
 // Several arrays in one allocation: add() each, alloc(), then take() them in the same
-// order.  (An allocation takes some 30 us: the first apply of a small symmetric matrix
-// 226 -> 146 us.)
+// order.  (An allocation of a megabyte or more takes some 40 to 80 us, a smaller one 4.)
 struct Block {
     std::vector<size_t> at;
     size_t bytes = 0, next = 0;
@@ -743,7 +747,9 @@ double column_randomness(const int32_t *rp, const int32_t *col, int32_t n_rows) 
 // indices.
 double diagonal_rows(const int32_t *rp, const int32_t *col, int32_t n_rows) {
     if (!col || n_rows < 2) return 0.0;
-    const int32_t step = std::max<int32_t>(1, n_rows / 32768) | 1;  // odd: no grid line is sampled alone
+    // (8,192 rows: with 32,768 the statistic took 9 % of spmv_create on the 27-point
+    // 64^3 pattern)
+    const int32_t step = std::max<int32_t>(1, n_rows / 8192) | 1;  // odd: no grid line is sampled alone
     int64_t same = 0, total = 0;
     for (int32_t i = 1; i < n_rows; i += step) {
         const int32_t len = rp[i + 1] - rp[i];
@@ -792,18 +798,24 @@ SlotTable *get_slots(spmv_matrix *h, int E, cudaStream_t s, bool transposed = fa
         t.n = static_cast<int32_t>(d.size());
         const size_t nslots = static_cast<size_t>(t.n) * 32 * E;
         const size_t vb = (h->vk == kF64) ? 8 : 4;
-        Block b;
-        b.add(sizeof(ChunkDesc) * d.size());
-        b.add(4 * lm.size());
-        b.add(nslots * vb + 16);
-        b.add(4 * (nslots + 4));
-        bool ok = b.alloc();
-        if (ok) {
-            t.block = b.base;
-            b.take(&t.d);
-            b.take(&t.lmask);
-            b.take(&t.vals);
-            b.take(&t.cols);
+        bool ok;
+        if (nslots * vb + 16 < (size_t(1) << 20)) {
+            ok = dmalloc(&t.d, d.size()) == cudaSuccess && dmalloc(&t.lmask, lm.size()) == cudaSuccess &&
+                 cudaMalloc(&t.vals, nslots * vb + 16) == cudaSuccess && dmalloc(&t.cols, nslots + 4) == cudaSuccess;
+        } else {
+            Block b;
+            b.add(sizeof(ChunkDesc) * d.size());
+            b.add(4 * lm.size());
+            b.add(nslots * vb + 16);
+            b.add(4 * (nslots + 4));
+            ok = b.alloc();
+            if (ok) {
+                t.block = b.base;
+                b.take(&t.d);
+                b.take(&t.lmask);
+                b.take(&t.vals);
+                b.take(&t.cols);
+            }
         }
         ok = ok && (d.empty() || cudaMemcpy(t.d, d.data(), sizeof(ChunkDesc) * d.size(), cudaMemcpyHostToDevice) ==
                                      cudaSuccess);
@@ -829,6 +841,10 @@ SlotTable *get_slots(spmv_matrix *h, int E, cudaStream_t s, bool transposed = fa
     }
     return &t;
 }
+
+// Fewer rows than this: the host sorts them faster than six launches and a read-back take
+// (27-point 12^3, first product: 102 against 131 us).
+constexpr int32_t kSellHostRows = 8192;
 
 // The tables of a row-slice copy built on the device, in one allocation, when the
 // window is the default and no row is long; *done tells whether they were.  Waits for
@@ -955,7 +971,8 @@ SellTable *get_sell(spmv_matrix *h, int32_t sigma, cudaStream_t s, bool transpos
         t.n_ctas = o.ctas_for(t.n);
         if (t.n_ctas <= 0) return nullptr;
         bool done = false;
-        bool ok = (!transposed && h->max_row > kSellLongRow) || build_sell(t, d_rp, nr, sigma, &done, s);
+        bool ok = nr < kSellHostRows || (!transposed && h->max_row > kSellLongRow) ||
+                  build_sell(t, d_rp, nr, sigma, &done, s);
         if (ok && !done) {
             std::vector<int2> d;
             std::vector<int32_t> sr, ws;
@@ -1010,15 +1027,14 @@ SellTable *get_sell_positions(spmv_matrix *h, cudaStream_t s) {
     if (!t || !t->diagonal) return nullptr;
     if (t->vpos.count(h->sigma)) return t;
     if (capture_id(s)) return nullptr;  // nothing is built
-    const size_t nslots = static_cast<size_t>(t->slot_rows) * kSellC;
-    int32_t *vpos = nullptr, *rowpos = nullptr;
-    bool ok = dmalloc(&vpos, nslots + 4) == cudaSuccess &&
-              dmalloc(&rowpos, static_cast<size_t>(h->n_rows)) == cudaSuccess &&
-              cudaMemsetAsync(vpos, 0xff, static_cast<size_t>(kSellU) * kSellC * 4, s) == cudaSuccess &&
-              launch_sell_vpos(a.d, a.srows, a.n, t->d, t->srows, t->n, h->d_rp, h->d_rowT, h->d_colT, h->d_perm, rowpos,
-                               vpos, s) == cudaSuccess &&
-              cudaStreamSynchronize(s) == cudaSuccess;
-    cudaFree(rowpos);
+    const size_t nslots = (static_cast<size_t>(t->slot_rows) * kSellC + 7) / 4 * 4;
+    int32_t *vpos = nullptr;  // and behind it a work array, kept: freeing it would wait once more
+    bool ok = dmalloc(&vpos, nslots + static_cast<size_t>(h->n_rows)) == cudaSuccess;
+    int32_t *rowpos = ok ? vpos + nslots : nullptr;
+    ok = ok && cudaMemsetAsync(vpos, 0xff, static_cast<size_t>(kSellU) * kSellC * 4, s) == cudaSuccess &&
+         launch_sell_vpos(a.d, a.srows, a.n, t->d, t->srows, t->n, h->d_rp, h->d_rowT, h->d_colT, h->d_perm, rowpos,
+                          vpos, s) == cudaSuccess &&
+         cudaStreamSynchronize(s) == cudaSuccess;
     if (!ok) {
         cudaFree(vpos);
         (void)cudaGetLastError();
