@@ -251,13 +251,17 @@ template <> __device__ __forceinline__ void end_run<AccFRF>(AccFRF &a) { a.fold(
 // Row r of m summed again with exact FP64 products of its (FP32-stored)
 // operands, in CRS order: the fallback for a poisoned float-float row sum (see
 // AccFF).  x[j] is read at x + j*ldx.
-template <typename VT, bool INDIRECT, typename XT>
+// MAPPED: the values may lie elsewhere (m.vind not null, a symmetric handle's expanded
+// matrix); a test in the kernels that never meet it costs the plain FP32 product 2 %.
+template <typename VT, bool INDIRECT, bool MAPPED = false, typename XT>
 __device__ __forceinline__ double row_sum_exact(const MatRef m, int64_t r, const XT *__restrict__ x, int64_t ldx = 1) {
     double s = 0.0;
     const int kb = __ldg(m.rp + r), ke = __ldg(m.rp + r + 1);
     for (int k = kb; k < ke; ++k) {
         VT v;
-        if (INDIRECT || m.vind)  // (a full matrix's values stay where the symmetric handle has them)
+        if constexpr (INDIRECT)
+            v = __ldg(static_cast<const VT *>(m.vind) + __ldg(static_cast<const int32_t *>(m.vs) + k));
+        else if (MAPPED && m.vind)
             v = __ldg(static_cast<const VT *>(m.vind) + __ldg(static_cast<const int32_t *>(m.vs) + k));
         else
             v = __ldg(static_cast<const VT *>(m.vs) + k);
@@ -268,11 +272,11 @@ __device__ __forceinline__ double row_sum_exact(const MatRef m, int64_t r, const
 
 // The row sum of a finished accumulator: a poisoned float-float sum is summed
 // again from the CRS arrays of m (row r, operand x); anything else as it is.
-template <typename VT, bool INDIRECT, typename XT, typename ACC>
+template <typename VT, bool INDIRECT, bool MAPPED = false, typename XT, typename ACC>
 __device__ __forceinline__ double acc_value(const ACC &a, const MatRef &m, int64_t r, const XT *__restrict__ x) {
     if constexpr (std::is_same<ACC, AccFF>::value || std::is_same<ACC, AccFR>::value ||
                   std::is_same<ACC, AccFRF>::value) {
-        if (a.poisoned()) return row_sum_exact<VT, INDIRECT>(m, r, x);
+        if (a.poisoned()) return row_sum_exact<VT, INDIRECT, MAPPED>(m, r, x);
     }
     return a.get();
 }

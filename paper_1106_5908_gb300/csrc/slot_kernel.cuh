@@ -230,7 +230,7 @@ __device__ __forceinline__ void slot_loop(const SlotParams &p, ACC *srow, int c,
                                 continue;
                             }
                         }
-                        store_acc<VT, false>(m, x, y, r0 + q, srow[q], alpha, beta, plain);
+                        store_acc<VT, false, std::is_same<ACC, AccFF>::value>(m, x, y, r0 + q, srow[q], alpha, beta, plain);
                     }
                 }
             }

@@ -88,12 +88,12 @@ __device__ __forceinline__ void store_row(YT *__restrict__ y, int64_t row, doubl
 // m.rmap).  A float-float sum bound for an FP32 y with alpha = 1, beta = 0 is
 // rounded to float directly (h + l on the FP32 pipe); a poisoned one is summed
 // again in FP64; every other case goes through FP64.
-template <typename VT, bool INDIRECT, typename XT, typename YT, typename ACC>
+template <typename VT, bool INDIRECT, bool MAPPED = false, typename XT, typename YT, typename ACC>
 __device__ __forceinline__ void store_acc(const MatRef &m, const XT *__restrict__ x, YT *__restrict__ y,
                                           int64_t row, const ACC &a, double alpha, double beta, bool plain) {
     if constexpr (std::is_same<ACC, AccFF>::value || std::is_same<ACC, AccFR>::value) {
         if (a.poisoned()) {
-            store_row(y, row, row_sum_exact<VT, INDIRECT>(m, row, x), alpha, beta, plain, m.rmap);
+            store_row(y, row, row_sum_exact<VT, INDIRECT, MAPPED>(m, row, x), alpha, beta, plain, m.rmap);
             return;
         }
         if constexpr (std::is_same<YT, float>::value) {
@@ -163,7 +163,7 @@ struct RowEpilogue {
                     continue;
                 }
             }
-            const double v = acc_value<VT, false>(srow[q], m, r0 + q, x);
+            const double v = acc_value<VT, false, std::is_same<ACC, AccFF>::value>(srow[q], m, r0 + q, x);
             YT &out = y[row_of(k, r0 + q)];
             if constexpr (UPD == kUpdAdd || MAP) out = narrow<YT>(fma(alpha, v, widen(old[k])));
             else if constexpr (UPD == kUpdGeneral && std::is_same<ACC, AccF64>::value)

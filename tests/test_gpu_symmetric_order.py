@@ -111,6 +111,22 @@ def test_first_new_values_captured(kind, dtype):
         check(y, val, 2, turn)
 
 
+@pytest.mark.parametrize("kind", ["scattered", "uneven"])
+def test_fp32_sums_out_of_range_follow_new_values(kind):
+    """Products below 2^-100 are summed again in FP64, from the values of U."""
+    U = _upper(kind)
+    M = _sym(U, torch.float32)
+    x = dev(W.uniform(U.n_rows, 3) * 2.0 ** -40, torch.float32)
+    M.apply(x)
+    for seed in (8, 9, 10):
+        val = dev(W.uniform(U.nnz, seed) * 2.0 ** -70, torch.float32)
+        M.set_values(val)
+        ref, bound = oracle.spmv_sym(U.row_ptr, U.col_idx, host(val.double()), host(x.double()), with_bound=True)
+        for _ in range(2):
+            y = M.apply(x)
+            assert_within(host(y), ref, bound, 2.0 ** -23, f"{kind} {seed}")  # the store's rounding alone
+
+
 def test_first_apply_captured():
     U = _upper("grid")
     M = _sym(U, torch.float64)
