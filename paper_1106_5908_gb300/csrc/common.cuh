@@ -305,24 +305,32 @@ __device__ __forceinline__ double epi_apply(double v, const YT *__restrict__ y, 
     return v;
 }
 
-// The same update of FP32 rows without FP64 instructions: alpha and beta as pairs
-// of floats (48 bits each), products and sums by exact two-products and two-sums
-// (Dekker 1971, Knuth), so that as in FP64 only the store rounds.  An FP64 update costs
-// a row eight instructions of a pipe with 2 lanes per SM and clock (widening included):
-// -0.75*A*x + 0.5*y, 5-point 2000^2 61 -> 32 us, 7-point 160^3 62 -> 35, 27-point
-// 128^3 54 -> 51.
+// The same update of FP32 rows without FP64 instructions: alpha and beta as three floats
+// each (all 53 bits), the row sum as two, every product that counts split exactly (Dekker
+// 1971, Knuth).  Where the terms do not cancel (|result| above 2^-8 of them) what is
+// below 2^-24 of them is added in single precision: 2^-46 of the terms are left out,
+// 2^-13 of the half ulp that the store rounds.  Where they do, the parts are added by
+// two-sums in three orders of magnitude (the expansions of Shewchuk, 1997), and what is
+// left out lies below 2^-58 of the terms, less than FP64 rounds away.  An FP64 update
+// costs a row eight instructions of a pipe with 2 lanes per SM and clock (widening
+// included), this one some 25, seldom 70, of a pipe with 128: -0.75*A*x + 0.5*y,
+// 5-point 2000^2 58 -> 31 us, 7-point 160^3 61 -> 34 (with the diagonal slices).
 struct EpiFF {
-    float ah, al, bh, bl;
+    float a[3], b[3];
     int on;  // 0: the update runs in FP64
 };
 inline EpiFF epi_ff(double alpha, double beta) {
     auto fits = [](double a) { return a >= -0x1p20 && a <= 0x1p20 && (a >= 0x1p-20 || a <= -0x1p-20); };
+    auto split = [](double a, float (&out)[3]) {
+        for (float &part : out) {
+            part = static_cast<float>(a);
+            a -= part;
+        }
+    };
     EpiFF f{};
     if (!fits(alpha) || !(beta == 0.0 || fits(beta)) || epi_mode(alpha, beta) == kEpiPlain) return f;
-    f.ah = static_cast<float>(alpha);
-    f.al = static_cast<float>(alpha - f.ah);
-    f.bh = static_cast<float>(beta);
-    f.bl = static_cast<float>(beta - f.bh);
+    split(alpha, f.a);
+    split(beta, f.b);
     f.on = 1;
     return f;
 }
@@ -331,22 +339,54 @@ template <> struct IsFloatPair<AccFF> { static constexpr bool value = true; };
 template <> struct IsFloatPair<AccFR> { static constexpr bool value = true; };
 template <> struct IsFloatPair<AccFRF> { static constexpr bool value = true; };
 
+// a + b = s + e exactly; a * b = p + e exactly (no underflow).  The rounded operations by
+// name: contracted into an FMA with the product that feeds it, a sum here is another.
+__device__ __forceinline__ float two_sum(float a, float b, float &e) {
+    const float s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    return s;
+}
+__device__ __forceinline__ float two_prod(float a, float b, float &e) {
+    const float p = __fmul_rn(a, b);
+    e = __fmaf_rn(a, b, -p);
+    return p;
+}
+
 // out = alpha * (a.h + a.l) + beta * old; false when the row needs FP64: operands
 // outside [2^-70, 2^100], where an exact split could underflow or a product overflow,
-// and zeros, whose sign the pair sum does not keep (old = 0 is harmless: it adds
-// nothing to a nonzero product).
+// and zeros, whose sign the parts do not keep (old = 0 is harmless: it adds nothing to a
+// nonzero product).
 template <typename ACC>
-__device__ __forceinline__ bool epi_ff_row(const EpiFF &f, const ACC &a, float old, float &out) {
-    const float h = fabsf(a.h), o = fabsf(old);
-    if (!(f.on && h >= 0x1p-70f && h <= 0x1p100f && ((o >= 0x1p-70f && o <= 0x1p100f) || old == 0.0f)) ||
-        a.poisoned())
+__device__ __forceinline__ bool epi_ff_row(const EpiFF &f, const ACC &acc, float old, float &out) {
+    float l;
+    const float h = two_sum(acc.h, acc.l, l);  // |l| <= 2^-24 |h|
+    const float ah = fabsf(h), o = fabsf(old);
+    if (!(f.on && ah >= 0x1p-70f && ah <= 0x1p100f && ((o >= 0x1p-70f && o <= 0x1p100f) || old == 0.0f)) ||
+        acc.poisoned())
         return false;
-    const float p = f.ah * a.h, q = f.bh * old;
-    const float t = fmaf(f.al, a.h, fmaf(f.ah, a.l, fmaf(f.ah, a.h, -p)));
-    const float u = fmaf(f.bl, old, fmaf(f.bh, old, -q));
-    const float s = p + q;
-    const float bb = s - p;
-    out = s + (((p - (s - bb)) + (q - bb)) + (t + u));
+    float p0e, p1e, p2e, q0e, q1e, r, e;
+    const float p0 = two_prod(f.a[0], h, p0e), q0 = two_prod(f.b[0], old, q0e);
+    float s = two_sum(p0, q0, r);
+    if (fabsf(s) >= 0x1p-8f * fabsf(p0)) {  // (then |q0| is at most 257 |s| too)
+        out = s + (r + ((p0e + q0e) + fmaf(f.a[1], h, fmaf(f.a[0], l, f.b[1] * old))));
+        return true;
+    }
+    // parts of the order of the terms, of 2^-24 and of 2^-48 of them
+    const float p1 = two_prod(f.a[1], h, p1e), p2 = two_prod(f.a[0], l, p2e), q1 = two_prod(f.b[1], old, q1e);
+    float u = fmaf(f.a[2], h, fmaf(f.a[1], l, f.b[2] * old)) + ((p1e + p2e) + q1e);
+    float t = two_sum(r, p0e, e);
+    u += e;
+    t = two_sum(t, q0e, e);
+    u += e;
+    t = two_sum(t, p1, e);
+    u += e;
+    t = two_sum(t, p2, e);
+    u += e;
+    t = two_sum(t, q1, e);
+    u += e;
+    s = two_sum(s, t, r);
+    out = s + (r + u);
     return true;
 }
 

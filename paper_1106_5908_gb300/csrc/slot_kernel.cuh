@@ -529,8 +529,8 @@ struct SlotKernel {
         return cached;
     }
     // the kernel compiled for the update.  Hamiltonian-like 4 M rows, one kernel for
-    // all updates against these: -0.75*A*x + 0.5*y FP64 184 -> 161 us, FP32 E = 7 145 ->
-    // 127, E = 11 134 -> 117, E = 15 129 -> 123; y - A*x FP64 184 -> 153
+    // all updates against these: -0.75*A*x + 0.5*y FP64 194 -> 160 us, FP32 E = 7 143 ->
+    // 126, E = 9 127 -> 122, E = 11 133 -> 119, E = 15 161 -> 152; y - A*x FP64 184 -> 153
     static cudaError_t launch_any(const SlotParams &p, cudaStream_t s) {
         if constexpr (IsFloatPair<ACC>::value) {
             if (p.beta != 0.0 || p.ff.on) return SlotKernel<E, VT, XT, YT, ACC, kUpdGeneral, false>::launch(p, s);
