@@ -61,8 +61,8 @@ cudaError_t launch_slot_map(const void *chunks, int E, int64_t n_slots, const in
                             cudaStream_t s);
 
 struct SellBatchParams;
-// The batched launch over members on diagonal slices: FP64, or FP32 storage with FP32
-// runs (rows of at most 11 entries).
+// The batched launch over members on diagonal slices: FP64, or FP32 storage with short
+// FP32 runs (rows of at most 11 entries).
 cudaError_t launch_sell_diag_batch(const SellBatchParams &p, int vk, cudaStream_t s);
 
 struct SellParams;

@@ -58,7 +58,7 @@ static cudaError_t diag_batch_as(const SellBatchParams &p, cudaStream_t s) {
 
 cudaError_t launch_sell_diag_batch(const SellBatchParams &p, int vk, cudaStream_t s) {
     if (p.n_list <= 0) return cudaSuccess;
-    return vk == kF64 ? diag_batch_as<double, AccF64>(p, s) : diag_batch_as<float, AccFR>(p, s);
+    return vk == kF64 ? diag_batch_as<double, AccF64>(p, s) : diag_batch_as<float, AccFRF>(p, s);
 }
 
 // How a pass of R right-hand sides runs: V per lane, L = ceil(R/V) lanes per row, G =

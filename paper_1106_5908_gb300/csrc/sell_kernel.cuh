@@ -351,8 +351,8 @@ struct SellVals {
 };
 
 // CNT slot rows of a half slice (kSellC apart): their columns are row + diagonal
-// (DIAG; 8 diagonals at dp) or as stored (cb).
-template <int CNT, bool DIAG, bool IND, typename ACC, typename VT, typename XT>
+// (DIAG; 8 diagonals at dp) or as stored (cb).  RUN: the longest run of FP32 FMAs.
+template <int CNT, bool DIAG, int RUN, bool IND, typename ACC, typename VT, typename XT>
 __device__ __forceinline__ void sell_diag_block(ACC &acc, const SellVals<VT, IND> &sv, const int32_t *__restrict__ cb,
                                                 const int4 *__restrict__ dp, int row, const XT *__restrict__ x,
                                                 uint64_t pol) {
@@ -388,29 +388,29 @@ __device__ __forceinline__ void sell_diag_block(ACC &acc, const SellVals<VT, IND
 #pragma unroll
     for (int u = 0; u < CNT; ++u) {
         acc.fma(v[u], xv[u]);
-        if (u % kSellU == kSellU - 1 || u == CNT - 1) end_run(acc);
+        if (u % RUN == RUN - 1 || u == CNT - 1) end_run(acc);
     }
 }
 
 // All w slot rows of a half slice.
-template <bool DIAG, bool IND, typename ACC, typename VT, typename XT>
+template <bool DIAG, int RUN = kSellU, bool IND, typename ACC, typename VT, typename XT>
 __device__ __forceinline__ void sell_diag_row(ACC &acc, int w, SellVals<VT, IND> sv, const int32_t *__restrict__ cb,
                                               const int4 *__restrict__ dp, int row, const XT *__restrict__ x,
                                               uint64_t pol) {
     for (; w >= 8; w -= 8) {
-        sell_diag_block<8, DIAG>(acc, sv, cb, dp, row, x, pol);
+        sell_diag_block<8, DIAG, RUN>(acc, sv, cb, dp, row, x, pol);
         sv.skip(8);
         if constexpr (DIAG) dp += 2;
         else cb += 8 * kSellC;
     }
     switch (w) {
-        case 7: sell_diag_block<7, DIAG>(acc, sv, cb, dp, row, x, pol); break;
-        case 6: sell_diag_block<6, DIAG>(acc, sv, cb, dp, row, x, pol); break;
-        case 5: sell_diag_block<5, DIAG>(acc, sv, cb, dp, row, x, pol); break;
-        case 4: sell_diag_block<4, DIAG>(acc, sv, cb, dp, row, x, pol); break;
-        case 3: sell_diag_block<3, DIAG>(acc, sv, cb, dp, row, x, pol); break;
-        case 2: sell_diag_block<2, DIAG>(acc, sv, cb, dp, row, x, pol); break;
-        case 1: sell_diag_block<1, DIAG>(acc, sv, cb, dp, row, x, pol); break;
+        case 7: sell_diag_block<7, DIAG, RUN>(acc, sv, cb, dp, row, x, pol); break;
+        case 6: sell_diag_block<6, DIAG, RUN>(acc, sv, cb, dp, row, x, pol); break;
+        case 5: sell_diag_block<5, DIAG, RUN>(acc, sv, cb, dp, row, x, pol); break;
+        case 4: sell_diag_block<4, DIAG, RUN>(acc, sv, cb, dp, row, x, pol); break;
+        case 3: sell_diag_block<3, DIAG, RUN>(acc, sv, cb, dp, row, x, pol); break;
+        case 2: sell_diag_block<2, DIAG, RUN>(acc, sv, cb, dp, row, x, pol); break;
+        case 1: sell_diag_block<1, DIAG, RUN>(acc, sv, cb, dp, row, x, pol); break;
         default: break;
     }
 }
@@ -498,6 +498,13 @@ struct SellBatchParams {
     EpiFF ff;
 };
 
+// FP32 runs of up to 5 entries, folded into float-float: at most as long as in the chunks
+// that sum the other members (7 or 9 entries of a row in a lane), and no less exact on
+// average: relative error of members of 5, 7, 9 and 11 entries per row 4.4, 4.9, 4.7 and
+// 4.7e-8 (runs over whole rows 4.4, 5.0, 5.6, 6.2; of 4 entries 4.6, 4.7, 4.7, 4.7; the
+// chunks 4.4, 5.0, 5.6, 5.6).
+constexpr int kBatchRun = 5;
+
 template <typename VT, typename ACC>
 __global__ void __launch_bounds__(256, sizeof(VT) == 8 ? 4 : 5) k_sell_diag_batch(const SellBatchParams p) {
     constexpr int C = kSellC;
@@ -529,9 +536,9 @@ __global__ void __launch_bounds__(256, sizeof(VT) == 8 ? 4 : 5) k_sell_diag_batc
         acc.zero();
         const SellVals<VT, false> sv{static_cast<const VT *>(t.vals) + base, nullptr};
         if (d0.w >= 0)
-            sell_diag_row<true>(acc, d0.y, sv, static_cast<const int32_t *>(nullptr), t.diag + d0.w, r, x, pol);
+            sell_diag_row<true, kBatchRun>(acc, d0.y, sv, static_cast<const int32_t *>(nullptr), t.diag + d0.w, r, x, pol);
         else
-            sell_diag_row<false>(acc, d0.y, sv, t.cols + base, static_cast<const int4 *>(nullptr), r, x, pol);
+            sell_diag_row<false, kBatchRun>(acc, d0.y, sv, t.cols + base, static_cast<const int4 *>(nullptr), r, x, pol);
         if (r >= 0) {
             if constexpr (std::is_same<ACC, AccF64>::value) {
                 y[r] = epi_apply(acc.get(), y + r, alpha, beta, emode);
