@@ -3,6 +3,8 @@
 // (every row at most 11 entries, so a lane's chain over a row is a run) or FP32
 // runs of one block (4 slot rows) each folded into float-float.
 #include <algorithm>
+#include <map>
+#include <mutex>
 
 #include "internal.h"
 #include "sell_kernel.cuh"
@@ -43,15 +45,35 @@ cudaError_t launch_sell_mr(const SellParams &b, const double *X, double *Y, int6
     return cudaGetLastError();
 }
 
-template <typename VT, typename ACC>
-static cudaError_t diag_batch_as(const SellBatchParams &p, cudaStream_t s) {
+// Resident CTAs of 256 threads of KERNEL on the device with smem bytes of shared memory
+// (up to `most`), asked once per amount: the queries cost a few us, as much as a small
+// launch.  0: an error.
+template <auto KERNEL>
+static int resident(size_t smem, size_t most) {
+    static int dev_of = -1;
+    static std::map<size_t, int> known;
+    static std::mutex m;
+    std::lock_guard<std::mutex> lock(m);
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
+    if (dev != dev_of) {
+        known.clear();
+        if (most > 0 && cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             static_cast<int>(most)) != cudaSuccess)
+            return 0;
+        dev_of = dev;
+    }
+    const auto it = known.find(smem);
+    if (it != known.end()) return it->second;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sell_diag_batch<VT, ACC>, 256, 0) != cudaSuccess ||
-        per_sm <= 0)
-        return cudaErrorInvalidConfiguration;
-    const int64_t want = (2 * static_cast<int64_t>(p.n_list) + 7) / 8, lim = static_cast<int64_t>(per_sm) * sms;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, KERNEL, 256, smem) != cudaSuccess) return 0;
+    return known[smem] = per_sm * sms;
+}
+
+template <typename VT, typename ACC>
+static cudaError_t diag_batch_as(const SellBatchParams &p, cudaStream_t s) {
+    const int64_t want = (2 * static_cast<int64_t>(p.n_list) + 7) / 8, lim = resident<k_sell_diag_batch<VT, ACC>>(0, 0);
+    if (lim <= 0) return cudaErrorInvalidConfiguration;
     k_sell_diag_batch<VT, ACC><<<static_cast<int>(want < lim ? want : lim), 256, 0, s>>>(p);
     return cudaGetLastError();
 }
@@ -681,17 +703,10 @@ __global__ void __launch_bounds__(256) k_sell_grad_val(const SellParams p, const
 }
 
 // Grid of a tile kernel: its resident CTAs, 8 half slices per CTA and turn.
-template <typename K>
-static int tile_grid(K kernel, int32_t n_slices, size_t smem) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             8 * 8 * TilePack<double>::entries(kTileMaxW)) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 256, smem) != cudaSuccess || per_sm <= 0)
-        return 0;
+template <auto KERNEL>
+static int tile_grid(int32_t n_slices, size_t smem) {
     const int64_t want = (2 * static_cast<int64_t>(n_slices) + 7) / 8;
-    return static_cast<int>(std::min<int64_t>(want, static_cast<int64_t>(per_sm) * sms));
+    return static_cast<int>(std::min<int64_t>(want, resident<KERNEL>(smem, 8 * 8 * TilePack<double>::entries(kTileMaxW))));
 }
 
 int sell_tile_max_row() { return kTileMaxW; }
@@ -699,7 +714,7 @@ int sell_tile_max_row() { return kTileMaxW; }
 template <typename ST, typename VT, typename ACC = void>
 static cudaError_t set_values_as(const SellParams &p, const void *val, void *dval, int max_w, cudaStream_t s) {
     const size_t smem = sizeof(VT) * 8 * TilePack<VT>::entries(max_w);
-    const int grid = tile_grid(k_sell_set_values<ST, VT, ACC>, p.n_slices, smem);
+    const int grid = tile_grid<k_sell_set_values<ST, VT, ACC>>(p.n_slices, smem);
     if (grid <= 0) return cudaErrorInvalidConfiguration;
     k_sell_set_values<ST, VT, ACC>
         <<<grid, 256, smem, s>>>(p, static_cast<const ST *>(val), static_cast<VT *>(dval), max_w);
@@ -725,7 +740,7 @@ cudaError_t launch_sell_set_values(const SellParams &p, const void *val, int sk,
 template <typename VT>
 static cudaError_t grad_val_as(const SellParams &p, const void *g, void *gv, int max_w, cudaStream_t s) {
     const size_t smem = sizeof(VT) * 8 * TilePack<VT>::entries(max_w);
-    const int grid = tile_grid(k_sell_grad_val<VT>, p.n_slices, smem);
+    const int grid = tile_grid<k_sell_grad_val<VT>>(p.n_slices, smem);
     if (grid <= 0) return cudaErrorInvalidConfiguration;
     k_sell_grad_val<VT><<<grid, 256, smem, s>>>(p, static_cast<const VT *>(g), static_cast<VT *>(gv), max_w);
     return cudaGetLastError();

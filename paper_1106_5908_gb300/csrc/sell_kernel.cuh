@@ -334,8 +334,8 @@ __global__ void __launch_bounds__(256) k_sell(const SellParams p, const RedOut o
 // their column indices.
 // ---------------------------------------------------------------------------
 
-// Where a half slice's values are: in its own slots (vb), or, IND, at position
-// pb[slot] of another copy's values (the reverse pass: the slices of A^T read the
+// Where a half slice's values are: in its own slots (v), or, IND, at position
+// p[slot] of another copy's values (the reverse pass: the slices of A^T read the
 // values of A's slices, so new values need no layout in A^T's order).  On a grid
 // the 32 positions of a slot row are nearly consecutive in A's slices, where the
 // permutation of the CRS order put them in 32 places: 27-point 128^3, first pass

@@ -273,43 +273,6 @@ __global__ void __launch_bounds__(256, (slot_min_ctas<E, VT, BATCHED>())) k_slot
     slot_loop<E, VT, XT, YT, ACC, UPD, BATCHED>(p, s_rows[wib], blockIdx.x * 8 + wib, gridDim.x * 8);
 }
 
-// A batch whose members were tuned apart: the chunks of the members given 7
-// entries per lane (p7, their own slot-major copy) and those given 9 (p9), one
-// after the other in the same persistent launch (every warp takes its share of
-// each group).
-template <typename VT, typename XT, typename YT, typename ACC>
-__global__ void __launch_bounds__(256, (slot_min_ctas<9, VT, true>())) k_slot_mixed(const SlotParams p7, const SlotParams p9) {
-    static_assert(sizeof(ACC) == 8, "row buffer entries are 8 bytes");
-    __shared__ ACC s_rows[8][kWarpRowCap];
-    const int wib = threadIdx.x >> 5;
-    slot_loop<7, VT, XT, YT, ACC, kUpdPlain, true>(p7, s_rows[wib], blockIdx.x * 8 + wib, gridDim.x * 8);
-    __syncwarp();
-    slot_loop<9, VT, XT, YT, ACC, kUpdPlain, true>(p9, s_rows[wib], blockIdx.x * 8 + wib, gridDim.x * 8);
-}
-
-template <typename VT, typename XT, typename YT, typename ACC>
-struct SlotKernelMixed {
-    static cudaError_t launch(const SlotParams &p7, const SlotParams &p9, cudaStream_t s) {
-        static int cached = -1, cached_dev = -1;
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cached < 0 || cached_dev != dev) {
-            int per_sm = 0, sms = 0;
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_slot_mixed<VT, XT, YT, ACC>, 256, 0) !=
-                cudaSuccess)
-                return cudaErrorInvalidConfiguration;
-            cached = per_sm * sms;
-            cached_dev = dev;
-        }
-        const int n = p7.n_chunks > p9.n_chunks ? p7.n_chunks : p9.n_chunks;
-        if (n <= 0) return cudaSuccess;
-        const int want = (n + 7) / 8;
-        k_slot_mixed<VT, XT, YT, ACC><<<want < cached ? want : cached, 256, 0, s>>>(p7, p9);
-        return cudaGetLastError();
-    }
-};
-
 // Staged-values variant (TV).  The values of each chunk (32E contiguous
 // elements of the slot-major copy) arrive by one 1-D bulk copy (cp.async.bulk,
 // evict-first in L2) into a two-stage ring per warp in shared memory, requested
