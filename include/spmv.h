@@ -117,7 +117,9 @@ spmv_status spmv_create_symmetric(spmv_handle *out, int32_t n, int64_t nnz, cons
  * type t; t may differ from the handle's storage type only as FP64 -> FP32
  * storage or FP32 -> FP64 storage (converted on the device).  Asynchronous.  A
  * row-slice copy on diagonals that served the last values gets the new ones in
- * the same pass; other derived copies are laid out again when they are used. */
+ * the same pass; other derived copies are laid out again when they are used.
+ * Captured into a graph, the values change whenever the graph runs, which the
+ * handle does not see: capture the calls that use them with it. */
 spmv_status spmv_set_values(spmv_handle h, const void *val, spmv_dtype t, void *stream);
 
 /* spmv_set_values followed by y = alpha*A*x (spmv_apply with beta = 0), in one pass
@@ -267,8 +269,9 @@ spmv_status spmv_split_get_halo(spmv_split_handle hs, double *halo_out, void *st
  * X[j*nrhs + r], Y[i*nrhs + r] (row-major, leading dimension nrhs).
  * 1 <= nrhs <= 64.  vt: SPMV_F64 (X, Y FP64; FP64 values) only.  Runs on the sorted
  * row slices of plan family 5 (built on first use, whatever the handle's plan), up to
- * 32 right-hand sides per pass, when they pad at most 10 %; otherwise on the tile
- * kernel.  Results are unchanged up to summation order. */
+ * 32 right-hand sides per pass, when they pad at most 10 %; 2 or 3 right-hand sides on
+ * few rows, and what groups of 4 leave on matrices with rows of more than 128 entries,
+ * on the tile kernel, as everything else.  Results are unchanged up to summation order. */
 spmv_status spmm_apply(spmv_handle h, int32_t nrhs, double alpha, const void *X, double beta,
                        void *Y, spmv_dtype vt, void *stream);
 

@@ -305,7 +305,7 @@ constexpr int32_t kSellLongRow = 128;
 // Share of the slots that diagonal slices must cover for k_sell_diag to run (the
 // others read column indices there too, without k_sell's loads a block ahead).
 // The 27-point pattern on 24^3 (0.73) runs in 4.7 us (FP64; 3.5 FP32) against
-// 9.4 (7.0) on k_sell.
+// 9.4 (7.0) on k_sell; on 13^3 to 22^3 none is slower than there.
 constexpr double kDiagMinShare = 0.5;
 
 // Slices of the sorted row-slice layout: in each window of sigma rows, the rows
@@ -678,7 +678,8 @@ constexpr int32_t kDiagMinSize = 16384;
 // member at E = 9 (FP32 storage: 0.660 against 0.631 ms); the whole batch at
 // E = 7: 0.90 ms.  Members with shorter rows still get a group of their own.
 constexpr double kBatchSlotMeanE9 = 4.0;
-// Members of at least this many rows whose slices are diagonal run on them instead.
+// Members of at least this many rows whose slices are diagonal run on them instead
+// (64 5-point members of 182^2 rows: 25.5 us, 181^2 on the chunks 35.6).
 constexpr int32_t kBatchDiagMinSize = 32768;
 
 // Share of far entries (column_randomness) above which columns count as scattered.
@@ -2296,8 +2297,8 @@ spmv_status spmm_apply(spmv_handle h, int32_t nrhs, double alpha, const void *X,
     // sides, up to 32 per pass; exactly 4 with a lane per two rows (k_sell_mr) when
     // neighbouring rows share x in L1, or when X is too large for L2 to keep the
     // rows of X between its reads either way (Hamiltonian-like: 4.2 M rows, X 134
-    // MB, 461 against 478 us; 300,000 rows 50 against 36; 27-point 101^3 192
-    // against 194, 5-point 1400^2 74 against 80).
+    // MB, 461 against 478 us; 1.9 M rows, 61 MB, 201 against 196; 300,000 rows 50 against
+    // 36; 27-point 101^3 192 against 194, 5-point 1400^2 74 against 80).
     // Not for 2 or 3 right-hand sides on few rows: a warp then walks 16 or 32 whole rows
     // at the latency of its loads, where the tile kernel cuts the entries evenly (3:
     // 27-point 25^3 15.7 against 7.9 us, 32^3 17.6 / 13.9, 40^3 17.6 / 21.3; scattered
