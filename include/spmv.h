@@ -91,17 +91,18 @@ void spmv_destroy(spmv_handle h);
  * j >= i (repeated entries are summed; columns need not be sorted), so each
  * off-diagonal value is given once and serves a_ij and a_ji.  spmv_apply on the
  * handle computes y = alpha*A*x + beta*y with A = U + U_s^T (U_s: U without its
- * diagonal).  The first apply expands A into device memory (24 bytes per entry of A in
- * FP64, 16 in FP32, beside U and its transposed index: the CRS arrays of A, the copy that
- * its autotuned plan reads, and the place of each value in U) and applies run on it; the
- * first apply after new values fills it again from U.  The memory is held until
- * spmv_destroy.  When A does not fit, after spmv_set_plan, or when the first apply was
- * captured into a graph, an apply takes two passes instead: the row sums of U on U's plan
- * (with beta), then the row sums of U_s^T added onto y by the warp-chunk kernel that
- * reads each value through its position in U (a transposed index built once here, on
- * the host: rows of U_s^T list their entries by increasing position in U).  Either way
- * the summation order is fixed: the same values and x give the same bits in every apply
- * of a handle, until spmv_set_plan changes its kernels.  spmv_get_info reports U's plan.
+ * diagonal).  The first apply expands A into device memory (about 28 bytes per entry of A
+ * in FP64, 20 in FP32 and 24 from new values on, beside U and its transposed index: the
+ * CRS arrays of A, the copy that its autotuned plan reads, and the place of each value in
+ * U) and applies run on it; the first apply after new values fills it again from U.  The
+ * memory is held until spmv_destroy.  When A does not fit, after spmv_set_plan, or when
+ * the first apply was captured into a graph, an apply takes two passes instead: the row
+ * sums of U on U's plan (with beta), then the row sums of U_s^T added onto y by the
+ * warp-chunk kernel that reads each value through its position in U (a transposed index
+ * built once here, on the host: rows of U_s^T list their entries by increasing position
+ * in U).  Either way the summation order is fixed: the same values and x give the same
+ * bits in every apply of a handle, until spmv_set_plan or spmv_set_accumulator changes
+ * its kernels.  spmv_get_info reports U's plan.
  * spmv_set_values replaces U's values; spmv_apply (vector types as for
  * spmv_apply, except FP32 storage with an FP64 y), spmv_get_info, spmv_set_plan
  * (for the U pass), spmv_set_accumulator and spmv_destroy accept the handle;

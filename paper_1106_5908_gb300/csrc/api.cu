@@ -2357,6 +2357,13 @@ spmv_status spmm_apply(spmv_handle h, int32_t nrhs, double alpha, const void *X,
 // Reverse pass
 // ---------------------------------------------------------------------------
 
+// Entries per lane of the staged chunk kernel over A^T (ind: values through the permutation).
+static int ind_chunk_E(const spmv_matrix *h, bool ind = true) {
+    const double meanT = h->n_cols ? static_cast<double>(h->nnz) / h->n_cols : 0.0;
+    WarpOps ops;
+    return meanT < 20.0 && warp_ops(h->vk, h->vk, h->vk, h->vk == kF32 ? kAccFF : kAccF64, 7, ind, false, &ops) ? 7 : 15;
+}
+
 spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void *x, void *grad_x,
                           void *grad_val, void *stream) {
     if (!h) return SPMV_ERR_INVALID_ARG;
@@ -2406,8 +2413,12 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
             const bool longer = h->nnz > 8LL * h->n_rows;
             if ((longer || h->nnz >= kPosMinEntries) && sell_ops(h->vk, h->vk, h->vk, acc, &lops) &&
                 (t = get_sell_positions(h, s)) != nullptr) {
+                // (also where the capture of the other path would have to build its chunks)
                 const SellTable &own = h->sells.at(h->sigma);
-                a = longer ? get_sell(h, h->sigma, s) : own.vals && own.laid.on(s) ? &own : nullptr;
+                const bool laid = own.vals && own.laid.on(s);
+                a = longer || (!h->chunksT.count(ind_chunk_E(h)) && capture_id(s) != 0) ? get_sell(h, h->sigma, s)
+                    : laid                                                              ? &own
+                                                                                        : nullptr;
             }
             if (a) {
                 SellParams lp =
@@ -2463,8 +2474,7 @@ spmv_status spmv_backward(spmv_handle h, double alpha, const void *g, const void
         if (!done) {
             WarpOps ops;
             const int acc = (h->vk == kF32) ? kAccFF : kAccF64;
-            int ET = (meanT < 20.0) ? 7 : 15;
-            if (!warp_ops(h->vk, h->vk, h->vk, acc, ET, ind, false, &ops)) ET = 15;
+            const int ET = ind_chunk_E(h, ind);
             if (!warp_ops(h->vk, h->vk, h->vk, acc, ET, ind, false, &ops)) return SPMV_ERR_UNSUPPORTED;
             ChunkTable *ct = get_chunks(h, ET, true);
             if (!ct) return SPMV_ERR_ALLOC;

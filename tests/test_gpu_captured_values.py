@@ -151,3 +151,34 @@ def test_captured_reverse_pass_outlives_its_plan():
         gx.zero_()
         graph.replay()
         assert_within(host(gx), ref, bound, 1e-13, f"replayed after {window}")
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_first_reverse_pass_captured_on_short_rows(dtype):
+    """On large grids of short rows a first reverse pass takes A's slices when a product has
+    laid them out and the permutation when not: a capture of the one that has not run yet
+    builds nothing either."""
+    from paper_1106_5908_gb300 import Matrix
+    A = W.laplace2d(290)  # 419,340 entries
+    ft, tol = (np.float64, 1e-13) if dtype == "f64" else (np.float32, 1e-6)
+    M = Matrix.from_csr(A.row_ptr, A.col_idx, A.val.astype(ft), A.n_cols)
+    x, g = dev(W.uniform(A.n_cols, 3).astype(ft)), dev(W.uniform(A.n_rows, 4).astype(ft))
+    source = dev(A.val.astype(ft))
+    T = oracle.transpose(A.row_ptr, A.col_idx, A.n_cols)
+    M.apply(x)
+    for _ in range(2):  # on the slices
+        M.set_values_apply(source, x)
+        M.backward(g, x)
+    M.set_values(source)
+    M.backward(g, x)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        M.set_values(source)  # nothing has read the slices since the last values
+        gx, gv = M.backward(g, x)
+    for seed in (5, 6):
+        val = W.uniform(A.nnz, seed).astype(ft)
+        source.copy_(dev(val))
+        graph.replay()
+        ref, bound = oracle.spmv(T[0], T[1], val[T[2]].astype(np.float64), host(g).astype(np.float64), with_bound=True)
+        assert_within(host(gx), ref, bound, tol, f"replayed {seed}")
