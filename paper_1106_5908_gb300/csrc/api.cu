@@ -420,13 +420,18 @@ void free_slots(SlotTable &t) {
 
 // Several arrays in one allocation: add() each, alloc(), then take() them in the same
 // order.  (An allocation of a megabyte or more takes some 40 to 80 us, a smaller one 4.)
+// Large arrays start where allocations of their own would, on 2 MB: on 256 bytes the
+// symmetric product of 1 M rows took 42.1 to 42.6 us instead of 42.0, the split 63.0 to
+// 63.9 instead of 62.8.
 struct Block {
     std::vector<size_t> at;
     size_t bytes = 0, next = 0;
     char *base = nullptr;
     void add(size_t b) {
+        const size_t unit = b >= (size_t(1) << 20) ? size_t(2) << 20 : 256;
+        bytes = (bytes + unit - 1) / unit * unit;
         at.push_back(bytes);
-        bytes += (b + 255) / 256 * 256;
+        bytes += b;
     }
     bool alloc() {
         if (cudaMalloc(&base, std::max<size_t>(bytes, 256)) != cudaSuccess) base = nullptr;
